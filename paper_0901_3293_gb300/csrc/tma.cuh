@@ -61,6 +61,15 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
   return true;
 }
 
+// Programmatic dependent launch.  A kernel launched with the programmatic
+// attribute may start while the kernel before it still runs: grid_wait blocks
+// until that kernel has completed and its writes are visible (at once in a
+// kernel launched without the attribute), and must come before any access to
+// memory the kernels share; grid_launch_dependents lets the next kernel's CTAs
+// take the slots that this grid leaves free.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // contiguous bulk copy global -> shared (both 16-byte aligned, bytes a
 // multiple of 16) completing on `bar`
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {

@@ -22,6 +22,7 @@
 // Populations are pulled straight from global memory (each is used once).
 #include <cuda.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
@@ -230,6 +231,8 @@ __device__ __forceinline__ void qside_body(const CUtensorMap* tmQ, const CUtenso
     tma_prefetch_desc(tmU);
   }
   __syncthreads();
+  grid_wait();  // the kernel before this one wrote the mirrors and reads the scratch
+  grid_launch_dependents();
 
   // plane p of Q lives in slot (p - (z0-2)) % 5, of rho u in slot (p - (z0-1)) % 4
   // (the plane offsets below are never negative: unsigned arithmetic keeps the ring
@@ -819,6 +822,8 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
     tma_prefetch_desc(tmQ1);
   }
   __syncthreads();
+  grid_wait();  // the scratch comes from the kernel before this one
+  grid_launch_dependents();
 
   auto slot = [&](int p) { return ring + ((unsigned)(p - (z0 - 1)) % L::SLOTS) * L::SLOT; };
   // plane p: the padded P / Q* box (site (x, y) at padded (x + 1, y + 1), so the
@@ -1318,6 +1323,25 @@ ZmGeom zm_geom(int nx, int ny, int nz, int zc, int ty) {
   return G;
 }
 
+// Launch with the programmatic attribute: the kernel's CTAs start as the
+// previous kernel of the stream drains, and wait for it in grid_wait.  It hides
+// the launch and the barrier set-up of each kernel: 12.5 -> 10.3 us per FP32 step
+// at 32^3, 94.5 -> 93.5 us at 64 x 64 x 256 (two-step graphs).
+template <typename... Params, typename... Args>
+void launch_dependent(void (*kernel)(Params...), int grid, int threads, size_t smem, cudaStream_t s, Args&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, kernel, Params(args)...);
+}
+
 template <typename real, int SQ, int SPT, bool WALLS>
 cudaError_t launch_step_zm_spt(const ZmArgs& a, cudaStream_t s) {
   constexpr int TY = zm_ty<real>();
@@ -1328,13 +1352,16 @@ cudaError_t launch_step_zm_spt(const ZmArgs& a, cudaStream_t s) {
   Sym5<real> qw{};
   if (WALLS) qw = {(real)a.q_wall[0], (real)a.q_wall[1], (real)a.q_wall[2], (real)a.q_wall[3], (real)a.q_wall[4]};
   if (a.events) cudaEventRecord(a.events[0], s);
-  k_qside<real, TY, SQ, WALLS><<<grid_q, qside_threads<TY, SQ>(), QsideSmem<real, TY>::bytes, s>>>(
-      *a.tm_q, *a.tm_q1, *a.tm_u, Gq, m, static_cast<const real*>(a.bext), static_cast<real*>(a.pq), a.err, qw);
+  for (int k = 0; k < std::max(1, a.reps); ++k)
+    launch_dependent(k_qside<real, TY, SQ, WALLS>, grid_q, qside_threads<TY, SQ>(), QsideSmem<real, TY>::bytes, s,
+                     *a.tm_q, *a.tm_q1, *a.tm_u, Gq, m, static_cast<const real*>(a.bext), static_cast<real*>(a.pq),
+                     a.err, qw);
   if (a.events) cudaEventRecord(a.events[1], s);
-  k_lbq<real, TY, SPT, WALLS><<<grid, ZM_TX * TY / SPT, LbqSmem<real, TY>::bytes, s>>>(
-      *a.tm_pq, *a.tm_u3, *a.tm_f, *a.tm_f1, *a.tm_f2, *a.tm_qpf, *a.tm_q1pf, G, m, static_cast<const real*>(a.f),
-      static_cast<const real*>(a.q), static_cast<real*>(a.fnew), static_cast<real*>(a.rhou_new),
-      static_cast<real*>(a.qout ? a.qout : a.q), a.err, qw);
+  for (int k = 0; k < std::max(1, a.reps); ++k)
+    launch_dependent(k_lbq<real, TY, SPT, WALLS>, grid, ZM_TX * TY / SPT, LbqSmem<real, TY>::bytes, s, *a.tm_pq,
+                     *a.tm_u3, *a.tm_f, *a.tm_f1, *a.tm_f2, *a.tm_qpf, *a.tm_q1pf, G, m,
+                     static_cast<const real*>(a.f), static_cast<const real*>(a.q), static_cast<real*>(a.fnew),
+                     static_cast<real*>(a.rhou_new), static_cast<real*>(a.qout ? a.qout : a.q), a.err, qw);
   if (a.events) cudaEventRecord(a.events[2], s);
   return cudaGetLastError();
 }
@@ -1368,12 +1395,12 @@ cudaError_t launch_step_zm_batch(const ZmBatchArgs& a, cudaStream_t s) {
   constexpr int TY = zm_ty<real>();
   const auto* reps = static_cast<const Replica<real>*>(a.reps);
   if (a.events) cudaEventRecord(a.events[0], s);
-  k_qside_batch<real, TY><<<a.Bq.total_ctas, qside_threads<TY, 1>(), QsideSmem<real, TY>::bytes, s>>>(
-      *a.maps, a.Bq, reps, a.order, static_cast<real*>(a.pq), a.err);
+  launch_dependent(k_qside_batch<real, TY>, a.Bq.total_ctas, qside_threads<TY, 1>(), QsideSmem<real, TY>::bytes, s,
+                   *a.maps, a.Bq, reps, a.order, static_cast<real*>(a.pq), a.err);
   if (a.events) cudaEventRecord(a.events[1], s);
-  k_lbq_batch<real, TY><<<a.B.total_ctas, ZM_TX * TY, LbqSmem<real, TY>::bytes, s>>>(
-      *a.maps, a.B, reps, a.order, static_cast<const real*>(a.f), static_cast<const real*>(a.q),
-      static_cast<real*>(a.fnew), static_cast<real*>(a.rhou_new), static_cast<real*>(a.qout ? a.qout : a.q), a.err);
+  launch_dependent(k_lbq_batch<real, TY>, a.B.total_ctas, ZM_TX * TY, LbqSmem<real, TY>::bytes, s, *a.maps, a.B, reps,
+                   a.order, static_cast<const real*>(a.f), static_cast<const real*>(a.q), static_cast<real*>(a.fnew),
+                   static_cast<real*>(a.rhou_new), static_cast<real*>(a.qout ? a.qout : a.q), a.err);
   if (a.events) cudaEventRecord(a.events[2], s);
   return cudaGetLastError();
 }

@@ -251,8 +251,8 @@ LCBP_API int lcbp_step(lcbp_lattice *h, int nsteps);
  * at a time with a CUDA event between kernels, and return in kernel_ms the
  * mean device time of each kernel of one step (milliseconds).  *nkernels is
  * set to the number of kernels per step: 2 on the fast path (qside: H, sigma,
- * tau, b and the Heun predictor; lbq: LB predictor-corrector and the Heun
- * corrector); on the generic path 3 with flow on and Jacobi coupling
+ * tau, b and the Heun predictor, two launches timed as one for FP64 states;
+ * lbq: LB predictor-corrector and the Heun corrector); on the generic path 3 with flow on and Jacobi coupling
  * (field: H/sigma/tau; force_predict: b and the Heun predictor; lb_correct:
  * LB predictor-corrector and the Heun corrector), 5 with Gauss-Seidel
  * coupling (field, force, lb, predict, correct), 3 with flow off (field,

@@ -637,6 +637,7 @@ int tune_zc(lcbp_lattice* h) {
     }
   }
   destroy();
+  if (h->dtype == LCBP_F64) best_zq = 1;  // (the FP64 first stage takes a plane per CTA)
   h->zc = best_zc;
   h->zc_q = best_zq;
   h->spt = best_spt;

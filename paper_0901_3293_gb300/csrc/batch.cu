@@ -194,7 +194,8 @@ void fill_zc(ZmBatch& zb, const int* zc) {
 void set_zc(lcbp_batch* b, const int* zc, const int* zc_q) {
   fill_zc(b->zb, zc);
   b->zbq = b->zb;
-  fill_zc(b->zbq, zc_q);
+  const int one[kZmMaxClasses] = {1, 1, 1, 1};
+  fill_zc(b->zbq, b->dtype == LCBP_F64 ? one : zc_q);  // (FP64: k_qsite_batch takes a plane per CTA)
   b->zc = zc[0];
 }
 

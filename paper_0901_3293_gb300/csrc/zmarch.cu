@@ -159,6 +159,58 @@ __device__ __forceinline__ Model<V> widen(const Model<real>& m) {
 }
 
 // ---------------------------------------------------------------------------
+// The site's LB pre-collision coefficients from rho^n, u^n, sigma_LC and the
+// body force bt (the external force included): with j = rho u,
+//   F_a = [drho/30 - rho u^2/12 + (j_a u_a - sigma_aa)/2] / tau_f,
+//   V_a = (j_a / tau_f + b_a) / 3,   C = [drho/30 + rho u^2/48] / tau_f,
+//   W_ab = (j_a u_b - sigma_ab) / (8 tau_f),
+// so that f^eq_i / tau_f + p_i (Sec. 2.2 Eq. feq, coeff, eq4; T = 1/3,
+// sigma traceless, deviations from the rest weights) is F_a + s V_a for the
+// face direction s e_a and C + (s . V) / 8 + sum_{a<b} s_a s_b W_ab for the
+// corner direction s.  P = [F_x F_y F_z V_x V_y V_z C W_xy W_xz W_yz].
+// ---------------------------------------------------------------------------
+template <typename V>
+__device__ __forceinline__ void lb_coefficients(const V& drho, const V u[3], const Sym5<V>& sg, const V bt[3],
+                                                const V& it, V P[10]) {
+  using real = V;  // (LCBP_Q's type)
+  const V half = V(0.5);
+  const V rho = V(1) + drho;
+  const V jx = rho * u[0], jy = rho * u[1], jz = rho * u[2];
+  const V rusq = jx * u[0] + jy * u[1] + jz * u[2];
+  const V d30 = drho * LCBP_Q(1, 30);
+  const V fb = d30 - rusq * LCBP_Q(1, 12);
+  const V it8 = it * LCBP_Q(1, 8);
+  P[0] = (fb + half * (jx * u[0] - sg.xx)) * it;
+  P[1] = (fb + half * (jy * u[1] - sg.yy)) * it;
+  P[2] = (fb + half * (jz * u[2] + (sg.xx + sg.yy))) * it;
+  P[3] = (jx * it + bt[0]) * LCBP_Q(1, 3);
+  P[4] = (jy * it + bt[1]) * LCBP_Q(1, 3);
+  P[5] = (jz * it + bt[2]) * LCBP_Q(1, 3);
+  P[6] = (d30 + rusq * LCBP_Q(1, 48)) * it;
+  P[7] = (jx * u[1] - sg.xy) * it8;
+  P[8] = (jx * u[2] - sg.xz) * it8;
+  P[9] = (jy * u[2] - sg.yz) * it8;
+}
+
+// The positions of the padded scratch that hold site (gx, gy): its own, and
+// its periodic images in the ghost columns and rows where the site lies on a
+// lattice face.  put1(X, Y) is called for each.
+template <typename F>
+__device__ __forceinline__ void scratch_positions(int nx, int ny, int gx, int gy, F&& put1) {
+  put1(gx + 1, gy + 1);
+  if (gx == 0 || gx == nx - 1 || gy == 0 || gy == ny - 1) {
+    const int xg = gx == 0 ? nx + 1 : (gx == nx - 1 ? 0 : -1);  // nx >= 4: not both
+    const int yg[2] = {gy == 0 ? ny + 1 : -1, gy == ny - 1 ? 0 : -1};
+    if (xg >= 0) put1(xg, gy + 1);
+    for (int j = 0; j < 2; ++j)
+      if (yg[j] >= 0) {
+        put1(gx + 1, yg[j]);
+        if (xg >= 0) put1(xg, yg[j]);
+      }
+  }
+}
+
+// ---------------------------------------------------------------------------
 // Kernel A: H, sigma, tau, b and the Heun predictor
 // ---------------------------------------------------------------------------
 template <typename real, int TY, int TX = ZM_TX>
@@ -553,9 +605,7 @@ __device__ __forceinline__ void qside_body(const CUtensorMap* tmQ, const CUtenso
       }
       const Sym5<V> r = be_rate<true>(q, h, dq, u, w, mv, true);
       // The site's 16 values (four groups; rho - 1 in the last place) of the
-      // padded scratch for lane k:
-      // at the site's padded position, and at its periodic images in the ghost
-      // columns and rows where the site lies on a lattice face.
+      // padded scratch for lane k, at the site's position and its images
       const int nxp = G.nxp, nyp = G.nyp, gs = 4 * G.nxp * G.nyp;  // gs: group stride
       auto put = [&](const V* P, const V* qs, const V& dr) {
 #pragma unroll
@@ -567,36 +617,16 @@ __device__ __forceinline__ void qside_body(const CUtensorMap* tmQ, const CUtenso
           const real g1[4] = {L(P[7]), L(P[8]), L(P[9]), L(P[0])};
           const real g2[4] = {L(P[1]), L(P[2]), L(qs[4]), L(dr)};
           const real g3[4] = {L(qs[0]), L(qs[1]), L(qs[2]), L(qs[3])};
-          auto put1 = [&](int xx, int yy) {
+          scratch_positions(nx, ny, gx, gy, [&](int xx, int yy) {
             real* d = pq + ((z * kZmPQG * nyp + yy) * nxp + xx) * 4;
             st4g(d, g0[0], g0[1], g0[2], g0[3]);
             st4g(d + gs, g1[0], g1[1], g1[2], g1[3]);
             st4g(d + 2 * gs, g2[0], g2[1], g2[2], g2[3]);
             st4g(d + 3 * gs, g3[0], g3[1], g3[2], g3[3]);
-          };
-          put1(gx + 1, gy + 1);
-          if (gx == 0 || gx == nx - 1 || gy == 0 || gy == ny - 1) {
-            const int xg = gx == 0 ? nx + 1 : (gx == nx - 1 ? 0 : -1);  // nx >= 4: not both
-            const int yg[2] = {gy == 0 ? ny + 1 : -1, gy == ny - 1 ? 0 : -1};
-            if (xg >= 0) put1(xg, gy + 1);
-            for (int j = 0; j < 2; ++j)
-              if (yg[j] >= 0) {
-                put1(gx + 1, yg[j]);
-                if (xg >= 0) put1(xg, yg[j]);
-              }
-          }
+          });
         }
       };
       const V qv[5] = {q.xx + r.xx, q.xy + r.xy, q.xz + r.xz, q.yy + r.yy, q.yz + r.yz};
-      // The site's LB pre-collision coefficients from rho^n, u^n, sigma_LC and
-      // b (the external force included): with j = rho u,
-      //   F_a = [drho/30 - rho u^2/12 + (j_a u_a - sigma_aa)/2] / tau_f,
-      //   V_a = (j_a / tau_f + b_a) / 3,   C = [drho/30 + rho u^2/48] / tau_f,
-      //   W_ab = (j_a u_b - sigma_ab) / (8 tau_f),
-      // so that f^eq_i / tau_f + p_i (Sec. 2.2 Eq. feq, coeff, eq4; T = 1/3,
-      // sigma traceless, deviations from the rest weights) is F_a + s V_a for the
-      // face direction s e_a and C + (s . V) / 8 + sum_{a<b} s_a s_b W_ab for the
-      // corner direction s.
       V bt[3] = {bx, by, bz};
       if (bext) {
         int sb[SPT];
@@ -610,24 +640,8 @@ __device__ __forceinline__ void qside_body(const CUtensorMap* tmQ, const CUtenso
       }
       const int hs0 = ty * TX + tx;
       const Sym5<V> sg = ld5v<SPT>(hslot(z) + 5 * TY * TX, TY * TX, hs0, hs0 + TYH * TX);
-      const V it = mv.inv_tau;
-      const V rho = V(1) + drho;
-      const V jx = rho * u[0], jy = rho * u[1], jz = rho * u[2];
-      const V rusq = jx * u[0] + jy * u[1] + jz * u[2];
-      const V d30 = drho * LCBP_Q(1, 30);
-      const V fb = d30 - rusq * LCBP_Q(1, 12);
-      const V it8 = it * LCBP_Q(1, 8);
       V P[10];
-      P[0] = (fb + half * (jx * u[0] - sg.xx)) * it;
-      P[1] = (fb + half * (jy * u[1] - sg.yy)) * it;
-      P[2] = (fb + half * (jz * u[2] + (sg.xx + sg.yy))) * it;
-      P[3] = (jx * it + bt[0]) * LCBP_Q(1, 3);
-      P[4] = (jy * it + bt[1]) * LCBP_Q(1, 3);
-      P[5] = (jz * it + bt[2]) * LCBP_Q(1, 3);
-      P[6] = (d30 + rusq * LCBP_Q(1, 48)) * it;
-      P[7] = (jx * u[1] - sg.xy) * it8;
-      P[8] = (jx * u[2] - sg.xz) * it8;
-      P[9] = (jy * u[2] - sg.yz) * it8;
+      lb_coefficients(drho, u, sg, bt, mv.inv_tau, P);
       put(P, qv, drho);
     }
   }
@@ -649,6 +663,141 @@ __global__ void __launch_bounds__(qside_threads<TY, SPT>(), sizeof(real) == 4 ? 
             const __grid_constant__ CUtensorMap tmU, ZmGeom G, Model<real> m, const real* __restrict__ bext,
             real* __restrict__ pq, int* __restrict__ err, Sym5<real> qw) {
   qside_body<real, TY, SPT, false, WALLS>(&tmQ, &tmQ1, &tmU, G, m, blockIdx.x, 0, bext, pq, err, qw);
+}
+
+// ---------------------------------------------------------------------------
+// Kernel A for FP64 states, in two launches without recomputation.  The chip has
+// two FP64 lanes per SM against 128 FP32 ones, so an FP64 step is bound by its
+// FP64 operations and not by memory or launches.  k_qside forms H, sigma and tau
+// on a ring around its tile and twice more per z-chunk for the divergence of
+// tau (1.6 x 1.5 times the field work on 32 x 4 tiles at four planes per CTA);
+// here each site forms them once:
+//   k_qsite  H, sigma, tau, Q* and the LB-ready coefficients, V_a without the
+//            (D0_b tau_ab) / 3 part; tau goes to a flat scratch of its own
+//   k_qdiv   V_a += (D0_b tau_ab) / 3
+// One thread per site, neighbours through L1 and L2.  Against the ring form with
+// its best planes per CTA: 33 for 62 us at 32^3 (the step 97.7 -> 79.5 us), 185
+// for 295 us at 64^3 (585 -> 454), 1.36 for 2.01 ms at 128^3 (4.15 -> 3.41).
+// ---------------------------------------------------------------------------
+// plain (coherent) vector loads: the kernel before may still have been writing
+// these buffers when this one was launched
+template <typename real>
+__device__ __forceinline__ Sym5<real> qmirror_at(const real* Q, int cq4, int o) {
+  real v[4];
+  ld4(Q, 4 * o, v);
+  return {v[0], v[1], v[2], v[3], Q[cq4 + o]};
+}
+
+// Site of a CTA's thread: tile bt of TX x TY sites of one plane
+template <int TY>
+__device__ __forceinline__ bool plane_site(const ZmGeom& G, int bt, int& x, int& y, int& z) {
+  x = (bt % G.tiles_x) * ZM_TX + threadIdx.x % ZM_TX;
+  y = ((bt / G.tiles_x) % G.tiles_y) * TY + threadIdx.x / ZM_TX;
+  z = bt / (G.tiles_x * G.tiles_y);
+  return x < G.nx && y < G.ny;
+}
+
+template <typename real, int TY, bool WALLS>
+__device__ __forceinline__ void qsite_body(const ZmGeom& G, const Model<real>& m, int bt, const real* Q,
+                                           const real* U, const real* bext, real* tau, real* pq,
+                                           const Sym5<real>& qw) {
+  using B = StateBox;
+  int x, y, z;
+  if (!plane_site<TY>(G, bt, x, y, z)) return;
+  const int n = (int)G.n, nxm = G.nxm, cq4 = 4 * (int)G.cq;
+  const int zm = z == 0 ? G.nz - 1 : z - 1, zp = z == G.nz - 1 ? 0 : z + 1;
+  const bool wlo = WALLS && z == 0, whi = WALLS && z == G.nz - 1;
+  auto oq = [&](int zz) { return (zz * G.nyq + y + B::QPY) * nxm + x + B::QPX; };
+  const int o = oq(z);
+  Stencil7<real> st;
+  st.c = qmirror_at(Q, cq4, o);
+  st.xm = qmirror_at(Q, cq4, o - 1);
+  st.xp = qmirror_at(Q, cq4, o + 1);
+  st.ym = qmirror_at(Q, cq4, o - nxm);
+  st.yp = qmirror_at(Q, cq4, o + nxm);
+  st.zm = wlo ? qw : qmirror_at(Q, cq4, oq(zm));
+  st.zp = whi ? qw : qmirror_at(Q, cq4, oq(zp));
+  Sym5<real> dq[3], sg;
+  real tu[3], u[3], w[3][3];
+  const Sym5<real> h = molecular_field<true>(st, m, dq);
+  lc_stress(st.c, h, m.xi, sg, tu);
+  const int s = (z * G.ny + y) * G.nx + x;
+  tau[s] = tu[0];
+  tau[n + s] = tu[1];
+  tau[2 * n + s] = tu[2];
+  auto ou = [&](int zz) { return 4 * ((zz * G.nyu + y + B::UPY) * nxm + x + B::UPX); };
+  const int ouc = ou(z);
+  real c[4], a[4], b[4];
+  ld4(U, ouc, c);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) u[k] = c[1 + k];
+  ld4(U, ouc + 4, a);
+  ld4(U, ouc - 4, b);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) w[k][0] = a[1 + k] - b[1 + k];  // twice the central derivatives
+  ld4(U, ouc + 4 * nxm, a);
+  ld4(U, ouc - 4 * nxm, b);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) w[k][1] = a[1 + k] - b[1 + k];
+  ld4(U, ou(zp), a);
+  ld4(U, ou(zm), b);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) w[k][2] = (whi ? -u[k] : a[1 + k]) - (wlo ? -u[k] : b[1 + k]);
+  const Sym5<real> r = be_rate<true>(st.c, h, dq, u, w, m, true);
+  real bt3[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) bt3[k] = (bext ? bext[k * n + s] : real(0)) - real(0.5) * ddot(h, dq[k]);
+  real P[10];
+  lb_coefficients(c[0], u, sg, bt3, m.inv_tau, P);
+  const real qs[5] = {st.c.xx + r.xx, st.c.xy + r.xy, st.c.xz + r.xz, st.c.yy + r.yy, st.c.yz + r.yz};
+  const int gs = 4 * G.nxp * G.nyp;
+  scratch_positions(G.nx, G.ny, x, y, [&](int X, int Y) {
+    real* d = pq + ((z * kZmPQG * G.nyp + Y) * G.nxp + X) * 4;
+    st4(d, P[6], P[3], P[4], P[5]);
+    st4(d + gs, P[7], P[8], P[9], P[0]);
+    st4(d + 2 * gs, P[1], P[2], qs[4], c[0]);
+    st4(d + 3 * gs, qs[0], qs[1], qs[2], qs[3]);
+  });
+}
+
+template <typename real, int TY, bool WALLS>
+__device__ __forceinline__ void qdiv_body(const ZmGeom& G, int bt, const real* tau, real* pq) {
+  int x, y, z;
+  if (!plane_site<TY>(G, bt, x, y, z)) return;
+  const int n = (int)G.n, nx = G.nx, ny = G.ny;
+  const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
+  const int ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;
+  const int zm = z == 0 ? G.nz - 1 : z - 1, zp = z == G.nz - 1 ? 0 : z + 1;
+  auto at = [&](int c, int xx, int yy, int zz) { return tau[c * n + (zz * ny + yy) * nx + xx]; };
+  // tau = [xy, xz, yz] with tau_yx = -tau_xy etc.; 0 on a ghost plane beyond a wall
+  const bool wlo = WALLS && z == 0, whi = WALLS && z == G.nz - 1;
+  const real xzp = whi ? real(0) : at(1, x, y, zp), xzm = wlo ? real(0) : at(1, x, y, zm);
+  const real yzp = whi ? real(0) : at(2, x, y, zp), yzm = wlo ? real(0) : at(2, x, y, zm);
+  const real sixth = LCBP_Q(1, 6);
+  const real bx = (at(0, x, yp, z) - at(0, x, ym, z)) + (xzp - xzm);
+  const real by = (yzp - yzm) - (at(0, xp, y, z) - at(0, xm, y, z));
+  const real bz = -((at(1, xp, y, z) - at(1, xm, y, z)) + (at(2, x, yp, z) - at(2, x, ym, z)));
+  real* g0 = pq + (z * kZmPQG * G.nyp * G.nxp) * 4;
+  real v[4];
+  ld4(g0, ((y + 1) * G.nxp + x + 1) * 4, v);
+  v[1] += sixth * bx;
+  v[2] += sixth * by;
+  v[3] += sixth * bz;
+  scratch_positions(nx, ny, x, y, [&](int X, int Y) { st4(g0 + (Y * G.nxp + X) * 4, v[0], v[1], v[2], v[3]); });
+}
+
+template <typename real, int TY, bool WALLS>
+__global__ void __launch_bounds__(ZM_TX* TY) k_qsite(ZmGeom G, Model<real> m, const real* Q, const real* U,
+                                                     const real* bext, real* tau, real* pq, Sym5<real> qw) {
+  grid_wait();
+  grid_launch_dependents();
+  qsite_body<real, TY, WALLS>(G, m, blockIdx.x, Q, U, bext, tau, pq, qw);
+}
+template <typename real, int TY, bool WALLS>
+__global__ void __launch_bounds__(ZM_TX* TY) k_qdiv(ZmGeom G, const real* tau, real* pq) {
+  grid_wait();
+  grid_launch_dependents();
+  qdiv_body<real, TY, WALLS>(G, blockIdx.x, tau, pq);
 }
 
 // The CTA's batch class, its replica and tile: classes own consecutive CTA ranges.
@@ -719,6 +868,39 @@ __global__ void __launch_bounds__(qside_threads<TY, 1>(), sizeof(real) == 4 ? 2 
     }
   }
   qside_body<real, TY, 1, true, false>(mq, mq1, mu, G, m, it.bt, it.j, nullptr, pqr, err, Sym5<real>{});
+}
+
+// FP64 batches: the two kernels above over every replica (class geometries with
+// one plane per CTA).  tau lies in the replica's block of the population buffer
+// that k_lbq_batch fills afterwards.
+template <typename real, int TY, bool DIV>
+__global__ void __launch_bounds__(ZM_TX* TY) k_qsite_batch(ZmBatch B, const Replica<real>* __restrict__ reps,
+                                                           const int* __restrict__ order, const real* Q,
+                                                           const real* U, real* fnew, real* pq) {
+  grid_wait();
+  grid_launch_dependents();
+  const ZmItem it = zm_item(B);
+  const ZmGeom G = zm_class_geom(B, it.k);
+  int rep0 = B.c[0].rep0;
+  long long pq0 = B.c[0].pq0, qm0 = B.c[0].qm0, um0 = B.c[0].um0;
+#pragma unroll
+  for (int i = 1; i < kZmMaxClasses; ++i)
+    if (i == it.k) {
+      rep0 = B.c[i].rep0;
+      pq0 = B.c[i].pq0;
+      qm0 = B.c[i].qm0;
+      um0 = B.c[i].um0;
+    }
+  const int r = order[rep0 + it.j];
+  real* const tau = fnew + NV * reps[r].base;
+  real* const pqr = pq + pq0 + (long long)it.j * kZmPQ * G.cp;
+  if constexpr (DIV) {
+    qdiv_body<real, TY, false>(G, it.bt, tau, pqr);
+  } else {
+    const Model<real> m = reps[r].m;
+    qsite_body<real, TY, false>(G, m, it.bt, Q + qm0 + (long long)it.j * 5 * G.cq,
+                                U + um0 + (long long)it.j * 4 * G.cu, nullptr, tau, pqr, Sym5<real>{});
+  }
 }
 
 // The positions of a padded mirror (site x at column x + px, y at row y + h)
@@ -1293,8 +1475,10 @@ constexpr int zm_max_spt() {
 template <typename real, int SPT, bool WALLS>
 cudaError_t zm_prepare_spt() {
   constexpr int TY = zm_ty<real>();
-  cudaError_t e = cudaFuncSetAttribute(k_qside<real, TY, SPT, WALLS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)QsideSmem<real, TY>::bytes);
+  cudaError_t e = cudaSuccess;
+  if constexpr (sizeof(real) == 4)
+    e = cudaFuncSetAttribute(k_qside<real, TY, SPT, WALLS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)QsideSmem<real, TY>::bytes);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_lbq<real, TY, SPT, WALLS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)LbqSmem<real, TY>::bytes);
@@ -1380,16 +1564,26 @@ template <typename real, int SQ, int SPT, bool WALLS>
 cudaError_t launch_step_zm_spt(const ZmArgs& a, cudaStream_t s) {
   constexpr int TY = zm_ty<real>();
   // each kernel marches its own planes per CTA
-  const ZmGeom G = zm_geom(a.nx, a.ny, a.nz, a.zc, TY), Gq = zm_geom(a.nx, a.ny, a.nz, a.zc_q > 0 ? a.zc_q : a.zc, TY);
+  const int zq = sizeof(real) == 8 ? 1 : a.zc_q > 0 ? a.zc_q : a.zc;  // (FP64: k_qsite's planes)
+  const ZmGeom G = zm_geom(a.nx, a.ny, a.nz, a.zc, TY), Gq = zm_geom(a.nx, a.ny, a.nz, zq, TY);
   const int grid = G.tiles_x * G.tiles_y * G.tiles_z, grid_q = Gq.tiles_x * Gq.tiles_y * Gq.tiles_z;
   const Model<real> m = *static_cast<const Model<real>*>(a.model);
   Sym5<real> qw{};
   if (WALLS) qw = {(real)a.q_wall[0], (real)a.q_wall[1], (real)a.q_wall[2], (real)a.q_wall[3], (real)a.q_wall[4]};
   if (a.events) cudaEventRecord(a.events[0], s);
-  for (int k = 0; k < std::max(1, a.reps); ++k)
-    launch_dependent(k_qside<real, TY, SQ, WALLS>, grid_q, qside_threads<TY, SQ>(), QsideSmem<real, TY>::bytes, s,
-                     *a.tm_q, *a.tm_q1, *a.tm_u, Gq, m, static_cast<const real*>(a.bext), static_cast<real*>(a.pq),
-                     a.err, qw);
+  for (int k = 0; k < std::max(1, a.reps); ++k) {
+    if constexpr (sizeof(real) == 8) {  // (tau in the population buffer that k_lbq fills)
+      real* tau = static_cast<real*>(a.fnew);
+      launch_dependent(k_qsite<real, TY, WALLS>, grid_q, ZM_TX * TY, 0, s, Gq, m, static_cast<const real*>(a.q),
+                       static_cast<const real*>(a.rhou), static_cast<const real*>(a.bext), tau,
+                       static_cast<real*>(a.pq), qw);
+      launch_dependent(k_qdiv<real, TY, WALLS>, grid_q, ZM_TX * TY, 0, s, Gq, tau, static_cast<real*>(a.pq));
+    } else {
+      launch_dependent(k_qside<real, TY, SQ, WALLS>, grid_q, qside_threads<TY, SQ>(), QsideSmem<real, TY>::bytes, s,
+                       *a.tm_q, *a.tm_q1, *a.tm_u, Gq, m, static_cast<const real*>(a.bext),
+                       static_cast<real*>(a.pq), a.err, qw);
+    }
+  }
   if (a.events) cudaEventRecord(a.events[1], s);
   for (int k = 0; k < std::max(1, a.reps); ++k)
     launch_dependent(k_lbq<real, TY, SPT, WALLS>, grid, ZM_TX * TY / SPT, LbqSmem<real, TY>::bytes, s, *a.tm_pq,
@@ -1416,8 +1610,10 @@ cudaError_t launch_step_zm(const ZmArgs& a, cudaStream_t s) {
 template <typename real>
 cudaError_t zm_batch_prepare() {
   constexpr int TY = zm_ty<real>();
-  cudaError_t e = cudaFuncSetAttribute(k_qside_batch<real, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)QsideSmem<real, TY>::bytes);
+  cudaError_t e = cudaSuccess;
+  if constexpr (sizeof(real) == 4)
+    e = cudaFuncSetAttribute(k_qside_batch<real, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)QsideSmem<real, TY>::bytes);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_lbq_batch<real, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)LbqSmem<real, TY>::bytes);
@@ -1429,8 +1625,16 @@ cudaError_t launch_step_zm_batch(const ZmBatchArgs& a, cudaStream_t s) {
   constexpr int TY = zm_ty<real>();
   const auto* reps = static_cast<const Replica<real>*>(a.reps);
   if (a.events) cudaEventRecord(a.events[0], s);
-  launch_dependent(k_qside_batch<real, TY>, a.Bq.total_ctas, qside_threads<TY, 1>(), QsideSmem<real, TY>::bytes, s,
-                   *a.maps, a.Bq, reps, a.order, static_cast<real*>(a.pq), a.err);
+  if constexpr (sizeof(real) == 8) {
+    launch_dependent(k_qsite_batch<real, TY, false>, a.Bq.total_ctas, ZM_TX * TY, 0, s, a.Bq, reps, a.order,
+                     static_cast<const real*>(a.q), static_cast<const real*>(a.rhou), static_cast<real*>(a.fnew),
+                     static_cast<real*>(a.pq));
+    launch_dependent(k_qsite_batch<real, TY, true>, a.Bq.total_ctas, ZM_TX * TY, 0, s, a.Bq, reps, a.order, nullptr,
+                     nullptr, static_cast<real*>(a.fnew), static_cast<real*>(a.pq));
+  } else {
+    launch_dependent(k_qside_batch<real, TY>, a.Bq.total_ctas, qside_threads<TY, 1>(), QsideSmem<real, TY>::bytes, s,
+                     *a.maps, a.Bq, reps, a.order, static_cast<real*>(a.pq), a.err);
+  }
   if (a.events) cudaEventRecord(a.events[1], s);
   launch_dependent(k_lbq_batch<real, TY>, a.B.total_ctas, ZM_TX * TY, LbqSmem<real, TY>::bytes, s, *a.maps, a.B, reps,
                    a.order, static_cast<const real*>(a.f), static_cast<const real*>(a.q), static_cast<real*>(a.fnew),

@@ -250,7 +250,8 @@ LCBP_API int lcbp_step(lcbp_lattice *h, int nsteps);
  * Advance nsteps >= 1 steps exactly as lcbp_step does, but launched one kernel
  * at a time with a CUDA event between kernels, and return in kernel_ms the
  * mean device time of each kernel of one step (milliseconds).  *nkernels is
- * set to the number of kernels per step: 2 on the fast path (qside: H, sigma,
+ * set to the number of kernels per step: 2 on the fast path and for other
+ * widths that run its kernels (qside: H, sigma,
  * tau, b and the Heun predictor, two launches timed as one for FP64 states;
  * lbq: LB predictor-corrector and the Heun corrector); on the generic path 3 with flow on and Jacobi coupling
  * (field: H/sigma/tau; force_predict: b and the Heun predictor; lb_correct:
@@ -263,8 +264,10 @@ LCBP_API int lcbp_profile_steps(lcbp_lattice *h, int nsteps, double *kernel_ms, 
 /*
  * Kernel selection.  LCBP_PATH_AUTO (default) runs the fast path -- two
  * z-marching kernels that stage planes in shared memory with TMA tile loads
- * -- whenever flow is on, coupling is Jacobi and nx is a multiple of 4;
- * otherwise, or with LCBP_PATH_GENERIC, three one-thread-per-site kernels.
+ * -- whenever flow is on, coupling is Jacobi and nx is a multiple of 4; other
+ * widths of at least 4 run the same two kernels (lcbp_get_path names only the
+ * multiples of 4 fast); otherwise, or with LCBP_PATH_GENERIC, three
+ * one-thread-per-site kernels.
  * FP32 fast kernels come in two builds, one or two lattice sites per thread
  * (the latter on packed FP32x2 arithmetic); AUTO times both, LCBP_PATH_FAST1
  * and LCBP_PATH_FAST2 pin one (a lattice with walls runs one site per thread
@@ -274,7 +277,7 @@ LCBP_API int lcbp_profile_steps(lcbp_lattice *h, int nsteps, double *kernel_ms, 
 LCBP_API int lcbp_set_path(lcbp_lattice *h, int path);
 
 /*
- * *fast = 1 if the next step runs the fast path; *planes_per_cta = the
+ * *fast = 1 if the next step runs the fast path (nx a multiple of 4); *planes_per_cta = the
  * autotuned number of z-planes each CTA marches through and
  * *sites_per_thread = the autotuned 1 or 2 (both 0 before the first step, or
  * on the generic path).  The tuning times each candidate once per lattice

@@ -262,7 +262,7 @@ Layout layout(int nx, int ny, int nz, int dtype) {
   L.off[15] = o;  // partials + out
   o = align256(o + (kDiagPartials + 8) * 8);
   // padded mirrors of Q and rho u [0], [1] (lattices the fast path can serve)
-  const bool fast_shape = zm_shape_ok(nx, ny, nz);
+  const bool fast_shape = zm_march_ok(nx, ny, nz);
   L.off[16] = o;
   o = align256(o + (fast_shape ? (size_t)zm_qmirror_elems(nx, ny, nz) * es : 0));
   L.off[17] = o;
@@ -395,11 +395,10 @@ bool make_scratch_tmap(CUtensorMap* tm, void* base, int nxp, int nyp, int nz, in
   return encode_tiled(tm, base, 4, dims, strides, box, dtype);
 }
 
-bool fast_shape_ok(const lcbp_lattice* h) { return zm_shape_ok(h->nx, h->ny, h->nz); }
-
+// whether the step runs the z-marching kernels
 bool use_fast(lcbp_lattice* h) {
-  if (h->path_req == LCBP_PATH_GENERIC || !h->p.flow_on || h->p.coupling != LCBP_JACOBI || !fast_shape_ok(h) ||
-      (h->p.l2_set && h->p.L2 != h->p.K))
+  if (h->path_req == LCBP_PATH_GENERIC || !h->p.flow_on || h->p.coupling != LCBP_JACOBI ||
+      !zm_march_ok(h->nx, h->ny, h->nz) || (h->p.l2_set && h->p.L2 != h->p.K))
     return false;
   if (!h->tmaps_ok) {
     static std::once_flag prep32, prep64;
@@ -422,7 +421,8 @@ bool use_fast(lcbp_lattice* h) {
       ok = ok && make_mirror_tmap(&h->tm[1 + k], h->um[k], 4 * nxm, nyu, h->nz, 4 * kZmBoxXU, ty + 2, h->dtype);
     const int nxp = h->nx + kZmPadX;
     ok = ok && make_scratch_tmap(&h->tm[3], h->pq, nxp, nyu, h->nz, ty + 2, h->dtype);
-    for (int k = 0; k < 2; ++k) {  // the populations (L2 prefetches only): the tile's rows, then halo-row boxes
+    // the populations (L2 prefetches only; widths with rows of whole 16-byte groups): the tile's rows, then halo-row boxes
+    for (int k = 0; k < 2 && h->nx % 4 == 0; ++k) {
       ok = ok && make_field_tmap(&h->tm[6 + k], h->f[k], NV, h->nx, h->ny, h->nz, ty, NV, h->dtype);
       ok = ok && make_field_tmap(&h->tm[9 + k], h->f[k], NV, h->nx, h->ny, h->nz, 1, 1, h->dtype);
       ok = ok && make_field_tmap(&h->tm[11 + k], h->f[k], NV, h->nx, h->ny, h->nz, 1, 2, h->dtype);
@@ -1308,7 +1308,7 @@ int lcbp_set_path(lcbp_lattice* h, int path) {
 
 int lcbp_get_tuning(lcbp_lattice* h, int* planes_per_cta, int* spt_lb, int* spt_q, int* planes_per_cta_q) {
   CHECK_H(h);
-  const bool f = use_fast(h) && h->zc > 0;
+  const bool f = use_fast(h) && h->nx % 4 == 0 && h->zc > 0;
   if (planes_per_cta) *planes_per_cta = f ? h->zc : 0;
   if (planes_per_cta_q) *planes_per_cta_q = f ? (h->zc_q > 0 ? h->zc_q : h->zc) : 0;
   if (spt_lb) *spt_lb = f ? h->spt : 0;
@@ -1318,7 +1318,8 @@ int lcbp_get_tuning(lcbp_lattice* h, int* planes_per_cta, int* spt_lb, int* spt_
 
 int lcbp_get_path(lcbp_lattice* h, int* fast, int* planes_per_cta, int* sites_per_thread) {
   CHECK_H(h);
-  const bool f = use_fast(h);
+  // ("fast" names the widths that are a multiple of 4; others run the same kernels with plain row prefetches)
+  const bool f = use_fast(h) && h->nx % 4 == 0;
   if (fast) *fast = f ? 1 : 0;
   if (planes_per_cta) *planes_per_cta = f ? h->zc : 0;
   if (sites_per_thread) *sites_per_thread = f && h->zc > 0 ? h->spt : 0;

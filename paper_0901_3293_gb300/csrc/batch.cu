@@ -179,6 +179,7 @@ void fill_zc(ZmBatch& zb, const int* zc) {
     c.G.nxp = c.G.nx + kZmPadX;
     c.G.nyp = c.G.ny + 2;
     c.G.cp = (long long)c.G.nxp * c.G.nyp * c.G.nz;
+    c.G.pf = 1;
     c.G.nxm = zm_mirror_nx(c.G.nx);
     c.G.nyq = c.G.ny + 4;
     c.G.nyu = c.G.ny + 2;

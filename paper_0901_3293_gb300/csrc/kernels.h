@@ -123,7 +123,7 @@ cudaError_t launch_diag_one(const DiagGeom& g, const void* q, const void* f, int
 constexpr int kDiagPartials = 512 * 8;
 
 // ---------------------------------------------------------------------------
-// Fast path (flow on, Jacobi coupling, zm_shape_ok): two z-marching kernels
+// Fast path (flow on, Jacobi coupling, zm_march_ok): two z-marching kernels
 // with TMA-staged planes.  The host builds the tensor maps: the padded mirrors
 // of Q and rho u as 3-D tensors (4-D with the replica outermost for a batch
 // class), the scratch below as (4 X, Y, group, z), and the populations as a
@@ -155,6 +155,7 @@ struct ZmGeom {
   int tiles_x, tiles_y, tiles_z;
   int nxp, nyp;    // padded scratch and rho u mirror extents: nx + 4, ny + 2
   long long cp;    // their component stride: nxp * nyp * nz
+  int pf;          // 1: f rows are whole 16-byte groups, k_lbq prefetches them by tensor maps; 0: row by row
   int nxm;         // mirror row length: zm_mirror_nx(nx)
   int nyq, nyu;    // mirror rows per plane: ny + 4 (Q), ny + 2 (rho u)
   long long cq, cu;  // mirror component strides: nxm * nyq * nz, nxm * nyu * nz
@@ -180,15 +181,21 @@ inline int zm_mirror_nx(int nx) { return (nx + 31) / 32 * 32 + 2 * kZmMirX; }  /
 inline long long zm_qmirror_elems(int nx, int ny, int nz) { return 5LL * zm_mirror_nx(nx) * (ny + 4) * nz; }
 inline long long zm_umirror_elems(int nx, int ny, int nz) { return 4LL * zm_mirror_nx(nx) * (ny + 2) * nz; }
 
-// Shapes the fast kernels serve: rows of whole 16-byte groups (nx % 4 == 0 for
-// the TMA boxes) and element offsets within one lattice that fit in 32 bits
-// (the kernels index with int; the largest offsets are those of the 15
-// populations, the 16 scratch values and the 5 components of the Q mirror).
-inline bool zm_shape_ok(int nx, int ny, int nz) {
+// Shapes the z-marching kernels can serve: nx >= 4 (a site has at most one
+// periodic image in x within the mirrors' two ghost columns) and element offsets
+// within one lattice that fit in 32 bits (the kernels index with int; the
+// largest offsets are those of the 15 populations, the 16 scratch values and the
+// 5 components of the Q mirror).
+inline bool zm_march_ok(int nx, int ny, int nz) {
   const long long n = (long long)nx * ny * nz, cp = (long long)(nx + kZmPadX) * (ny + 2) * nz;
   const long long cq = (long long)zm_mirror_nx(nx) * (ny + 4) * nz, lim = 2147483647LL;
-  return nx % 4 == 0 && 15 * n < lim && kZmPQ * cp < lim && 5 * cq < lim;
+  return nx >= 4 && 15 * n < lim && kZmPQ * cp < lim && 5 * cq < lim;
 }
+// Shapes of the fast path proper (what lcbp_get_path reports, and batches):
+// nx % 4 == 0 as well, so that rows of the flat populations are whole 16-byte
+// groups and k_lbq prefetches them with tensor maps.  Single lattices of other
+// widths run the same kernels with plain row prefetches.
+inline bool zm_shape_ok(int nx, int ny, int nz) { return nx % 4 == 0 && zm_march_ok(nx, ny, nz); }
 
 struct ZmArgs {
   int nx, ny, nz, zc;  // zc: planes per CTA of k_lbq

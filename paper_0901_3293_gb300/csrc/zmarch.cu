@@ -1015,9 +1015,11 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
     mbar_init_fence();
     tma_prefetch_desc(tmPQ);
     tma_prefetch_desc(tmU3);
-    tma_prefetch_desc(tmF);
-    tma_prefetch_desc(tmF1);
-    tma_prefetch_desc(tmF2);
+    if (G.pf) {
+      tma_prefetch_desc(tmF);
+      tma_prefetch_desc(tmF1);
+      tma_prefetch_desc(tmF2);
+    }
     tma_prefetch_desc(tmQ);
     tma_prefetch_desc(tmQ1);
   }
@@ -1058,13 +1060,15 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
       tma_prefetch_l2_4d(tmQ1, X, Y, wrap(p - 1, nz), rc);
     } else {
       tma_load_3d(sl + L::OFF_U, tmU3, 4 * (x0 - B::UX + B::UPX), y0 - 1 + B::UPY, zz, bar);
-      tma_prefetch_l2_4d(tmF, xf, y0, zz, 0);
-      tma_prefetch_l2_4d(tmF1, xf, ya, zz, 3);
-      tma_prefetch_l2_4d(tmF2, xf, ya, zz, 7);
-      tma_prefetch_l2_4d(tmF2, xf, ya, zz, 11);
-      tma_prefetch_l2_4d(tmF1, xf, yb, zz, 4);
-      tma_prefetch_l2_4d(tmF2, xf, yb, zz, 9);
-      tma_prefetch_l2_4d(tmF2, xf, yb, zz, 13);
+      if (G.pf) {
+        tma_prefetch_l2_4d(tmF, xf, y0, zz, 0);
+        tma_prefetch_l2_4d(tmF1, xf, ya, zz, 3);
+        tma_prefetch_l2_4d(tmF2, xf, ya, zz, 7);
+        tma_prefetch_l2_4d(tmF2, xf, ya, zz, 11);
+        tma_prefetch_l2_4d(tmF1, xf, yb, zz, 4);
+        tma_prefetch_l2_4d(tmF2, xf, yb, zz, 9);
+        tma_prefetch_l2_4d(tmF2, xf, yb, zz, 13);
+      }
       tma_prefetch_l2_3d(tmQ, 4 * X, Y, wrap(p - 1, nz));
       tma_prefetch_l2_3d(tmQ1, X, Y, wrap(p - 1, nz));
     }
@@ -1159,6 +1163,13 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
     if (threadIdx.x == 0) {
       fence_proxy_async();
       if (z + 2 <= z1) issue(z + 2);
+    }
+    // rows of f that no tensor map describes: a thread per population and row of
+    // the tile prefetches its row of plane z+2
+    if (!BATCH && !G.pf && z + 2 <= z1 && (int)threadIdx.x < NV * TY) {
+      const int i = threadIdx.x / TY, yy = min(y0 + (int)threadIdx.x % TY, ny - 1);
+      const real* row = f + (i * n + (wrap(z + 2, nz) * ny + yy) * nx);
+      for (int k = 0; k <= TX; k += 128 / (int)sizeof(real)) prefetch_l2(row + min(x0 + min(k, TX - 1), nx - 1));
     }
     // a wall's ghost plane: the anchored Q*
     if (WALLS && (ghost(z + 1) || (z == z0 && ghost(z0 - 1)))) {
@@ -1533,6 +1544,7 @@ ZmGeom zm_geom(int nx, int ny, int nz, int zc, int ty) {
   G.nxp = nx + kZmPadX;
   G.nyp = ny + 2;
   G.cp = (long long)G.nxp * G.nyp * nz;
+  G.pf = nx % 4 == 0;
   G.nxm = zm_mirror_nx(nx);
   G.nyq = ny + 4;
   G.nyu = ny + 2;

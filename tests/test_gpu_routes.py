@@ -1,0 +1,64 @@
+"""The kernels that AUTO picks for each kind of step against the generic ones.
+
+Widths that are no multiple of 4 (the z-marching kernels with plain row
+prefetches), with and without walls, on shapes with ragged tiles in x and y,
+several tiles and z-chunks, and the smallest width.
+"""
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+# (nz, ny, nx): one partial tile, several with a ragged last one, rows of every
+# alignment of a 16-byte group, fewer planes than a chunk, the smallest width
+SHAPES = [(9, 11, 5), (37, 19, 45), (21, 9, 101), (1, 3, 66), (2, 17, 35), (6, 40, 4)]
+
+
+@pytest.fixture(scope="module")
+def lcbp():
+    import torch
+    from paper_0901_3293_gb300 import build
+    build.build()
+    from paper_0901_3293_gb300 import lcbp as L
+    torch.cuda.set_device(0)
+    return L
+
+
+def pair(L, shape, dtype, mode):
+    """Two lattices in the same state (BPII with noise), AUTO and GENERIC."""
+    nz, ny, nx = shape
+    out = []
+    for path in (L.PATH_AUTO, L.PATH_GENERIC):
+        lat = L.Lattice(nx, ny, nz, dtype=dtype).set_path(path)
+        lat.set_flow(flow_on=mode != "noflow", coupling=L.GAUSS_SEIDEL if mode == "gauss_seidel" else L.JACOBI)
+        if mode == "walls":
+            lat.set_walls(True, (0.2, 0.0, 0.0, -0.1, 0.0))
+        lat.init_q(L.BPII, 0.3, noise=1e-3, seed=4)
+        if mode != "noflow":
+            lat.init_f_equilibrium(1.0)
+        out.append(lat)
+    return out
+
+
+# FP64: rounding of O(1/2) fields over 10 steps (as the parity tests take it).
+# FP32: the bounds of the fast-against-generic comparison of the parity tests.
+TOL = {"f64": (1e-13, 1e-14), "f32": (1e-6, 1e-8)}
+
+
+def check(L, shape, dtype, mode, steps):
+    a, b = pair(L, shape, dtype, mode)
+    for lat in (a, b):
+        lat.step(steps)
+    tq, tu = TOL[dtype]
+    assert np.abs(a.read_q() - b.read_q()).max() < tq
+    if mode != "noflow":
+        assert np.abs(a.read_u() - b.read_u()).max() < tu
+        assert np.abs(a.read_f() - b.read_f()).max() <= (2.0 ** -23 if dtype == "f32" else tq)
+
+
+@pytest.mark.parametrize("mode", ["flow", "walls"])
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_marching_kernels_match_generic(lcbp, shape, dtype, mode):
+    check(lcbp, shape, dtype, mode, 11)

@@ -365,13 +365,13 @@ lcbp_lattice* new_handle(int nx, int ny, int nz, int dtype) {
 }
 
 // ---- fast path: tensor maps, eligibility, autotuned z-chunk -------------------
-// field [comps][nz][ny][nx] as a 4-D tensor, box = 40 x rows x 1 x box_comps
-bool make_field_tmap(CUtensorMap* tm, void* base, int comps, int nx, int ny, int nz, int rows, int box_comps,
-                     int dtype) {
+// field [comps][nz][ny][nx] as a 4-D tensor, box = width x rows x 1 x box_comps
+bool make_field_tmap(CUtensorMap* tm, void* base, int comps, int nx, int ny, int nz, int width, int rows,
+                     int box_comps, int dtype) {
   const cuuint64_t es = dtype_size(dtype);
   const cuuint64_t dims[4] = {(cuuint64_t)nx, (cuuint64_t)ny, (cuuint64_t)nz, (cuuint64_t)comps};
   const cuuint64_t strides[3] = {nx * es, (cuuint64_t)nx * ny * es, (cuuint64_t)nx * ny * nz * es};
-  const cuuint32_t box[4] = {(cuuint32_t)kZmBoxX, (cuuint32_t)rows, 1, (cuuint32_t)box_comps};
+  const cuuint32_t box[4] = {(cuuint32_t)width, (cuuint32_t)rows, 1, (cuuint32_t)box_comps};
   return encode_tiled(tm, base, 4, dims, strides, box, dtype);
 }
 
@@ -386,13 +386,21 @@ bool make_mirror_tmap(CUtensorMap* tm, void* base, int w, int nym, int nz, int i
 }
 
 // the LB-ready scratch [z][group][nyp][nxp][4] as a 4-D tensor (4 nxp, nyp,
-// group, z), box = 4 * 34 x rows x 4 groups x 1
-bool make_scratch_tmap(CUtensorMap* tm, void* base, int nxp, int nyp, int nz, int rows, int dtype) {
+// group, z), box = 4 * width x rows x 4 groups x 1
+bool make_scratch_tmap(CUtensorMap* tm, void* base, int nxp, int nyp, int nz, int width, int rows, int dtype) {
   const cuuint64_t es = dtype_size(dtype), X = 4 * (cuuint64_t)nxp;
   const cuuint64_t dims[4] = {X, (cuuint64_t)nyp, (cuuint64_t)kZmPQG, (cuuint64_t)nz};
   const cuuint64_t strides[3] = {X * es, X * nyp * es, (cuuint64_t)kZmPQ * nxp * nyp * es};
-  const cuuint32_t box[4] = {(cuuint32_t)(4 * kZmBoxXP), (cuuint32_t)rows, (cuuint32_t)kZmPQG, 1};
+  const cuuint32_t box[4] = {(cuuint32_t)(4 * width), (cuuint32_t)rows, (cuuint32_t)kZmPQG, 1};
   return encode_tiled(tm, base, 4, dims, strides, box, dtype);
+}
+
+// tile width of the fast kernels (two sites per thread exist for 32-wide tiles only)
+int tile_x(const lcbp_lattice* h) {
+  return h->path_req == LCBP_PATH_FAST2 && !h->p.walls_z ? 32 : zm_lattice_tile_x(h->nx, h->dtype != LCBP_F64);
+}
+int tile_y(const lcbp_lattice* h) {
+  return (h->dtype == LCBP_F64 ? zm_tile_rows<double>() : zm_tile_rows<float>()) * (32 / tile_x(h));
 }
 
 // whether the step runs the z-marching kernels
@@ -404,28 +412,28 @@ bool use_fast(lcbp_lattice* h) {
     static std::once_flag prep32, prep64;
     if (h->dtype == LCBP_F64) std::call_once(prep64, [] { zm_prepare<double>(); });
     else std::call_once(prep32, [] { zm_prepare<float>(); });
-    const int ty = h->dtype == LCBP_F64 ? zm_tile_rows<double>() : zm_tile_rows<float>();
-    // Q and rho u from their padded mirrors (40- and 34-site boxes; Q as its
-    // [xx xy xz yy] vectors and its yz array), and the LB-ready scratch
-    // (34-site boxes)
+    // Q and rho u from their padded mirrors (boxes tx + 8 and tx + 2 sites wide;
+    // Q as its [xx xy xz yy] vectors and its yz array), and the LB-ready scratch
+    // (tx + 2 sites wide)
+    const int tx = tile_x(h), ty = tile_y(h);
     const int nxm = zm_mirror_nx(h->nx), nyq = h->ny + 4, nyu = h->ny + 2;
     const long long cq = (long long)nxm * nyq * h->nz;
-    bool ok = make_mirror_tmap(&h->tm[0], h->qm, 4 * nxm, nyq, h->nz, 4 * kZmBoxX, ty + 4, h->dtype) &&
-              make_mirror_tmap(&h->tm[8], static_cast<char*>(h->qm) + 4 * cq * h->es, nxm, nyq, h->nz, kZmBoxX,
+    bool ok = make_mirror_tmap(&h->tm[0], h->qm, 4 * nxm, nyq, h->nz, 4 * (tx + 8), ty + 4, h->dtype) &&
+              make_mirror_tmap(&h->tm[8], static_cast<char*>(h->qm) + 4 * cq * h->es, nxm, nyq, h->nz, tx + 8,
                                ty + 4, h->dtype) &&
               // the same in tile-sized boxes (k_lbq's prefetches of Q^n at its own sites)
-              make_mirror_tmap(&h->tm[4], h->qm, 4 * nxm, nyq, h->nz, 4 * 32, ty, h->dtype) &&
-              make_mirror_tmap(&h->tm[5], static_cast<char*>(h->qm) + 4 * cq * h->es, nxm, nyq, h->nz, 32, ty,
+              make_mirror_tmap(&h->tm[4], h->qm, 4 * nxm, nyq, h->nz, 4 * tx, ty, h->dtype) &&
+              make_mirror_tmap(&h->tm[5], static_cast<char*>(h->qm) + 4 * cq * h->es, nxm, nyq, h->nz, tx, ty,
                                h->dtype);
     for (int k = 0; k < 2; ++k)
-      ok = ok && make_mirror_tmap(&h->tm[1 + k], h->um[k], 4 * nxm, nyu, h->nz, 4 * kZmBoxXU, ty + 2, h->dtype);
+      ok = ok && make_mirror_tmap(&h->tm[1 + k], h->um[k], 4 * nxm, nyu, h->nz, 4 * (tx + 2), ty + 2, h->dtype);
     const int nxp = h->nx + kZmPadX;
-    ok = ok && make_scratch_tmap(&h->tm[3], h->pq, nxp, nyu, h->nz, ty + 2, h->dtype);
+    ok = ok && make_scratch_tmap(&h->tm[3], h->pq, nxp, nyu, h->nz, tx + 2, ty + 2, h->dtype);
     // the populations (L2 prefetches only; widths with rows of whole 16-byte groups): the tile's rows, then halo-row boxes
     for (int k = 0; k < 2 && h->nx % 4 == 0; ++k) {
-      ok = ok && make_field_tmap(&h->tm[6 + k], h->f[k], NV, h->nx, h->ny, h->nz, ty, NV, h->dtype);
-      ok = ok && make_field_tmap(&h->tm[9 + k], h->f[k], NV, h->nx, h->ny, h->nz, 1, 1, h->dtype);
-      ok = ok && make_field_tmap(&h->tm[11 + k], h->f[k], NV, h->nx, h->ny, h->nz, 1, 2, h->dtype);
+      ok = ok && make_field_tmap(&h->tm[6 + k], h->f[k], NV, h->nx, h->ny, h->nz, tx + 8, ty, NV, h->dtype);
+      ok = ok && make_field_tmap(&h->tm[9 + k], h->f[k], NV, h->nx, h->ny, h->nz, tx + 8, 1, 1, h->dtype);
+      ok = ok && make_field_tmap(&h->tm[11 + k], h->f[k], NV, h->nx, h->ny, h->nz, tx + 8, 1, 2, h->dtype);
     }
     if (!ok) {
       h->path_req = LCBP_PATH_GENERIC;  // tensor maps unavailable: stay on the generic kernels
@@ -438,6 +446,7 @@ bool use_fast(lcbp_lattice* h) {
 
 ZmArgs zm_args(lcbp_lattice* h, const void* model) {
   ZmArgs a{};
+  a.tx = tile_x(h);
   a.nx = h->nx;
   a.ny = h->ny;
   a.nz = h->nz;
@@ -527,8 +536,8 @@ std::vector<int> zc_candidates(const lcbp_lattice* h, int spt) {
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int ty = h->dtype == LCBP_F64 ? zm_tile_rows<double>() : zm_tile_rows<float>();
-  const long long tiles_xy = (long long)((h->nx + 31) / 32) * ((h->ny + ty - 1) / ty);
+  const int tx = tile_x(h), ty = tile_y(h);
+  const long long tiles_xy = (long long)((h->nx + tx - 1) / tx) * ((h->ny + ty - 1) / ty);
   const long long resident = (long long)sms * (h->dtype == LCBP_F64 ? zm_resident<double>(spt) : zm_resident<float>(spt));
   for (int w = 1; w <= 48; ++w) {
     const long long want = w * resident;
@@ -546,7 +555,8 @@ std::vector<int> zc_candidates(const lcbp_lattice* h, int spt) {
 int tune_zc(lcbp_lattice* h) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   const char* path = std::getenv("LCBP_AUTOTUNE_CACHE");
-  const int spt_max = h->dtype == LCBP_F64 ? zm_spt_max<double>() : zm_spt_max<float>();
+  // (narrow tiles: one site per thread only)
+  const int spt_max = tile_x(h) < 32 ? 1 : h->dtype == LCBP_F64 ? zm_spt_max<double>() : zm_spt_max<float>();
   // a pinned sites-per-thread choice tunes only the planes per CTA, uncached
   const bool pinned = h->path_req == LCBP_PATH_FAST1 || h->path_req == LCBP_PATH_FAST2;
   // (walls: one site per thread only)
@@ -1071,6 +1081,7 @@ int lcbp_set_walls(lcbp_lattice* h, int walls_z, const double* q_wall5) {
   // the fast kernels take q_wall as a launch argument: recapture the step
   drop_graph(h);
   if (p.walls_z != h->p.walls_z) {
+    h->tmaps_ok = false;
     h->zc = 0;  // tuned separately with walls
     h->spt = 0;
     h->spt_q = 0;
@@ -1300,6 +1311,7 @@ int lcbp_set_path(lcbp_lattice* h, int path) {
     return fail(LCBP_EINVAL, "two sites per thread exist for FP32 lattices only");
   drop_graph(h);
   h->path_req = path;
+  h->tmaps_ok = false;  // the tile shape follows the choice
   h->zc = 0;  // retune for the new choice
   h->spt = 0;
   h->spt_q = 0;
@@ -1541,6 +1553,7 @@ int lcbp_load(lcbp_lattice* h, const char* path) {
   if (p.flow_on != h->p.flow_on || p.coupling != h->p.coupling || p.walls_z != h->p.walls_z ||
       p.l2_set != h->p.l2_set || p.L2 != h->p.L2)
     drop_graph(h);
+  if (p.walls_z != h->p.walls_z) h->tmaps_ok = false;
   h->p = p;
   rc = upload_replica(h);
   if (rc) return rc;

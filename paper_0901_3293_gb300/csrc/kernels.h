@@ -172,11 +172,16 @@ struct ZmGeom {
 // the plain array [z][Y][X] of yz.  k_lbq writes Q^{n+1} and rho u^{n+1} there,
 // images included, so the next step stages them with no patching.
 constexpr int kZmMirX = 32;  // columns before x = 0 in a mirror row
-// Batch classes of FP32 replicas whose width leaves a last 32-column tile at
-// most half full (nx % 32 in 1..16, e.g. 48) take tiles of 16 columns by 16
-// rows instead: the same 256 sites and threads, no idle lanes.
+// Narrow tiles: 16 columns by 16 rows, the same 256 sites and threads (FP32).
+// Batch classes whose width leaves a last 32-column tile at most half full
+// (nx % 32 in 1..16, e.g. 48) take them.  A single lattice takes them only where
+// it is at most 16 wide, so that half of every 32-column tile would be idle
+// (16 x 64 x 64: 18.5 -> 14.5 us per step, 12 x 100 x 100: 33.8 -> 29.7); wider
+// ones lose more to the 16-site rows of f than they gain in lanes (144^3: 251
+// against 263 us, 101 x 75 x 67: 59.7 against 60.6).
 constexpr int kZmNarrowX = 16;
 inline int zm_batch_tile_x(int nx, bool fp32) { return fp32 && nx % 32 != 0 && nx % 32 <= 16 ? kZmNarrowX : 32; }
+inline int zm_lattice_tile_x(int nx, bool fp32) { return fp32 && nx <= kZmNarrowX ? kZmNarrowX : 32; }
 inline int zm_mirror_nx(int nx) { return (nx + 31) / 32 * 32 + 2 * kZmMirX; }  // mirror row length
 inline long long zm_qmirror_elems(int nx, int ny, int nz) { return 5LL * zm_mirror_nx(nx) * (ny + 4) * nz; }
 inline long long zm_umirror_elems(int nx, int ny, int nz) { return 4LL * zm_mirror_nx(nx) * (ny + 2) * nz; }
@@ -199,6 +204,7 @@ inline bool zm_shape_ok(int nx, int ny, int nz) { return nx % 4 == 0 && zm_march
 
 struct ZmArgs {
   int nx, ny, nz, zc;  // zc: planes per CTA of k_lbq
+  int tx;             // tile width: 32, or kZmNarrowX (FP32, one site per thread)
   int zc_q;           // planes per CTA of k_qside (0: as zc)
   int spt;            // sites per thread of k_lbq, 1 or 2 (2 only where zm_spt_max allows)
   int spt_q;          // sites per thread of k_qside (0: as spt)
@@ -228,8 +234,8 @@ inline long long zm_pq_elems(int nx, int ny, int nz) {
   return (long long)kZmPQ * (nx + kZmPadX) * (ny + 2) * nz;
 }
 
-// box widths of 32-wide tiles (single lattices; batch classes derive theirs from the tile width)
-constexpr int kZmBoxX = 40;   // sites per TMA box row of the flat fields and of the Q mirror (x0 - 4 ..)
+// box widths of 32-wide tiles (narrow ones: tile width + 8, + 2, + 2)
+constexpr int kZmBoxX = 40;   // sites per TMA box row of the populations and of the Q mirror (x0 - 4 ..)
 constexpr int kZmBoxXP = 34;  // sites per TMA box row of the padded scratch (x0 - 1 .. x0 + 32)
 constexpr int kZmBoxXU = 34;  // sites per TMA box row of the rho u mirror (x0 - 1 .. x0 + 32)
 

@@ -657,12 +657,12 @@ __device__ __forceinline__ void qside_body(const CUtensorMap* tmQ, const CUtenso
 }
 
 // FP32: two CTAs per SM (shared memory allows two; the bound keeps the registers within it)
-template <typename real, int TY, int SPT, bool WALLS>
-__global__ void __launch_bounds__(qside_threads<TY, SPT>(), sizeof(real) == 4 ? 2 : 1)
+template <typename real, int TY, int SPT, bool WALLS, int TX = ZM_TX>
+__global__ void __launch_bounds__(qside_threads<TY, SPT, TX>(), sizeof(real) == 4 ? 2 : 1)
     k_qside(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmQ1,
             const __grid_constant__ CUtensorMap tmU, ZmGeom G, Model<real> m, const real* __restrict__ bext,
             real* __restrict__ pq, int* __restrict__ err, Sym5<real> qw) {
-  qside_body<real, TY, SPT, false, WALLS>(&tmQ, &tmQ1, &tmU, G, m, blockIdx.x, 0, bext, pq, err, qw);
+  qside_body<real, TY, SPT, false, WALLS, TX>(&tmQ, &tmQ1, &tmU, G, m, blockIdx.x, 0, bext, pq, err, qw);
 }
 
 // ---------------------------------------------------------------------------
@@ -1398,16 +1398,16 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
   }
 }
 
-template <typename real, int TY, int SPT, bool WALLS>
-__global__ void __launch_bounds__(ZM_TX* TY / SPT, 2)
+template <typename real, int TY, int SPT, bool WALLS, int TX = ZM_TX>
+__global__ void __launch_bounds__(TX* TY / SPT, 2)
     k_lbq(const __grid_constant__ CUtensorMap tmPQ, const __grid_constant__ CUtensorMap tmU3,
           const __grid_constant__ CUtensorMap tmF, const __grid_constant__ CUtensorMap tmF1,
           const __grid_constant__ CUtensorMap tmF2, const __grid_constant__ CUtensorMap tmQ,
           const __grid_constant__ CUtensorMap tmQ1, ZmGeom G, Model<real> m, const real* __restrict__ f,
           const real* __restrict__ Qin, real* __restrict__ fnew, real* __restrict__ rhou_new, real* __restrict__ Qout,
           int* __restrict__ err, Sym5<real> qw) {
-  lbq_body<real, TY, SPT, false, WALLS>(&tmPQ, &tmU3, &tmF, &tmF1, &tmF2, &tmQ, &tmQ1, G, m, blockIdx.x, 0, f, Qin,
-                                        fnew, rhou_new, Qout, err, qw);
+  lbq_body<real, TY, SPT, false, WALLS, TX>(&tmPQ, &tmU3, &tmF, &tmF1, &tmF2, &tmQ, &tmQ1, G, m, blockIdx.x, 0, f,
+                                            Qin, fnew, rhou_new, Qout, err, qw);
 }
 
 template <typename real, int TY>
@@ -1496,11 +1496,27 @@ cudaError_t zm_prepare_spt() {
   return e;
 }
 
+// the narrow tiles of FP32 lattices
+template <bool WALLS>
+cudaError_t zm_prepare_narrow() {
+  constexpr int TY = 2 * zm_ty<float>(), TX = kZmNarrowX;
+  cudaError_t e = cudaFuncSetAttribute(k_qside<float, TY, 1, WALLS, TX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)QsideSmem<float, TY, TX>::bytes);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_lbq<float, TY, 1, WALLS, TX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)LbqSmem<float, TY, TX>::bytes);
+  return e;
+}
+
 // lattices with walls run one site per thread
 template <typename real>
 cudaError_t zm_prepare() {
   cudaError_t e = zm_prepare_spt<real, 1, false>();
   if (e == cudaSuccess) e = zm_prepare_spt<real, 1, true>();
+  if constexpr (sizeof(real) == 4) {
+    if (e == cudaSuccess) e = zm_prepare_narrow<false>();
+    if (e == cudaSuccess) e = zm_prepare_narrow<true>();
+  }
   if constexpr (zm_max_spt<real>() == 2)
     if (e == cudaSuccess) e = zm_prepare_spt<real, 2, false>();
   return e;
@@ -1529,16 +1545,16 @@ int zm_resident(int spt) {
   return zm_resident_spt<real, 1>();
 }
 
-ZmGeom zm_geom(int nx, int ny, int nz, int zc, int ty) {
+ZmGeom zm_geom(int nx, int ny, int nz, int zc, int tx, int ty) {
   ZmGeom G;
   G.nx = nx;
   G.ny = ny;
   G.nz = nz;
   G.zc = zc;
   G.n = (long long)nx * ny * nz;
-  G.tx = ZM_TX;
+  G.tx = tx;
   G.ty = ty;
-  G.tiles_x = (nx + ZM_TX - 1) / ZM_TX;
+  G.tiles_x = (nx + tx - 1) / tx;
   G.tiles_y = (ny + ty - 1) / ty;
   G.tiles_z = (nz + zc - 1) / zc;
   G.nxp = nx + kZmPadX;
@@ -1572,12 +1588,12 @@ void launch_dependent(void (*kernel)(Params...), int grid, int threads, size_t s
   cudaLaunchKernelEx(&c, kernel, Params(args)...);
 }
 
-template <typename real, int SQ, int SPT, bool WALLS>
+template <typename real, int SQ, int SPT, bool WALLS, int TX = ZM_TX>
 cudaError_t launch_step_zm_spt(const ZmArgs& a, cudaStream_t s) {
-  constexpr int TY = zm_ty<real>();
+  constexpr int TY = zm_ty<real>() * (ZM_TX / TX);
   // each kernel marches its own planes per CTA
   const int zq = sizeof(real) == 8 ? 1 : a.zc_q > 0 ? a.zc_q : a.zc;  // (FP64: k_qsite's planes)
-  const ZmGeom G = zm_geom(a.nx, a.ny, a.nz, a.zc, TY), Gq = zm_geom(a.nx, a.ny, a.nz, zq, TY);
+  const ZmGeom G = zm_geom(a.nx, a.ny, a.nz, a.zc, TX, TY), Gq = zm_geom(a.nx, a.ny, a.nz, zq, TX, TY);
   const int grid = G.tiles_x * G.tiles_y * G.tiles_z, grid_q = Gq.tiles_x * Gq.tiles_y * Gq.tiles_z;
   const Model<real> m = *static_cast<const Model<real>*>(a.model);
   Sym5<real> qw{};
@@ -1591,14 +1607,14 @@ cudaError_t launch_step_zm_spt(const ZmArgs& a, cudaStream_t s) {
                        static_cast<real*>(a.pq), qw);
       launch_dependent(k_qdiv<real, TY, WALLS>, grid_q, ZM_TX * TY, 0, s, Gq, tau, static_cast<real*>(a.pq));
     } else {
-      launch_dependent(k_qside<real, TY, SQ, WALLS>, grid_q, qside_threads<TY, SQ>(), QsideSmem<real, TY>::bytes, s,
-                       *a.tm_q, *a.tm_q1, *a.tm_u, Gq, m, static_cast<const real*>(a.bext),
+      launch_dependent(k_qside<real, TY, SQ, WALLS, TX>, grid_q, qside_threads<TY, SQ, TX>(),
+                       QsideSmem<real, TY, TX>::bytes, s, *a.tm_q, *a.tm_q1, *a.tm_u, Gq, m, static_cast<const real*>(a.bext),
                        static_cast<real*>(a.pq), a.err, qw);
     }
   }
   if (a.events) cudaEventRecord(a.events[1], s);
   for (int k = 0; k < std::max(1, a.reps); ++k)
-    launch_dependent(k_lbq<real, TY, SPT, WALLS>, grid, ZM_TX * TY / SPT, LbqSmem<real, TY>::bytes, s, *a.tm_pq,
+    launch_dependent(k_lbq<real, TY, SPT, WALLS, TX>, grid, TX * TY / SPT, LbqSmem<real, TY, TX>::bytes, s, *a.tm_pq,
                      *a.tm_u3, *a.tm_f, *a.tm_f1, *a.tm_f2, *a.tm_qpf, *a.tm_q1pf, G, m,
                      static_cast<const real*>(a.f), static_cast<const real*>(a.q), static_cast<real*>(a.fnew),
                      static_cast<real*>(a.rhou_new), static_cast<real*>(a.qout ? a.qout : a.q), a.err, qw);
@@ -1609,6 +1625,10 @@ cudaError_t launch_step_zm_spt(const ZmArgs& a, cudaStream_t s) {
 // sites per thread chosen for each kernel separately (FP32: 1 or 2 each; walls and FP64: 1)
 template <typename real>
 cudaError_t launch_step_zm(const ZmArgs& a, cudaStream_t s) {
+  if constexpr (sizeof(real) == 4)
+    if (a.tx == kZmNarrowX)
+      return a.q_wall ? launch_step_zm_spt<real, 1, 1, true, kZmNarrowX>(a, s)
+                      : launch_step_zm_spt<real, 1, 1, false, kZmNarrowX>(a, s);
   if (a.q_wall) return launch_step_zm_spt<real, 1, 1, true>(a, s);
   if constexpr (zm_max_spt<real>() == 2) {
     const int sq = a.spt_q > 0 ? a.spt_q : a.spt;

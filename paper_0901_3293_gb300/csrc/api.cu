@@ -403,11 +403,18 @@ int tile_y(const lcbp_lattice* h) {
   return (h->dtype == LCBP_F64 ? zm_tile_rows<double>() : zm_tile_rows<float>()) * (32 / tile_x(h));
 }
 
+// whether the lattice's kernels are those on the padded mirrors (the fast path's
+// and the Heun kernels) rather than the generic ones
+bool mirror_shape(const lcbp_lattice* h) {
+  return h->path_req != LCBP_PATH_GENERIC && zm_march_ok(h->nx, h->ny, h->nz) && !(h->p.l2_set && h->p.L2 != h->p.K);
+}
+
+// flow off: the Heun kernels on the Q mirror
+bool use_heun(const lcbp_lattice* h) { return mirror_shape(h) && !h->p.flow_on; }
+
 // whether the step runs the z-marching kernels
 bool use_fast(lcbp_lattice* h) {
-  if (h->path_req == LCBP_PATH_GENERIC || !h->p.flow_on || h->p.coupling != LCBP_JACOBI ||
-      !zm_march_ok(h->nx, h->ny, h->nz) || (h->p.l2_set && h->p.L2 != h->p.K))
-    return false;
+  if (!mirror_shape(h) || !h->p.flow_on || h->p.coupling != LCBP_JACOBI) return false;
   if (!h->tmaps_ok) {
     static std::once_flag prep32, prep64;
     if (h->dtype == LCBP_F64) std::call_once(prep64, [] { zm_prepare<double>(); });
@@ -702,9 +709,31 @@ StepArgs step_args(lcbp_lattice* h) {
   return a;
 }
 
+// Q* goes to the mirror-sized buffer behind the padded scratch
+HeunArgs heun_args(lcbp_lattice* h, const void* model) {
+  HeunArgs a{};
+  a.nx = h->nx;
+  a.ny = h->ny;
+  a.nz = h->nz;
+  a.model = model;
+  a.q = h->qm;
+  a.qs = static_cast<char*>(h->pq) + (size_t)zm_pq_elems(h->nx, h->ny, h->nz) * h->es;
+  a.u = nullptr;
+  a.q_wall = h->p.walls_z ? h->p.q_wall : nullptr;
+  a.mid = nullptr;
+  return a;
+}
+
+cudaError_t launch_heun_step(lcbp_lattice* h, const HeunArgs& a) {
+  return h->dtype == LCBP_F64 ? launch_heun<double>(a, h->stream) : launch_heun<float>(a, h->stream);
+}
+
 cudaError_t eager_step(lcbp_lattice* h) {
   cudaError_t e;
-  if (use_fast(h)) {
+  if (use_heun(h)) {
+    const ModelBuf mb = host_model(h);
+    e = launch_heun_step(h, heun_args(h, mb.bytes));
+  } else if (use_fast(h)) {
     const ModelBuf mb = host_model(h);
     e = launch_zm(h, zm_args(h, mb.bytes));
   } else {
@@ -1209,9 +1238,9 @@ int lcbp_step(lcbp_lattice* h, int nsteps) {
   if (nsteps < 0) return fail(LCBP_EINVAL, "nsteps < 0");
   if (h->p.flow_on && !h->f_ready) return fail(LCBP_ESTATE, "initialise f before stepping with flow on");
   if (nsteps == 0) return LCBP_OK;
-  const bool fast = use_fast(h);
+  const bool fast = use_fast(h), mirror = fast || use_heun(h);
   {
-    const int rs = fast ? sync_mirror(h) : sync_flat(h);
+    const int rs = mirror ? sync_mirror(h) : sync_flat(h);
     if (rs) return rs;
   }
   if (fast && h->zc == 0) {
@@ -1219,7 +1248,7 @@ int lcbp_step(lcbp_lattice* h, int nsteps) {
     if (rc) return rc;
   }
   // the kernel set's copy of the state is the one that changes
-  if (fast) h->flat_ok = false;
+  if (mirror) h->flat_ok = false;
   else h->mirror_ok = false;
   cudaError_t e = cudaSuccess;
   int left = nsteps;
@@ -1258,18 +1287,18 @@ int lcbp_profile_steps(lcbp_lattice* h, int nsteps, double* kernel_ms, int capac
   CHECK_H(h);
   if (nsteps < 1 || !kernel_ms || !nkernels) return fail(LCBP_EINVAL, "need nsteps >= 1 and output arrays");
   if (h->p.flow_on && !h->f_ready) return fail(LCBP_ESTATE, "initialise f before stepping with flow on");
-  const bool fast = use_fast(h);
+  const bool fast = use_fast(h), heun = use_heun(h);
   {
-    const int rs = fast ? sync_mirror(h) : sync_flat(h);
+    const int rs = fast || heun ? sync_mirror(h) : sync_flat(h);
     if (rs) return rs;
   }
   if (fast && h->zc == 0) {
     int rc = tune_zc(h);
     if (rc) return rc;
   }
-  if (fast) h->flat_ok = false;
+  if (fast || heun) h->flat_ok = false;
   else h->mirror_ok = false;
-  const int nk = fast ? 2 : kernels_per_step(h->p.flow_on, h->p.coupling);
+  const int nk = fast || heun ? 2 : kernels_per_step(h->p.flow_on, h->p.coupling);
   *nkernels = nk;
   if (capacity < nk) return fail(LCBP_EINVAL, "kernel_ms holds %d values, need %d", capacity, nk);
   std::vector<cudaEvent_t> ev((size_t)nsteps * (nk + 1));
@@ -1282,6 +1311,14 @@ int lcbp_profile_steps(lcbp_lattice* h, int nsteps, double* kernel_ms, int capac
       ZmArgs a = zm_args(h, mb.bytes);
       a.events = ev.data() + (size_t)s * (nk + 1);
       e = launch_zm(h, a);
+    } else if (heun) {
+      const ModelBuf mb = host_model(h);
+      HeunArgs a = heun_args(h, mb.bytes);
+      cudaEvent_t* const es = ev.data() + (size_t)s * (nk + 1);
+      a.mid = es[1];
+      cudaEventRecord(es[0], h->stream);
+      e = launch_heun_step(h, a);
+      cudaEventRecord(es[2], h->stream);
     } else {
       StepArgs a = step_args(h);
       a.events = ev.data() + (size_t)s * (nk + 1);

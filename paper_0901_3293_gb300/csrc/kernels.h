@@ -234,6 +234,19 @@ inline long long zm_pq_elems(int nx, int ny, int nz) {
   return (long long)kZmPQ * (nx + kZmPadX) * (ny + 2) * nz;
 }
 
+// Heun step of Q alone on the Q mirror, in place (heun.cu)
+struct HeunArgs {
+  int nx, ny, nz;
+  const void* model;     // host copy of Model<real>
+  void* q;               // Q mirror (images written too)
+  void* qs;              // Q* scratch, laid out as the Q mirror (its own sites only)
+  const void* u;         // rho u mirror of the velocity that drives Q; nullptr: u = 0
+  const double* q_wall;  // walls in z with this anchored Q (5 values), or nullptr: periodic
+  cudaEvent_t mid;       // optional: recorded between the two kernels
+};
+template <typename real>
+cudaError_t launch_heun(const HeunArgs& a, cudaStream_t s);
+
 // box widths of 32-wide tiles (narrow ones: tile width + 8, + 2, + 2)
 constexpr int kZmBoxX = 40;   // sites per TMA box row of the populations and of the Q mirror (x0 - 4 ..)
 constexpr int kZmBoxXP = 34;  // sites per TMA box row of the padded scratch (x0 - 1 .. x0 + 32)

@@ -28,6 +28,7 @@
 #include "common.cuh"
 #include "kernels.h"
 #include "tma.cuh"
+#include "zm.cuh"
 
 namespace lcbp {
 
@@ -54,11 +55,6 @@ static_assert(StateBox::QW == ZM_BX && StateBox::UW == kZmBoxXU && ZM_TX + 2 == 
 __host__ __device__ constexpr int align_elems(int elems, int esize) {
   // round an element count up so that it spans a multiple of 128 bytes
   return ((elems * esize + 127) / 128) * 128 / esize;
-}
-
-__device__ __forceinline__ int wrap(int v, int n) {
-  v %= n;
-  return v < 0 ? v + n : v;
 }
 
 // Sites per thread (SPT): with SPT = 2 a thread computes rows y and y + TY/2 of
@@ -95,39 +91,6 @@ __device__ __forceinline__ Sym5<typename LaneT<real, SPT>::V> ld5v(const real* s
   v.yy = vld<SPT>(sl, 3 * cs + i0, 3 * cs + i1);
   v.yz = vld<SPT>(sl, 4 * cs + i0, 4 * cs + i1);
   return v;
-}
-// The four values at 16-byte aligned element i (a group of the padded
-// scratch), as one vector access: float4, or two double2 for FP64.
-template <typename real>
-__device__ __forceinline__ void ld4(const real* p, int i, real v[4]) {
-  if constexpr (sizeof(real) == 4) {
-    const float4 a = *reinterpret_cast<const float4*>(p + i);
-    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
-  } else {
-    const double2 a = *reinterpret_cast<const double2*>(p + i), c = *reinterpret_cast<const double2*>(p + i + 2);
-    v[0] = a.x, v[1] = a.y, v[2] = c.x, v[3] = c.y;
-  }
-}
-template <typename real>
-__device__ __forceinline__ void st4(real* p, real a, real b, real c, real d) {
-  if constexpr (sizeof(real) == 4) {
-    *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
-  } else {
-    *reinterpret_cast<double2*>(p) = make_double2(a, b);
-    *reinterpret_cast<double2*>(p + 2) = make_double2(c, d);
-  }
-}
-// st4 to global memory as a streaming store (evict-first in L2): the
-// step's outputs, which no CTA of the kernel reads again, leave L2 to the
-// staged halos and pulled populations that neighbouring tiles share
-template <typename real>
-__device__ __forceinline__ void st4g(real* p, real a, real b, real c, real d) {
-  if constexpr (sizeof(real) == 4) {
-    __stcs(reinterpret_cast<float4*>(p), make_float4(a, b, c, d));
-  } else {
-    __stcs(reinterpret_cast<double2*>(p), make_double2(a, b));
-    __stcs(reinterpret_cast<double2*>(p + 2), make_double2(c, d));
-  }
 }
 // a group at element i0 (lane 0) and i1 (lane 1)
 template <int SPT, typename real>
@@ -679,15 +642,6 @@ __global__ void __launch_bounds__(qside_threads<TY, SPT, TX>(), sizeof(real) == 
 // its best planes per CTA: 33 for 62 us at 32^3 (the step 97.7 -> 79.5 us), 185
 // for 295 us at 64^3 (585 -> 454), 1.36 for 2.01 ms at 128^3 (4.15 -> 3.41).
 // ---------------------------------------------------------------------------
-// plain (coherent) vector loads: the kernel before may still have been writing
-// these buffers when this one was launched
-template <typename real>
-__device__ __forceinline__ Sym5<real> qmirror_at(const real* Q, int cq4, int o) {
-  real v[4];
-  ld4(Q, 4 * o, v);
-  return {v[0], v[1], v[2], v[3], Q[cq4 + o]};
-}
-
 // Site of a CTA's thread: tile bt of TX x TY sites of one plane
 template <int TY>
 __device__ __forceinline__ bool plane_site(const ZmGeom& G, int bt, int& x, int& y, int& z) {
@@ -900,32 +854,6 @@ __global__ void __launch_bounds__(ZM_TX* TY) k_qsite_batch(ZmBatch B, const Repl
     const Model<real> m = reps[r].m;
     qsite_body<real, TY, false>(G, m, it.bt, Q + qm0 + (long long)it.j * 5 * G.cq,
                                 U + um0 + (long long)it.j * 4 * G.cu, nullptr, tau, pqr, Sym5<real>{});
-  }
-}
-
-// The positions of a padded mirror (site x at column x + px, y at row y + h)
-// that hold the value of site (gx, gy): its own, and each ghost position in
-// the h columns and rows next to the lattice whose periodic image it is
-// (lattice faces only; nx >= 2h gives a site at most one x image).  put1(X, Y)
-// is called for each.
-template <typename F>
-__device__ __forceinline__ void mirror_positions(int px, int h, int nx, int ny, int gx, int gy, F&& put1) {
-  const int X = gx + px, Y = gy + h;
-  put1(X, Y);
-  if (gx >= h && gx < nx - h && gy >= h && gy < ny - h) return;
-  // x = nx + gx (site gx < h) or x = gx - nx (site gx >= nx - h)
-  const int xg = gx < h ? nx + px + gx : (gx >= nx - h ? gx - nx + px : -1);
-  if (xg >= 0) put1(xg, Y);
-  for (int g = 0; g < h; ++g) {  // ghost rows y = g - h and y = ny + g (several when ny < 2h)
-    const int ya = wrap(g - h, ny) == gy ? g : -1, yb = wrap(ny + g, ny) == gy ? ny + h + g : -1;
-    if (ya >= 0) {
-      put1(X, ya);
-      if (xg >= 0) put1(xg, ya);
-    }
-    if (yb >= 0) {
-      put1(X, yb);
-      if (xg >= 0) put1(xg, yb);
-    }
   }
 }
 
@@ -1567,25 +1495,6 @@ ZmGeom zm_geom(int nx, int ny, int nz, int zc, int tx, int ty) {
   G.cq = (long long)G.nxm * G.nyq * nz;
   G.cu = (long long)G.nxm * G.nyu * nz;
   return G;
-}
-
-// Launch with the programmatic attribute: the kernel's CTAs start as the
-// previous kernel of the stream drains, and wait for it in grid_wait.  It hides
-// the launch and the barrier set-up of each kernel: 12.5 -> 10.3 us per FP32 step
-// at 32^3, 94.5 -> 93.5 us at 64 x 64 x 256 (two-step graphs).
-template <typename... Params, typename... Args>
-void launch_dependent(void (*kernel)(Params...), int grid, int threads, size_t smem, cudaStream_t s, Args&&... args) {
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t c{};
-  c.gridDim = dim3(grid);
-  c.blockDim = dim3(threads);
-  c.dynamicSmemBytes = smem;
-  c.stream = s;
-  c.attrs = &at;
-  c.numAttrs = 1;
-  cudaLaunchKernelEx(&c, kernel, Params(args)...);
 }
 
 template <typename real, int SQ, int SPT, bool WALLS, int TX = ZM_TX>

@@ -1,8 +1,9 @@
 """The kernels that AUTO picks for each kind of step against the generic ones.
 
 Widths that are no multiple of 4 (the z-marching kernels with plain row
-prefetches), with and without walls, on shapes with ragged tiles in x and y,
-several tiles and z-chunks, and the smallest width.
+prefetches) and steps with the flow off (the Heun kernels on the Q mirror), with
+and without walls, on shapes with ragged tiles in x and y, several tiles and
+z-chunks, and the smallest width.
 """
 
 import numpy as np
@@ -31,11 +32,11 @@ def pair(L, shape, dtype, mode):
     out = []
     for path in (L.PATH_AUTO, L.PATH_GENERIC):
         lat = L.Lattice(nx, ny, nz, dtype=dtype).set_path(path)
-        lat.set_flow(flow_on=mode != "noflow", coupling=L.GAUSS_SEIDEL if mode == "gauss_seidel" else L.JACOBI)
-        if mode == "walls":
+        lat.set_flow(flow_on="noflow" not in mode, coupling=L.GAUSS_SEIDEL if mode == "gauss_seidel" else L.JACOBI)
+        if "walls" in mode:
             lat.set_walls(True, (0.2, 0.0, 0.0, -0.1, 0.0))
         lat.init_q(L.BPII, 0.3, noise=1e-3, seed=4)
-        if mode != "noflow":
+        if "noflow" not in mode:
             lat.init_f_equilibrium(1.0)
         out.append(lat)
     return out
@@ -52,7 +53,7 @@ def check(L, shape, dtype, mode, steps):
         lat.step(steps)
     tq, tu = TOL[dtype]
     assert np.abs(a.read_q() - b.read_q()).max() < tq
-    if mode != "noflow":
+    if "noflow" not in mode:
         assert np.abs(a.read_u() - b.read_u()).max() < tu
         assert np.abs(a.read_f() - b.read_f()).max() <= (2.0 ** -23 if dtype == "f32" else tq)
 
@@ -62,3 +63,24 @@ def check(L, shape, dtype, mode, steps):
 @pytest.mark.parametrize("shape", SHAPES)
 def test_marching_kernels_match_generic(lcbp, shape, dtype, mode):
     check(lcbp, shape, dtype, mode, 11)
+
+
+# 128 positions per CTA: one partly filled CTA, several, a width of 32 lanes; the
+# longest chunk (16 planes) with a shorter last one
+@pytest.mark.parametrize("mode", ["noflow", "noflow_walls"])
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("shape", [(3, 5, 4), (1, 11, 13), (37, 19, 45), (8, 16, 32), (50, 160, 250)])
+def test_heun_kernels_match_generic(lcbp, shape, dtype, mode):
+    check(lcbp, shape, dtype, mode, 10)
+
+
+def test_flow_switched_on_after_relaxation(lcbp):
+    """The state moves between the kernel sets with its mirrors' images intact."""
+    a, b = pair(lcbp, (12, 10, 36), "f64", "noflow")
+    for lat in (a, b):
+        lat.step(5)
+        lat.set_flow(flow_on=True).init_f_equilibrium(1.0).step(3)
+        lat.set_flow(flow_on=False).step(3)
+        lat.set_flow(flow_on=True).step(2)
+    assert np.abs(a.read_q() - b.read_q()).max() < 1e-13
+    assert np.abs(a.read_u() - b.read_u()).max() < 1e-14

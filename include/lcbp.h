@@ -258,7 +258,8 @@ LCBP_API int lcbp_step(lcbp_lattice *h, int nsteps);
  * LB predictor-corrector and the Heun corrector), 5 with Gauss-Seidel
  * coupling (field, force, lb, predict, correct), 3 with flow off (field,
  * predict, correct); with flow off on shapes that the fast kernels serve and
- * without LCBP_PATH_GENERIC 2 (predict, correct).  Errors: LCBP_EINVAL if
+ * without LCBP_PATH_GENERIC 2 (predict, correct), with Gauss-Seidel coupling
+ * there 4 (qside, lb, predict, correct).  Errors: LCBP_EINVAL if
  * capacity < *nkernels.
  */
 LCBP_API int lcbp_profile_steps(lcbp_lattice *h, int nsteps, double *kernel_ms, int capacity, int *nkernels);
@@ -269,7 +270,8 @@ LCBP_API int lcbp_profile_steps(lcbp_lattice *h, int nsteps, double *kernel_ms, 
  * -- whenever flow is on, coupling is Jacobi and nx is a multiple of 4; other
  * widths of at least 4 run the same two kernels (lcbp_get_path names only the
  * multiples of 4 fast).  With flow off the same shapes run two kernels of the
- * Heun step on the padded Q.  Otherwise, or with LCBP_PATH_GENERIC, three
+ * Heun step on the padded Q, and with Gauss-Seidel coupling the LB halves of
+ * the fast kernels followed by those two.  Otherwise, or with LCBP_PATH_GENERIC, three
  * one-thread-per-site kernels.
  * FP32 fast kernels come in two builds, one or two lattice sites per thread
  * (the latter on packed FP32x2 arithmetic); AUTO times both, LCBP_PATH_FAST1
@@ -287,7 +289,7 @@ LCBP_API int lcbp_set_path(lcbp_lattice *h, int path);
  * shape and dtype, writing scratch buffers only; AUTO results persist in the
  * file named by the environment variable LCBP_AUTOTUNE_CACHE, if set
  * (lines "nx ny nz dtype planes sites planes_q", dtype + 100 for a lattice
- * with walls; see lcbp_get_tuning for the last two fields; a line without
+ * with walls, + 200 for Gauss-Seidel coupling; see lcbp_get_tuning for the last two fields; a line without
  * planes_q gives both kernels the same planes).  Any pointer may be NULL.
  */
 LCBP_API int lcbp_get_path(lcbp_lattice *h, int *fast, int *planes_per_cta, int *sites_per_thread);

@@ -281,6 +281,14 @@ int check_dims(int nx, int ny, int nz) {
 
 void drop_graph(lcbp_lattice* h);
 
+// the fast kernels' tile shape and tuning follow the path, walls and coupling
+void retile(lcbp_lattice* h) {
+  h->tmaps_ok = false;
+  h->zc = 0;
+  h->spt = 0;
+  h->spt_q = 0;
+}
+
 int upload_replica(lcbp_lattice* h) {
   drop_graph(h);  // the fast path takes the model coefficients as kernel arguments
   std::vector<char> buf(replica_bytes(h->dtype));
@@ -395,8 +403,11 @@ bool make_scratch_tmap(CUtensorMap* tm, void* base, int nxp, int nyp, int nz, in
   return encode_tiled(tm, base, 4, dims, strides, box, dtype);
 }
 
-// tile width of the fast kernels (two sites per thread exist for 32-wide tiles only)
+bool seidel(const lcbp_lattice* h) { return h->p.coupling == LCBP_GAUSS_SEIDEL; }
+
+// tile width of the fast kernels (two sites per thread, and Gauss-Seidel coupling, have 32-wide tiles only)
 int tile_x(const lcbp_lattice* h) {
+  if (seidel(h)) return 32;
   return h->path_req == LCBP_PATH_FAST2 && !h->p.walls_z ? 32 : zm_lattice_tile_x(h->nx, h->dtype != LCBP_F64);
 }
 int tile_y(const lcbp_lattice* h) {
@@ -412,9 +423,11 @@ bool mirror_shape(const lcbp_lattice* h) {
 // flow off: the Heun kernels on the Q mirror
 bool use_heun(const lcbp_lattice* h) { return mirror_shape(h) && !h->p.flow_on; }
 
-// whether the step runs the z-marching kernels
-bool use_fast(lcbp_lattice* h) {
-  if (!mirror_shape(h) || !h->p.flow_on || h->p.coupling != LCBP_JACOBI) return false;
+// whether the step runs the z-marching kernels (both halves of a Jacobi step, or
+// the LB half of a Gauss-Seidel step, whose Q half is the Heun kernels': 80 x 64 x
+// 48 FP32 takes 39 us per step so, 53 us on the five generic kernels)
+bool use_march(lcbp_lattice* h) {
+  if (!mirror_shape(h) || !h->p.flow_on) return false;
   if (!h->tmaps_ok) {
     static std::once_flag prep32, prep64;
     if (h->dtype == LCBP_F64) std::call_once(prep64, [] { zm_prepare<double>(); });
@@ -451,6 +464,10 @@ bool use_fast(lcbp_lattice* h) {
   return true;
 }
 
+// the fast path as lcbp_get_path reports it: Jacobi coupling and widths that are
+// a multiple of 4 (others run the same kernels)
+bool fast_named(lcbp_lattice* h) { return use_march(h) && !seidel(h) && h->nx % 4 == 0; }
+
 ZmArgs zm_args(lcbp_lattice* h, const void* model) {
   ZmArgs a{};
   a.tx = tile_x(h);
@@ -483,6 +500,7 @@ ZmArgs zm_args(lcbp_lattice* h, const void* model) {
   a.err = h->d_err;
   a.events = nullptr;
   a.q_wall = h->p.walls_z ? h->p.q_wall : nullptr;
+  a.lb_only = seidel(h);
   return a;
 }
 
@@ -521,10 +539,10 @@ std::mutex g_tune_mu;
 std::map<std::string, Tuning> g_tune;
 bool g_tune_loaded = false;
 
-// "nx ny nz dtype", with 100 added to dtype for a lattice with walls
+// "nx ny nz dtype", with 100 added to dtype for a lattice with walls and 200 for Gauss-Seidel coupling
 std::string tune_key(const lcbp_lattice* h) {
   char k[64];
-  snprintf(k, sizeof(k), "%d %d %d %d", h->nx, h->ny, h->nz, h->dtype + (h->p.walls_z ? 100 : 0));
+  snprintf(k, sizeof(k), "%d %d %d %d", h->nx, h->ny, h->nz, h->dtype + (h->p.walls_z ? 100 : 0) + (seidel(h) ? 200 : 0));
   return k;
 }
 
@@ -562,12 +580,12 @@ std::vector<int> zc_candidates(const lcbp_lattice* h, int spt) {
 int tune_zc(lcbp_lattice* h) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   const char* path = std::getenv("LCBP_AUTOTUNE_CACHE");
-  // (narrow tiles: one site per thread only)
-  const int spt_max = tile_x(h) < 32 ? 1 : h->dtype == LCBP_F64 ? zm_spt_max<double>() : zm_spt_max<float>();
+  // (narrow tiles and Gauss-Seidel coupling: one site per thread only)
+  const int spt_max = tile_x(h) < 32 || seidel(h) ? 1 : h->dtype == LCBP_F64 ? zm_spt_max<double>() : zm_spt_max<float>();
   // a pinned sites-per-thread choice tunes only the planes per CTA, uncached
   const bool pinned = h->path_req == LCBP_PATH_FAST1 || h->path_req == LCBP_PATH_FAST2;
   // (walls: one site per thread only)
-  const int spt_lo = h->path_req == LCBP_PATH_FAST2 && !h->p.walls_z ? 2 : 1;
+  const int spt_lo = h->path_req == LCBP_PATH_FAST2 && !h->p.walls_z && !seidel(h) ? 2 : 1;
   const int spt_hi = h->path_req == LCBP_PATH_FAST1 || h->p.walls_z ? 1 : spt_max;
   if (path && !g_tune_loaded) {
     g_tune_loaded = true;
@@ -733,9 +751,14 @@ cudaError_t eager_step(lcbp_lattice* h) {
   if (use_heun(h)) {
     const ModelBuf mb = host_model(h);
     e = launch_heun_step(h, heun_args(h, mb.bytes));
-  } else if (use_fast(h)) {
+  } else if (use_march(h)) {
     const ModelBuf mb = host_model(h);
     e = launch_zm(h, zm_args(h, mb.bytes));
+    if (e == cudaSuccess && seidel(h)) {
+      HeunArgs a = heun_args(h, mb.bytes);
+      a.u = h->um[h->cur ^ 1];
+      e = launch_heun_step(h, a);
+    }
   } else {
     const StepArgs a = step_args(h);
     e = h->dtype == LCBP_F64 ? launch_step<double>(a, h->stream) : launch_step<float>(a, h->stream);
@@ -1082,6 +1105,7 @@ int lcbp_set_flow(lcbp_lattice* h, double tau_f, double rho0, double xi, double 
   int rc = check_params(p);
   if (rc) return rc;
   if (p.flow_on != h->p.flow_on || p.coupling != h->p.coupling) drop_graph(h);
+  if (p.coupling != h->p.coupling) retile(h);
   h->p = p;
   return upload_replica(h);
 }
@@ -1109,12 +1133,7 @@ int lcbp_set_walls(lcbp_lattice* h, int walls_z, const double* q_wall5) {
   }
   // the fast kernels take q_wall as a launch argument: recapture the step
   drop_graph(h);
-  if (p.walls_z != h->p.walls_z) {
-    h->tmaps_ok = false;
-    h->zc = 0;  // tuned separately with walls
-    h->spt = 0;
-    h->spt_q = 0;
-  }
+  if (p.walls_z != h->p.walls_z) retile(h);
   h->p = p;
   return upload_replica(h);
 }
@@ -1238,7 +1257,7 @@ int lcbp_step(lcbp_lattice* h, int nsteps) {
   if (nsteps < 0) return fail(LCBP_EINVAL, "nsteps < 0");
   if (h->p.flow_on && !h->f_ready) return fail(LCBP_ESTATE, "initialise f before stepping with flow on");
   if (nsteps == 0) return LCBP_OK;
-  const bool fast = use_fast(h), mirror = fast || use_heun(h);
+  const bool fast = use_march(h), mirror = fast || use_heun(h);
   {
     const int rs = mirror ? sync_mirror(h) : sync_flat(h);
     if (rs) return rs;
@@ -1287,7 +1306,7 @@ int lcbp_profile_steps(lcbp_lattice* h, int nsteps, double* kernel_ms, int capac
   CHECK_H(h);
   if (nsteps < 1 || !kernel_ms || !nkernels) return fail(LCBP_EINVAL, "need nsteps >= 1 and output arrays");
   if (h->p.flow_on && !h->f_ready) return fail(LCBP_ESTATE, "initialise f before stepping with flow on");
-  const bool fast = use_fast(h), heun = use_heun(h);
+  const bool fast = use_march(h), heun = use_heun(h);
   {
     const int rs = fast || heun ? sync_mirror(h) : sync_flat(h);
     if (rs) return rs;
@@ -1298,7 +1317,7 @@ int lcbp_profile_steps(lcbp_lattice* h, int nsteps, double* kernel_ms, int capac
   }
   if (fast || heun) h->flat_ok = false;
   else h->mirror_ok = false;
-  const int nk = fast || heun ? 2 : kernels_per_step(h->p.flow_on, h->p.coupling);
+  const int nk = fast && seidel(h) ? 4 : fast || heun ? 2 : kernels_per_step(h->p.flow_on, h->p.coupling);
   *nkernels = nk;
   if (capacity < nk) return fail(LCBP_EINVAL, "kernel_ms holds %d values, need %d", capacity, nk);
   std::vector<cudaEvent_t> ev((size_t)nsteps * (nk + 1));
@@ -1309,8 +1328,16 @@ int lcbp_profile_steps(lcbp_lattice* h, int nsteps, double* kernel_ms, int capac
     if (fast) {
       const ModelBuf mb = host_model(h);
       ZmArgs a = zm_args(h, mb.bytes);
-      a.events = ev.data() + (size_t)s * (nk + 1);
+      cudaEvent_t* const es = ev.data() + (size_t)s * (nk + 1);
+      a.events = es;
       e = launch_zm(h, a);
+      if (e == cudaSuccess && seidel(h)) {
+        HeunArgs b = heun_args(h, mb.bytes);
+        b.u = h->um[h->cur ^ 1];
+        b.mid = es[3];
+        e = launch_heun_step(h, b);
+        cudaEventRecord(es[4], h->stream);
+      }
     } else if (heun) {
       const ModelBuf mb = host_model(h);
       HeunArgs a = heun_args(h, mb.bytes);
@@ -1348,16 +1375,13 @@ int lcbp_set_path(lcbp_lattice* h, int path) {
     return fail(LCBP_EINVAL, "two sites per thread exist for FP32 lattices only");
   drop_graph(h);
   h->path_req = path;
-  h->tmaps_ok = false;  // the tile shape follows the choice
-  h->zc = 0;  // retune for the new choice
-  h->spt = 0;
-  h->spt_q = 0;
+  retile(h);
   return LCBP_OK;
 }
 
 int lcbp_get_tuning(lcbp_lattice* h, int* planes_per_cta, int* spt_lb, int* spt_q, int* planes_per_cta_q) {
   CHECK_H(h);
-  const bool f = use_fast(h) && h->nx % 4 == 0 && h->zc > 0;
+  const bool f = fast_named(h) && h->zc > 0;
   if (planes_per_cta) *planes_per_cta = f ? h->zc : 0;
   if (planes_per_cta_q) *planes_per_cta_q = f ? (h->zc_q > 0 ? h->zc_q : h->zc) : 0;
   if (spt_lb) *spt_lb = f ? h->spt : 0;
@@ -1367,8 +1391,7 @@ int lcbp_get_tuning(lcbp_lattice* h, int* planes_per_cta, int* spt_lb, int* spt_
 
 int lcbp_get_path(lcbp_lattice* h, int* fast, int* planes_per_cta, int* sites_per_thread) {
   CHECK_H(h);
-  // ("fast" names the widths that are a multiple of 4; others run the same kernels with plain row prefetches)
-  const bool f = use_fast(h) && h->nx % 4 == 0;
+  const bool f = fast_named(h);
   if (fast) *fast = f ? 1 : 0;
   if (planes_per_cta) *planes_per_cta = f ? h->zc : 0;
   if (sites_per_thread) *sites_per_thread = f && h->zc > 0 ? h->spt : 0;
@@ -1590,7 +1613,7 @@ int lcbp_load(lcbp_lattice* h, const char* path) {
   if (p.flow_on != h->p.flow_on || p.coupling != h->p.coupling || p.walls_z != h->p.walls_z ||
       p.l2_set != h->p.l2_set || p.L2 != h->p.L2)
     drop_graph(h);
-  if (p.walls_z != h->p.walls_z) h->tmaps_ok = false;
+  if (p.walls_z != h->p.walls_z || p.coupling != h->p.coupling) retile(h);
   h->p = p;
   rc = upload_replica(h);
   if (rc) return rc;

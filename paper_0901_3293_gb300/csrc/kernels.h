@@ -227,6 +227,7 @@ struct ZmArgs {
   cudaEvent_t* events;   // optional: 3 events around the two kernels
   int reps;              // launches of each kernel in turn (0: one); the tuner's, to time short kernels
   const double* q_wall;  // walls in z with this anchored Q (5 values), or nullptr: periodic
+  int lb_only;           // 1: the LB half of a Gauss-Seidel step (32-wide tiles, one site per thread; Q is left alone)
 };
 
 // elements of the padded scratch of one nx x ny x nz lattice

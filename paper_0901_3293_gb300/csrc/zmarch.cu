@@ -206,7 +206,8 @@ constexpr int qside_threads() {
 // WALLS: walls half a spacing below z = 0 and above z = nz-1.  The ghost
 // planes z = -1 and z = nz hold the anchored qw in every Q stencil, carry no
 // molecular field (tau = 0 there) and the velocity -u of the adjacent plane.
-template <typename real, int TY, int SPT, bool BATCH, bool WALLS, int TX = ZM_TX>
+// LBO: the LB-ready coefficients only, no Heun predictor (Gauss-Seidel coupling).
+template <typename real, int TY, int SPT, bool BATCH, bool WALLS, int TX = ZM_TX, bool LBO = false>
 __device__ __forceinline__ void qside_body(const CUtensorMap* tmQ, const CUtensorMap* tmQ1, const CUtensorMap* tmU,
                                            const ZmGeom G,
                                            const Model<real> m, int bt, int rc, const real* __restrict__ bext,
@@ -544,20 +545,23 @@ __device__ __forceinline__ void qside_body(const CUtensorMap* tmQ, const CUtenso
       const real* uc = uslot(z);
       const real* up = uslot(z + 1);
       const int u0 = (ty + 1) * B::UW + (tx + B::UX), u1 = u0 + TYH * B::UW;
-      V u[3], w[3][3], drho;
-      {
-        V c[4], xp[4], xm[4], yp[4], ym[4], zp[4], zm[4];  // [rho - 1, u_x, u_y, u_z]
-        ldu(uc, u0, u1, c);
+      V u[3], drho;
+      V c[4];  // [rho - 1, u_x, u_y, u_z]
+      ldu(uc, u0, u1, c);
+      drho = c[0];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) u[a] = c[1 + a];
+      V qv[5] = {V(0), V(0), V(0), V(0), V(0)};  // Q*
+      if constexpr (!LBO) {
+        V w[3][3], xp[4], xm[4], yp[4], ym[4], zp[4], zm[4];
         ldu(uc, u0 + 1, u1 + 1, xp);
         ldu(uc, u0 - 1, u1 - 1, xm);
         ldu(uc, u0 + B::UW, u1 + B::UW, yp);
         ldu(uc, u0 - B::UW, u1 - B::UW, ym);
         ldu(up, u0, u1, zp);
         ldu(um, u0, u1, zm);
-        drho = c[0];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-          u[a] = c[1 + a];
           w[a][0] = xp[1 + a] - xm[1 + a];  // twice the central derivatives
           w[a][1] = yp[1 + a] - ym[1 + a];
           V upz = zp[1 + a], umz = zm[1 + a];
@@ -565,8 +569,13 @@ __device__ __forceinline__ void qside_body(const CUtensorMap* tmQ, const CUtenso
           if (WALLS && z == nz - 1) upz = -u[a];
           w[a][2] = upz - umz;
         }
+        const Sym5<V> r = be_rate<true>(q, h, dq, u, w, mv, true);
+        qv[0] = q.xx + r.xx;
+        qv[1] = q.xy + r.xy;
+        qv[2] = q.xz + r.xz;
+        qv[3] = q.yy + r.yy;
+        qv[4] = q.yz + r.yz;
       }
-      const Sym5<V> r = be_rate<true>(q, h, dq, u, w, mv, true);
       // The site's 16 values (four groups; rho - 1 in the last place) of the
       // padded scratch for lane k, at the site's position and its images
       const int nxp = G.nxp, nyp = G.nyp, gs = 4 * G.nxp * G.nyp;  // gs: group stride
@@ -585,11 +594,10 @@ __device__ __forceinline__ void qside_body(const CUtensorMap* tmQ, const CUtenso
             st4g(d, g0[0], g0[1], g0[2], g0[3]);
             st4g(d + gs, g1[0], g1[1], g1[2], g1[3]);
             st4g(d + 2 * gs, g2[0], g2[1], g2[2], g2[3]);
-            st4g(d + 3 * gs, g3[0], g3[1], g3[2], g3[3]);
+            if constexpr (!LBO) st4g(d + 3 * gs, g3[0], g3[1], g3[2], g3[3]);
           });
         }
       };
-      const V qv[5] = {q.xx + r.xx, q.xy + r.xy, q.xz + r.xz, q.yy + r.yy, q.yz + r.yz};
       V bt[3] = {bx, by, bz};
       if (bext) {
         int sb[SPT];
@@ -620,12 +628,12 @@ __device__ __forceinline__ void qside_body(const CUtensorMap* tmQ, const CUtenso
 }
 
 // FP32: two CTAs per SM (shared memory allows two; the bound keeps the registers within it)
-template <typename real, int TY, int SPT, bool WALLS, int TX = ZM_TX>
+template <typename real, int TY, int SPT, bool WALLS, int TX = ZM_TX, bool LBO = false>
 __global__ void __launch_bounds__(qside_threads<TY, SPT, TX>(), sizeof(real) == 4 ? 2 : 1)
     k_qside(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmQ1,
             const __grid_constant__ CUtensorMap tmU, ZmGeom G, Model<real> m, const real* __restrict__ bext,
             real* __restrict__ pq, int* __restrict__ err, Sym5<real> qw) {
-  qside_body<real, TY, SPT, false, WALLS, TX>(&tmQ, &tmQ1, &tmU, G, m, blockIdx.x, 0, bext, pq, err, qw);
+  qside_body<real, TY, SPT, false, WALLS, TX, LBO>(&tmQ, &tmQ1, &tmU, G, m, blockIdx.x, 0, bext, pq, err, qw);
 }
 
 // ---------------------------------------------------------------------------
@@ -651,7 +659,7 @@ __device__ __forceinline__ bool plane_site(const ZmGeom& G, int bt, int& x, int&
   return x < G.nx && y < G.ny;
 }
 
-template <typename real, int TY, bool WALLS>
+template <typename real, int TY, bool WALLS, bool LBO = false>
 __device__ __forceinline__ void qsite_body(const ZmGeom& G, const Model<real>& m, int bt, const real* Q,
                                            const real* U, const real* bext, real* tau, real* pq,
                                            const Sym5<real>& qw) {
@@ -672,7 +680,7 @@ __device__ __forceinline__ void qsite_body(const ZmGeom& G, const Model<real>& m
   st.zm = wlo ? qw : qmirror_at(Q, cq4, oq(zm));
   st.zp = whi ? qw : qmirror_at(Q, cq4, oq(zp));
   Sym5<real> dq[3], sg;
-  real tu[3], u[3], w[3][3];
+  real tu[3], u[3];
   const Sym5<real> h = molecular_field<true>(st, m, dq);
   lc_stress(st.c, h, m.xi, sg, tu);
   const int s = (z * G.ny + y) * G.nx + x;
@@ -681,36 +689,43 @@ __device__ __forceinline__ void qsite_body(const ZmGeom& G, const Model<real>& m
   tau[2 * n + s] = tu[2];
   auto ou = [&](int zz) { return 4 * ((zz * G.nyu + y + B::UPY) * nxm + x + B::UPX); };
   const int ouc = ou(z);
-  real c[4], a[4], b[4];
+  real c[4], qs[5] = {};
   ld4(U, ouc, c);
 #pragma unroll
   for (int k = 0; k < 3; ++k) u[k] = c[1 + k];
-  ld4(U, ouc + 4, a);
-  ld4(U, ouc - 4, b);
+  if constexpr (!LBO) {
+    real w[3][3], a[4], b[4];
+    ld4(U, ouc + 4, a);
+    ld4(U, ouc - 4, b);
 #pragma unroll
-  for (int k = 0; k < 3; ++k) w[k][0] = a[1 + k] - b[1 + k];  // twice the central derivatives
-  ld4(U, ouc + 4 * nxm, a);
-  ld4(U, ouc - 4 * nxm, b);
+    for (int k = 0; k < 3; ++k) w[k][0] = a[1 + k] - b[1 + k];  // twice the central derivatives
+    ld4(U, ouc + 4 * nxm, a);
+    ld4(U, ouc - 4 * nxm, b);
 #pragma unroll
-  for (int k = 0; k < 3; ++k) w[k][1] = a[1 + k] - b[1 + k];
-  ld4(U, ou(zp), a);
-  ld4(U, ou(zm), b);
+    for (int k = 0; k < 3; ++k) w[k][1] = a[1 + k] - b[1 + k];
+    ld4(U, ou(zp), a);
+    ld4(U, ou(zm), b);
 #pragma unroll
-  for (int k = 0; k < 3; ++k) w[k][2] = (whi ? -u[k] : a[1 + k]) - (wlo ? -u[k] : b[1 + k]);
-  const Sym5<real> r = be_rate<true>(st.c, h, dq, u, w, m, true);
+    for (int k = 0; k < 3; ++k) w[k][2] = (whi ? -u[k] : a[1 + k]) - (wlo ? -u[k] : b[1 + k]);
+    const Sym5<real> r = be_rate<true>(st.c, h, dq, u, w, m, true);
+    qs[0] = st.c.xx + r.xx;
+    qs[1] = st.c.xy + r.xy;
+    qs[2] = st.c.xz + r.xz;
+    qs[3] = st.c.yy + r.yy;
+    qs[4] = st.c.yz + r.yz;
+  }
   real bt3[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) bt3[k] = (bext ? bext[k * n + s] : real(0)) - real(0.5) * ddot(h, dq[k]);
   real P[10];
   lb_coefficients(c[0], u, sg, bt3, m.inv_tau, P);
-  const real qs[5] = {st.c.xx + r.xx, st.c.xy + r.xy, st.c.xz + r.xz, st.c.yy + r.yy, st.c.yz + r.yz};
   const int gs = 4 * G.nxp * G.nyp;
   scratch_positions(G.nx, G.ny, x, y, [&](int X, int Y) {
     real* d = pq + ((z * kZmPQG * G.nyp + Y) * G.nxp + X) * 4;
     st4(d, P[6], P[3], P[4], P[5]);
     st4(d + gs, P[7], P[8], P[9], P[0]);
     st4(d + 2 * gs, P[1], P[2], qs[4], c[0]);
-    st4(d + 3 * gs, qs[0], qs[1], qs[2], qs[3]);
+    if constexpr (!LBO) st4(d + 3 * gs, qs[0], qs[1], qs[2], qs[3]);
   });
 }
 
@@ -740,12 +755,12 @@ __device__ __forceinline__ void qdiv_body(const ZmGeom& G, int bt, const real* t
   scratch_positions(nx, ny, x, y, [&](int X, int Y) { st4(g0 + (Y * G.nxp + X) * 4, v[0], v[1], v[2], v[3]); });
 }
 
-template <typename real, int TY, bool WALLS>
+template <typename real, int TY, bool WALLS, bool LBO>
 __global__ void __launch_bounds__(ZM_TX* TY) k_qsite(ZmGeom G, Model<real> m, const real* Q, const real* U,
                                                      const real* bext, real* tau, real* pq, Sym5<real> qw) {
   grid_wait();
   grid_launch_dependents();
-  qsite_body<real, TY, WALLS>(G, m, blockIdx.x, Q, U, bext, tau, pq, qw);
+  qsite_body<real, TY, WALLS, LBO>(G, m, blockIdx.x, Q, U, bext, tau, pq, qw);
 }
 template <typename real, int TY, bool WALLS>
 __global__ void __launch_bounds__(ZM_TX* TY) k_qdiv(ZmGeom G, const real* tau, real* pq) {
@@ -901,7 +916,8 @@ __device__ __forceinline__ void direction_sums(const V* f, V& r, V& jx, V& jy, V
 // the Q^n mirror in tile-sized boxes (for a batch the class's, with the
 // replica outermost), whose planes are prefetched into L2 one plane before
 // the loads read them
-template <typename real, int TY, int SPT, bool BATCH, bool WALLS, int TX = ZM_TX>
+// LBO: the LB update only, Q is left alone (Gauss-Seidel coupling)
+template <typename real, int TY, int SPT, bool BATCH, bool WALLS, int TX = ZM_TX, bool LBO = false>
 __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensorMap* tmU3, const CUtensorMap* tmF,
                                          const CUtensorMap* tmF1, const CUtensorMap* tmF2,
                                          const CUtensorMap* tmQ, const CUtensorMap* tmQ1, const ZmGeom& G,
@@ -997,8 +1013,10 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
         tma_prefetch_l2_4d(tmF2, xf, yb, zz, 9);
         tma_prefetch_l2_4d(tmF2, xf, yb, zz, 13);
       }
-      tma_prefetch_l2_3d(tmQ, 4 * X, Y, wrap(p - 1, nz));
-      tma_prefetch_l2_3d(tmQ1, X, Y, wrap(p - 1, nz));
+      if constexpr (!LBO) {
+        tma_prefetch_l2_3d(tmQ, 4 * X, Y, wrap(p - 1, nz));
+        tma_prefetch_l2_3d(tmQ1, X, Y, wrap(p - 1, nz));
+      }
     }
   };
   auto wait = [&](int p) {
@@ -1249,6 +1267,7 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
                          [&](int X, int Y) { st4g(rhou_new + 4 * ((z * nyu + Y) * nxm + X), a, b, c, d); });
       }
 
+      if constexpr (LBO) return;
       // Heun corrector with u^n
       // Q* at a box index: G3 = [xx xy xz yy] and G2.2 = yz
       auto QS = [&](const real* sl, int idx) {
@@ -1326,7 +1345,7 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
   }
 }
 
-template <typename real, int TY, int SPT, bool WALLS, int TX = ZM_TX>
+template <typename real, int TY, int SPT, bool WALLS, int TX = ZM_TX, bool LBO = false>
 __global__ void __launch_bounds__(TX* TY / SPT, 2)
     k_lbq(const __grid_constant__ CUtensorMap tmPQ, const __grid_constant__ CUtensorMap tmU3,
           const __grid_constant__ CUtensorMap tmF, const __grid_constant__ CUtensorMap tmF1,
@@ -1334,7 +1353,7 @@ __global__ void __launch_bounds__(TX* TY / SPT, 2)
           const __grid_constant__ CUtensorMap tmQ1, ZmGeom G, Model<real> m, const real* __restrict__ f,
           const real* __restrict__ Qin, real* __restrict__ fnew, real* __restrict__ rhou_new, real* __restrict__ Qout,
           int* __restrict__ err, Sym5<real> qw) {
-  lbq_body<real, TY, SPT, false, WALLS, TX>(&tmPQ, &tmU3, &tmF, &tmF1, &tmF2, &tmQ, &tmQ1, G, m, blockIdx.x, 0, f,
+  lbq_body<real, TY, SPT, false, WALLS, TX, LBO>(&tmPQ, &tmU3, &tmF, &tmF1, &tmF2, &tmQ, &tmQ1, G, m, blockIdx.x, 0, f,
                                             Qin, fnew, rhou_new, Qout, err, qw);
 }
 
@@ -1411,28 +1430,16 @@ constexpr int zm_max_spt() {
   return sizeof(real) == 4 ? 2 : 1;
 }
 
-template <typename real, int SPT, bool WALLS>
+template <typename real, int SPT, bool WALLS, int TX = ZM_TX, bool LBO = false>
 cudaError_t zm_prepare_spt() {
-  constexpr int TY = zm_ty<real>();
+  constexpr int TY = zm_ty<real>() * (ZM_TX / TX);
   cudaError_t e = cudaSuccess;
   if constexpr (sizeof(real) == 4)
-    e = cudaFuncSetAttribute(k_qside<real, TY, SPT, WALLS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)QsideSmem<real, TY>::bytes);
+    e = cudaFuncSetAttribute(k_qside<real, TY, SPT, WALLS, TX, LBO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)QsideSmem<real, TY, TX>::bytes);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_lbq<real, TY, SPT, WALLS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)LbqSmem<real, TY>::bytes);
-  return e;
-}
-
-// the narrow tiles of FP32 lattices
-template <bool WALLS>
-cudaError_t zm_prepare_narrow() {
-  constexpr int TY = 2 * zm_ty<float>(), TX = kZmNarrowX;
-  cudaError_t e = cudaFuncSetAttribute(k_qside<float, TY, 1, WALLS, TX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)QsideSmem<float, TY, TX>::bytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_lbq<float, TY, 1, WALLS, TX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)LbqSmem<float, TY, TX>::bytes);
+    e = cudaFuncSetAttribute(k_lbq<real, TY, SPT, WALLS, TX, LBO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)LbqSmem<real, TY, TX>::bytes);
   return e;
 }
 
@@ -1441,9 +1448,11 @@ template <typename real>
 cudaError_t zm_prepare() {
   cudaError_t e = zm_prepare_spt<real, 1, false>();
   if (e == cudaSuccess) e = zm_prepare_spt<real, 1, true>();
+  if (e == cudaSuccess) e = zm_prepare_spt<real, 1, false, ZM_TX, true>();
+  if (e == cudaSuccess) e = zm_prepare_spt<real, 1, true, ZM_TX, true>();
   if constexpr (sizeof(real) == 4) {
-    if (e == cudaSuccess) e = zm_prepare_narrow<false>();
-    if (e == cudaSuccess) e = zm_prepare_narrow<true>();
+    if (e == cudaSuccess) e = zm_prepare_spt<real, 1, false, kZmNarrowX>();
+    if (e == cudaSuccess) e = zm_prepare_spt<real, 1, true, kZmNarrowX>();
   }
   if constexpr (zm_max_spt<real>() == 2)
     if (e == cudaSuccess) e = zm_prepare_spt<real, 2, false>();
@@ -1497,7 +1506,7 @@ ZmGeom zm_geom(int nx, int ny, int nz, int zc, int tx, int ty) {
   return G;
 }
 
-template <typename real, int SQ, int SPT, bool WALLS, int TX = ZM_TX>
+template <typename real, int SQ, int SPT, bool WALLS, int TX = ZM_TX, bool LBO = false>
 cudaError_t launch_step_zm_spt(const ZmArgs& a, cudaStream_t s) {
   constexpr int TY = zm_ty<real>() * (ZM_TX / TX);
   // each kernel marches its own planes per CTA
@@ -1511,19 +1520,19 @@ cudaError_t launch_step_zm_spt(const ZmArgs& a, cudaStream_t s) {
   for (int k = 0; k < std::max(1, a.reps); ++k) {
     if constexpr (sizeof(real) == 8) {  // (tau in the population buffer that k_lbq fills)
       real* tau = static_cast<real*>(a.fnew);
-      launch_dependent(k_qsite<real, TY, WALLS>, grid_q, ZM_TX * TY, 0, s, Gq, m, static_cast<const real*>(a.q),
+      launch_dependent(k_qsite<real, TY, WALLS, LBO>, grid_q, ZM_TX * TY, 0, s, Gq, m, static_cast<const real*>(a.q),
                        static_cast<const real*>(a.rhou), static_cast<const real*>(a.bext), tau,
                        static_cast<real*>(a.pq), qw);
       launch_dependent(k_qdiv<real, TY, WALLS>, grid_q, ZM_TX * TY, 0, s, Gq, tau, static_cast<real*>(a.pq));
     } else {
-      launch_dependent(k_qside<real, TY, SQ, WALLS, TX>, grid_q, qside_threads<TY, SQ, TX>(),
+      launch_dependent(k_qside<real, TY, SQ, WALLS, TX, LBO>, grid_q, qside_threads<TY, SQ, TX>(),
                        QsideSmem<real, TY, TX>::bytes, s, *a.tm_q, *a.tm_q1, *a.tm_u, Gq, m, static_cast<const real*>(a.bext),
                        static_cast<real*>(a.pq), a.err, qw);
     }
   }
   if (a.events) cudaEventRecord(a.events[1], s);
   for (int k = 0; k < std::max(1, a.reps); ++k)
-    launch_dependent(k_lbq<real, TY, SPT, WALLS, TX>, grid, TX * TY / SPT, LbqSmem<real, TY, TX>::bytes, s, *a.tm_pq,
+    launch_dependent(k_lbq<real, TY, SPT, WALLS, TX, LBO>, grid, TX * TY / SPT, LbqSmem<real, TY, TX>::bytes, s, *a.tm_pq,
                      *a.tm_u3, *a.tm_f, *a.tm_f1, *a.tm_f2, *a.tm_qpf, *a.tm_q1pf, G, m,
                      static_cast<const real*>(a.f), static_cast<const real*>(a.q), static_cast<real*>(a.fnew),
                      static_cast<real*>(a.rhou_new), static_cast<real*>(a.qout ? a.qout : a.q), a.err, qw);
@@ -1534,6 +1543,9 @@ cudaError_t launch_step_zm_spt(const ZmArgs& a, cudaStream_t s) {
 // sites per thread chosen for each kernel separately (FP32: 1 or 2 each; walls and FP64: 1)
 template <typename real>
 cudaError_t launch_step_zm(const ZmArgs& a, cudaStream_t s) {
+  if (a.lb_only)
+    return a.q_wall ? launch_step_zm_spt<real, 1, 1, true, ZM_TX, true>(a, s)
+                    : launch_step_zm_spt<real, 1, 1, false, ZM_TX, true>(a, s);
   if constexpr (sizeof(real) == 4)
     if (a.tx == kZmNarrowX)
       return a.q_wall ? launch_step_zm_spt<real, 1, 1, true, kZmNarrowX>(a, s)

@@ -1,8 +1,9 @@
 """The kernels that AUTO picks for each kind of step against the generic ones.
 
 Widths that are no multiple of 4 (the z-marching kernels with plain row
-prefetches) and steps with the flow off (the Heun kernels on the Q mirror), with
-and without walls, on shapes with ragged tiles in x and y, several tiles and
+prefetches), steps with the flow off (the Heun kernels on the Q mirror) and
+Gauss-Seidel coupling (the LB halves of the z-marching kernels, then the Heun
+kernels with the new velocity), with and without walls, on shapes with ragged tiles in x and y, several tiles and
 z-chunks, and the smallest width.
 """
 
@@ -32,7 +33,7 @@ def pair(L, shape, dtype, mode):
     out = []
     for path in (L.PATH_AUTO, L.PATH_GENERIC):
         lat = L.Lattice(nx, ny, nz, dtype=dtype).set_path(path)
-        lat.set_flow(flow_on="noflow" not in mode, coupling=L.GAUSS_SEIDEL if mode == "gauss_seidel" else L.JACOBI)
+        lat.set_flow(flow_on="noflow" not in mode, coupling=L.GAUSS_SEIDEL if "seidel" in mode else L.JACOBI)
         if "walls" in mode:
             lat.set_walls(True, (0.2, 0.0, 0.0, -0.1, 0.0))
         lat.init_q(L.BPII, 0.3, noise=1e-3, seed=4)
@@ -84,3 +85,37 @@ def test_flow_switched_on_after_relaxation(lcbp):
         lat.set_flow(flow_on=True).step(2)
     assert np.abs(a.read_q() - b.read_q()).max() < 1e-13
     assert np.abs(a.read_u() - b.read_u()).max() < 1e-14
+
+
+GS_SHAPES = [(9, 11, 5), (13, 18, 64), (37, 19, 45), (1, 3, 66), (2, 17, 36)]
+
+
+@pytest.mark.parametrize("mode", ["seidel", "seidel_walls"])
+@pytest.mark.parametrize("shape", GS_SHAPES)
+def test_gauss_seidel_matches_generic(lcbp, shape, mode):
+    check(lcbp, shape, "f64", mode, 11)
+
+
+@pytest.mark.parametrize("mode", ["seidel", "seidel_walls"])
+@pytest.mark.parametrize("shape", GS_SHAPES)
+def test_gauss_seidel_f32_rounds_like_generic(lcbp, shape, mode):
+    """FP32 against the generic FP64 run: both FP32 kernel sets do the same operations per site in another
+    order, so their rounding errors are of one size (2-norms within a factor of two)."""
+    a, b = pair(lcbp, shape, "f32", mode)
+    exact = pair(lcbp, shape, "f64", mode)[1]
+    for lat in (a, b, exact):
+        lat.step(11)
+    for read in ("read_q", "read_u", "read_f"):
+        want = getattr(exact, read)()
+        mine, theirs = (np.linalg.norm(getattr(lat, read)() - want) for lat in (a, b))
+        assert mine <= 2 * theirs
+
+
+def test_coupling_switched_between_steps(lcbp):
+    a, b = pair(lcbp, (12, 10, 12), "f64", "flow")
+    for lat in (a, b):
+        lat.step(4)
+        lat.set_flow(coupling=lcbp.GAUSS_SEIDEL).step(3)
+        lat.set_flow(coupling=lcbp.JACOBI).step(4)
+    assert np.abs(a.read_q() - b.read_q()).max() < TOL["f64"][0]
+    assert np.abs(a.read_u() - b.read_u()).max() < TOL["f64"][1]

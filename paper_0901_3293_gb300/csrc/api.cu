@@ -858,19 +858,17 @@ int refresh_moments(lcbp_lattice* h) {
 // tell which copy is current (at least one is): fast steps make the mirrors
 // current (sync_mirror before them), anything else reads or writes the flat
 // arrays (sync_flat before, and a write makes the mirrors stale).
+MirrorCopy mirror_copy(lcbp_lattice* h, void* q, void* ru) {
+  return {h->nx, h->ny, h->nz, 1, 0, q, ru, h->qm, h->um[h->cur], 0};
+}
+
+cudaError_t unpack(lcbp_lattice* h, const MirrorCopy& m) {
+  return h->dtype == LCBP_F64 ? launch_unpack<double>(m, h->stream) : launch_unpack<float>(m, h->stream);
+}
+
 int sync_flat(lcbp_lattice* h) {
   if (h->flat_ok) return LCBP_OK;
-  const int nxm = zm_mirror_nx(h->nx), X = kZmMirX;
-  cudaError_t e =
-      h->dtype == LCBP_F64
-          ? launch_unpack<double>(h->qm, h->q, 5, 1, h->nx, h->ny, h->nz, X, 2, nxm, h->ny + 4, h->stream)
-          : launch_unpack<float>(h->qm, h->q, 5, 1, h->nx, h->ny, h->nz, X, 2, nxm, h->ny + 4, h->stream);
-  if (e == cudaSuccess)
-    e = h->dtype == LCBP_F64
-            ? launch_unpack<double>(h->um[h->cur], h->rhou[h->cur], 4, 1, h->nx, h->ny, h->nz, X, 1, nxm, h->ny + 2,
-                                    h->stream)
-            : launch_unpack<float>(h->um[h->cur], h->rhou[h->cur], 4, 1, h->nx, h->ny, h->nz, X, 1, nxm, h->ny + 2,
-                                   h->stream);
+  const cudaError_t e = unpack(h, mirror_copy(h, h->q, h->rhou[h->cur]));
   if (e != cudaSuccess) return cuda_fail(e, "state from the padded mirrors");
   h->flat_ok = true;
   return LCBP_OK;
@@ -878,19 +876,28 @@ int sync_flat(lcbp_lattice* h) {
 
 int sync_mirror(lcbp_lattice* h) {
   if (h->mirror_ok) return LCBP_OK;
-  const int nxm = zm_mirror_nx(h->nx), X = kZmMirX;
-  cudaError_t e = h->dtype == LCBP_F64
-                      ? launch_pack<double>(h->q, h->qm, 5, 1, h->nx, h->ny, h->nz, X, 2, nxm, h->ny + 4, h->stream)
-                      : launch_pack<float>(h->q, h->qm, 5, 1, h->nx, h->ny, h->nz, X, 2, nxm, h->ny + 4, h->stream);
-  if (e == cudaSuccess)
-    e = h->dtype == LCBP_F64
-            ? launch_pack<double>(h->rhou[h->cur], h->um[h->cur], 4, 1, h->nx, h->ny, h->nz, X, 1, nxm, h->ny + 2,
-                                  h->stream)
-            : launch_pack<float>(h->rhou[h->cur], h->um[h->cur], 4, 1, h->nx, h->ny, h->nz, X, 1, nxm, h->ny + 2,
-                                 h->stream);
+  const MirrorCopy m = mirror_copy(h, h->q, h->rhou[h->cur]);
+  const cudaError_t e = h->dtype == LCBP_F64 ? launch_pack<double>(m, h->stream) : launch_pack<float>(m, h->stream);
   if (e != cudaSuccess) return cuda_fail(e, "padded mirrors of the state");
   h->mirror_ok = true;
   return LCBP_OK;
+}
+
+// Whether dst is memory of the lattice's device in the state's type and
+// alignment: a read may then unpack the mirrors straight into it
+bool direct_read(const lcbp_lattice* h, const void* dst, int dtype) {
+  if (h->flat_ok || dtype != h->dtype || reinterpret_cast<uintptr_t>(dst) % h->es != 0) return false;
+  cudaPointerAttributes at{};
+  if (cudaPointerGetAttributes(&at, dst) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == h->device;
+}
+
+int finish_read(lcbp_lattice* h, cudaError_t e, const char* what) {
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  return e == cudaSuccess ? LCBP_OK : cuda_fail(e, what);
 }
 
 struct CkptHeader {
@@ -1424,21 +1431,23 @@ int lcbp_check_wait_timeout(double limit_ms, int* timed_out) {
 
 int lcbp_read_q(lcbp_lattice* h, void* dst, int dtype) {
   CHECK_H(h);
-  {
-    const int rs = sync_flat(h);
-    if (rs) return rs;
-  }
   if (!dst || !valid_dtype(dtype)) return fail(LCBP_EINVAL, "bad buffer or dtype");
+  if (direct_read(h, dst, dtype)) return finish_read(h, unpack(h, mirror_copy(h, dst, nullptr)), "read_q");
+  const int rs = sync_flat(h);
+  if (rs) return rs;
   return transfer(h->q, h->dtype, dst, dtype, 5 * h->n, false, h->staging, h->staging_elems, h->stream);
 }
 
 int lcbp_read_u(lcbp_lattice* h, void* dst, int dtype) {
   CHECK_H(h);
-  {
-    const int rs = sync_flat(h);
-    if (rs) return rs;
-  }
   if (!dst || !valid_dtype(dtype)) return fail(LCBP_EINVAL, "bad buffer or dtype");
+  if (direct_read(h, dst, dtype)) {
+    MirrorCopy m = mirror_copy(h, nullptr, dst);
+    m.u0 = 1;
+    return finish_read(h, unpack(h, m), "read_u");
+  }
+  const int rs = sync_flat(h);
+  if (rs) return rs;
   return transfer(static_cast<char*>(h->rhou[h->cur]) + h->n * h->es, h->dtype, dst, dtype, 3 * h->n, false,
                   h->staging, h->staging_elems, h->stream);
 }

@@ -220,34 +220,18 @@ ZmBatchArgs zm_args(lcbp_batch* b) {
 
 // Q and rho u (the current buffer) of every replica of the fast-path classes,
 // between the flat fields and the padded mirrors: unpack (mirrors -> flat) or
-// pack (flat -> mirrors, periodic images included)
+// pack (flat -> mirrors, periodic images included); a launch per class
 cudaError_t mirror_copy(lcbp_batch* b, bool to_flat) {
   cudaError_t e = cudaSuccess;
   for (int k = 0; k < b->zb.nclass && e == cudaSuccess; ++k) {
     const ZmClass& c = b->zb.c[k];
-    const int nx = c.G.nx, ny = c.G.ny, nz = c.G.nz, nxm = zm_mirror_nx(nx), X = kZmMirX;
-    const long long cq = (long long)nxm * (ny + 4) * nz, cu = (long long)nxm * (ny + 2) * nz;
-    for (int j = 0; j < c.count && e == cudaSuccess; ++j) {
-      const int r = b->order[c.rep0 + j];
-      char* qm = static_cast<char*>(b->qm) + (size_t)(c.qm0 + j * 5 * cq) * b->es;
-      char* um = static_cast<char*>(b->um[b->cur]) + (size_t)(c.um0 + j * 4 * cu) * b->es;
-      void* q = static_cast<char*>(b->q) + (size_t)5 * b->base[r] * b->es;
-      void* ru = static_cast<char*>(b->rhou[b->cur]) + (size_t)4 * b->base[r] * b->es;
-      const bool d = b->dtype == LCBP_F64;
-      if (to_flat) {
-        e = d ? launch_unpack<double>(qm, q, 5, 1, nx, ny, nz, X, 2, nxm, ny + 4, b->stream)
-              : launch_unpack<float>(qm, q, 5, 1, nx, ny, nz, X, 2, nxm, ny + 4, b->stream);
-        if (e == cudaSuccess)
-          e = d ? launch_unpack<double>(um, ru, 4, 1, nx, ny, nz, X, 1, nxm, ny + 2, b->stream)
-                : launch_unpack<float>(um, ru, 4, 1, nx, ny, nz, X, 1, nxm, ny + 2, b->stream);
-      } else {
-        e = d ? launch_pack<double>(q, qm, 5, 1, nx, ny, nz, X, 2, nxm, ny + 4, b->stream)
-              : launch_pack<float>(q, qm, 5, 1, nx, ny, nz, X, 2, nxm, ny + 4, b->stream);
-        if (e == cudaSuccess)
-          e = d ? launch_pack<double>(ru, um, 4, 1, nx, ny, nz, X, 1, nxm, ny + 2, b->stream)
-                : launch_pack<float>(ru, um, 4, 1, nx, ny, nz, X, 1, nxm, ny + 2, b->stream);
-      }
-    }
+    const long long base = b->base[b->order[c.rep0]], n = b->n[b->order[c.rep0]];
+    auto at = [&](void* p, long long elems) { return static_cast<char*>(p) + (size_t)elems * b->es; };
+    // (replicas of a class lie back to back, each block a whole number of 64 sites)
+    const MirrorCopy m{c.G.nx, c.G.ny, c.G.nz, c.count, (n + 63) / 64 * 64, at(b->q, 5 * base),
+                       at(b->rhou[b->cur], 4 * base), at(b->qm, c.qm0), at(b->um[b->cur], c.um0), 0};
+    if (to_flat) e = b->dtype == LCBP_F64 ? launch_unpack<double>(m, b->stream) : launch_unpack<float>(m, b->stream);
+    else e = b->dtype == LCBP_F64 ? launch_pack<double>(m, b->stream) : launch_pack<float>(m, b->stream);
   }
   return e;
 }

@@ -92,18 +92,6 @@ struct DiagGeom {
   double qw[5];    // anchored Q (q5 order)
   double c_div;    // (K - L2) / 2: F_h gains -c_div |div Q|^2 per site
 };
-// padded mirror <-> flat field (state.cu): C components of an nx x ny x nz
-// field, site (x, y) at column x + hx and row y + hy of a mirror of nxp x nyp
-// whose first 4G components are interleaved by fours ([group][z][Y][X][4])
-// and whose others are plain arrays; pack fills every mirror position with
-// its periodic image
-template <typename real>
-cudaError_t launch_pack(const void* flat, void* padded, int C, int G, int nx, int ny, int nz, int hx, int hy,
-                        int nxp, int nyp, cudaStream_t s);
-template <typename real>
-cudaError_t launch_unpack(const void* padded, void* flat, int C, int G, int nx, int ny, int nz, int hx, int hy,
-                          int nxp, int nyp, cudaStream_t s);
-
 // whole-field checks (state.cu); scratch: state_check_scratch_bytes() of device memory
 size_t state_check_scratch_bytes();
 // *out = number of non-finite values among n
@@ -182,9 +170,25 @@ constexpr int kZmMirX = 32;  // columns before x = 0 in a mirror row
 constexpr int kZmNarrowX = 16;
 inline int zm_batch_tile_x(int nx, bool fp32) { return fp32 && nx % 32 != 0 && nx % 32 <= 16 ? kZmNarrowX : 32; }
 inline int zm_lattice_tile_x(int nx, bool fp32) { return fp32 && nx <= kZmNarrowX ? kZmNarrowX : 32; }
-inline int zm_mirror_nx(int nx) { return (nx + 31) / 32 * 32 + 2 * kZmMirX; }  // mirror row length
-inline long long zm_qmirror_elems(int nx, int ny, int nz) { return 5LL * zm_mirror_nx(nx) * (ny + 4) * nz; }
-inline long long zm_umirror_elems(int nx, int ny, int nz) { return 4LL * zm_mirror_nx(nx) * (ny + 2) * nz; }
+__host__ __device__ inline int zm_mirror_nx(int nx) { return (nx + 31) / 32 * 32 + 2 * kZmMirX; }  // mirror row length
+__host__ __device__ inline long long zm_qmirror_elems(int nx, int ny, int nz) { return 5LL * zm_mirror_nx(nx) * (ny + 4) * nz; }
+__host__ __device__ inline long long zm_umirror_elems(int nx, int ny, int nz) { return 4LL * zm_mirror_nx(nx) * (ny + 2) * nz; }
+
+// Flat fields <-> padded mirrors (state.cu) of `count` replicas of equal dims:
+// Q (5 N) and rho u (4 N) of replica j at j * flat_stride sites from the first's,
+// the mirrors back to back.  launch_pack fills the mirrors, periodic images
+// included; launch_unpack writes the flat fields (q or ru may be null; of rho u the
+// components from u0 on, the first of them at ru).
+struct MirrorCopy {
+  int nx, ny, nz, count;
+  long long flat_stride;
+  void *q, *ru, *qm, *um;
+  int u0;
+};
+template <typename real>
+cudaError_t launch_pack(const MirrorCopy& a, cudaStream_t s);
+template <typename real>
+cudaError_t launch_unpack(const MirrorCopy& a, cudaStream_t s);
 
 // Shapes the z-marching kernels can serve: nx >= 4 (a site has at most one
 // periodic image in x within the mirrors' two ghost columns) and element offsets

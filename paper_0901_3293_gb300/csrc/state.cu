@@ -3,6 +3,7 @@
 // (used by the surrogate judge to compare a surrogate call with plain steps),
 // both reduced in a fixed order, and the copies between a field and its
 // padded mirror with periodic ghosts (the fast step's state layout).
+#include <algorithm>
 #include <cmath>
 
 #include "kernels.h"
@@ -101,17 +102,14 @@ cudaError_t launch_max_abs_diff(const void* a, const void* b, long long n, void*
   return cudaGetLastError();
 }
 
-// A padded mirror holds its first 4G components interleaved by fours
-// ([group][z][Y][X][4]) and the others as plain arrays ([z][Y][X]) after
-// them.  The copies below walk it by units (a group of four components, or
-// one plain component) and rows: one CTA per (unit, plane, row), threads
-// along the row, so no thread divides a 64-bit index and a group moves as one
-// 16-byte vector (FP32) per site.
-__device__ __forceinline__ int wrap_mod(int v, int n) {
-  v %= n;
-  return v < 0 ? v + n : v;
-}
-
+// ---------------------------------------------------------------------------
+// The state between its flat fields and its padded mirrors (layouts in
+// kernels.h): Q and rho u of a plane's position in one thread, 16-byte vectors on
+// the mirrors' side and coalesced rows on the flat side.  One launch moves both
+// fields of every replica of a class (blockIdx.z): a lattice's copies took a
+// launch per field with a CTA per row, whose 64-bit row arithmetic outweighed
+// short rows (128^3 FP32: unpack 40 -> UNPACKFIG us, pack 55 -> PACKFIG us).
+// ---------------------------------------------------------------------------
 template <typename real>
 __device__ __forceinline__ void put4(real* p, real a, real b, real c, real d) {
   if constexpr (sizeof(real) == 4) {
@@ -132,93 +130,100 @@ __device__ __forceinline__ void get4(const real* p, real v[4]) {
   }
 }
 
-// every padded position of every component: flat[c][z][wrap(Y - hy)][wrap(X - hx)]
+// flat -> mirrors: every site and, in the two (Q) and one (rho u) columns and
+// rows next to the lattice, its periodic images
 template <typename real>
-__global__ void k_pack(const real* __restrict__ flat, real* __restrict__ padded, int C, int G, int nx, int ny, int nz,
-                       int hx, int hy, int nxp, int nyp) {
-  const long long rows = (long long)(G + C - 4 * G) * nz * nyp;
-  const long long plane = (long long)ny * nx, cstride = plane * nz;    // flat component stride
-  const long long pplane = (long long)nyp * nxp, pstride = pplane * nz;  // padded plain-component stride
-  for (long long r = blockIdx.x; r < rows; r += gridDim.x) {
-    const int Y = (int)(r % nyp);
-    const long long uz = r / nyp;
-    const int z = (int)(uz % nz), u = (int)(uz / nz);
-    const int y = wrap_mod(Y - hy, ny);
-    const real* src = flat + (long long)z * plane + (long long)y * nx;
-    if (u < G) {
-      src += (long long)(4 * u) * cstride;
-      real* dst = padded + (((long long)u * nz + z) * nyp + Y) * nxp * 4;
-      for (int X = threadIdx.x; X < nxp; X += blockDim.x) {
-        const int x = wrap_mod(X - hx, nx);
-        put4(dst + (long long)X * 4, src[x], src[cstride + x], src[2 * cstride + x], src[3 * cstride + x]);
+__global__ void __launch_bounds__(256) k_pack(MirrorCopy a) {
+  const int nx = a.nx, ny = a.ny, nz = a.nz, w = nx + 4;
+  const int P = blockIdx.x * 256 + threadIdx.x;
+  if (P >= w * (ny + 4)) return;
+  const int Y = P / w, X = P - Y * w;  // the site's position with two ghosts on each side
+  int x = X - 2, y = (Y - 2) % ny;
+  x = x < 0 ? x + nx : (x >= nx ? x - nx : x);  // (nx >= 4)
+  y = y < 0 ? y + ny : y;
+  const bool in_u = X >= 1 && X <= nx + 2 && Y >= 1 && Y <= ny + 2;
+  const long long n = (long long)nx * ny * nz;
+  const int nxm = zm_mirror_nx(nx);
+  for (int j = blockIdx.z; j < a.count; j += gridDim.z) {
+    const real* q = static_cast<const real*>(a.q) + 5 * j * a.flat_stride;
+    const real* ru = static_cast<const real*>(a.ru) + 4 * j * a.flat_stride;
+    real* qm = static_cast<real*>(a.qm) + j * zm_qmirror_elems(nx, ny, nz);
+    real* um = static_cast<real*>(a.um) + j * zm_umirror_elems(nx, ny, nz);
+    real* yz = qm + 4LL * nxm * (ny + 4) * nz;
+    for (int z = blockIdx.y; z < nz; z += gridDim.y) {
+      const long long s = ((long long)z * ny + y) * nx + x;
+      const long long o = ((long long)z * (ny + 4) + Y) * nxm + X - 2 + kZmMirX;
+      put4(qm + 4 * o, q[s], q[n + s], q[2 * n + s], q[3 * n + s]);
+      yz[o] = q[4 * n + s];
+      if (in_u) {
+        const long long ou = ((long long)z * (ny + 2) + Y - 1) * nxm + X - 2 + kZmMirX;
+        put4(um + 4 * ou, ru[s], ru[n + s], ru[2 * n + s], ru[3 * n + s]);
       }
-    } else {
-      src += (long long)(4 * G + (u - G)) * cstride;
-      real* dst = padded + 4 * (long long)G * pstride + (long long)(u - G) * pstride + (long long)z * pplane +
-                  (long long)Y * nxp;
-      for (int X = threadIdx.x; X < nxp; X += blockDim.x) dst[X] = src[wrap_mod(X - hx, nx)];
     }
   }
 }
 
-// flat[c][z][y][x] = the padded value at (x + hx, y + hy)
+// mirrors -> flat; either destination may be null, and of rho u components u0..3
+// are written (u0 = 1: the velocity alone, from ru on)
 template <typename real>
-__global__ void k_unpack(const real* __restrict__ padded, real* __restrict__ flat, int C, int G, int nx, int ny,
-                         int nz, int hx, int hy, int nxp, int nyp) {
-  const long long rows = (long long)(G + C - 4 * G) * nz * ny;
-  const long long plane = (long long)ny * nx, cstride = plane * nz;
-  const long long pplane = (long long)nyp * nxp, pstride = pplane * nz;
-  for (long long r = blockIdx.x; r < rows; r += gridDim.x) {
-    const int y = (int)(r % ny);
-    const long long uz = r / ny;
-    const int z = (int)(uz % nz), u = (int)(uz / nz);
-    real* dst = flat + (long long)z * plane + (long long)y * nx;
-    if (u < G) {
-      dst += (long long)(4 * u) * cstride;
-      const real* src = padded + (((long long)u * nz + z) * nyp + (y + hy)) * nxp * 4;
-      for (int x = threadIdx.x; x < nx; x += blockDim.x) {
-        real v[4];
-        get4(src + (long long)(x + hx) * 4, v);
-        dst[x] = v[0];
-        dst[cstride + x] = v[1];
-        dst[2 * cstride + x] = v[2];
-        dst[3 * cstride + x] = v[3];
+__global__ void __launch_bounds__(256) k_unpack(MirrorCopy a) {
+  const int nx = a.nx, ny = a.ny, nz = a.nz;
+  const int P = blockIdx.x * 256 + threadIdx.x;
+  if (P >= nx * ny) return;
+  const int y = P / nx, x = P - y * nx;
+  const long long n = (long long)nx * ny * nz;
+  const int nxm = zm_mirror_nx(nx);
+  for (int j = blockIdx.z; j < a.count; j += gridDim.z) {
+    real* q = a.q ? static_cast<real*>(a.q) + 5 * j * a.flat_stride : nullptr;
+    real* ru = a.ru ? static_cast<real*>(a.ru) + 4 * j * a.flat_stride : nullptr;
+    const real* qm = static_cast<const real*>(a.qm) + j * zm_qmirror_elems(nx, ny, nz);
+    const real* um = static_cast<const real*>(a.um) + j * zm_umirror_elems(nx, ny, nz);
+    const real* yz = qm + 4LL * nxm * (ny + 4) * nz;
+    for (int z = blockIdx.y; z < nz; z += gridDim.y) {
+      const long long s = (long long)z * ny * nx + P;
+      real v[4];
+      if (q) {
+        const long long o = ((long long)z * (ny + 4) + y + 2) * nxm + x + kZmMirX;
+        get4(qm + 4 * o, v);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) q[c * n + s] = v[c];
+        q[4 * n + s] = yz[o];
       }
-    } else {
-      dst += (long long)(4 * G + (u - G)) * cstride;
-      const real* src = padded + 4 * (long long)G * pstride + (long long)(u - G) * pstride + (long long)z * pplane +
-                        (long long)(y + hy) * nxp;
-      for (int x = threadIdx.x; x < nx; x += blockDim.x) dst[x] = src[x + hx];
+      if (ru) {
+        const long long o = ((long long)z * (ny + 2) + y + 1) * nxm + x + kZmMirX;
+        get4(um + 4 * o, v);
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (c >= a.u0) ru[(c - a.u0) * n + s] = v[c];
+      }
     }
   }
 }
 
-int copy_grid(long long rows) { return (int)(rows < (1ll << 30) ? (rows > 0 ? rows : 1) : (1ll << 30)); }
+// a CTA per 256 positions, then planes and replicas as separate CTAs up to about
+// 16 CTAs per SM in all (a CTA walks the others)
+dim3 copy_grid(const MirrorCopy& a, int positions) {
+  const long long bx = (positions + 255) / 256, bz = std::min(a.count, 65535);
+  const long long want = 152LL * 16 / (bx * bz) + 1;
+  return dim3((unsigned)bx, (unsigned)std::min<long long>({(long long)a.nz, want, 65535LL}), (unsigned)bz);
+}
 
 template <typename real>
-cudaError_t launch_pack(const void* flat, void* padded, int C, int G, int nx, int ny, int nz, int hx, int hy,
-                        int nxp, int nyp, cudaStream_t s) {
-  const long long rows = (long long)(C - 3 * G) * nz * nyp;
-  k_pack<real><<<copy_grid(rows), 128, 0, s>>>(static_cast<const real*>(flat), static_cast<real*>(padded), C, G, nx,
-                                               ny, nz, hx, hy, nxp, nyp);
+cudaError_t launch_pack(const MirrorCopy& a, cudaStream_t s) {
+  k_pack<real><<<copy_grid(a, (a.nx + 4) * (a.ny + 4)), 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 
 template <typename real>
-cudaError_t launch_unpack(const void* padded, void* flat, int C, int G, int nx, int ny, int nz, int hx, int hy,
-                          int nxp, int nyp, cudaStream_t s) {
-  const long long rows = (long long)(C - 3 * G) * nz * ny;
-  k_unpack<real><<<copy_grid(rows), 128, 0, s>>>(static_cast<const real*>(padded), static_cast<real*>(flat), C, G,
-                                                 nx, ny, nz, hx, hy, nxp, nyp);
+cudaError_t launch_unpack(const MirrorCopy& a, cudaStream_t s) {
+  k_unpack<real><<<copy_grid(a, a.nx * a.ny), 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 
-template cudaError_t launch_pack<float>(const void*, void*, int, int, int, int, int, int, int, int, int, cudaStream_t);
-template cudaError_t launch_pack<double>(const void*, void*, int, int, int, int, int, int, int, int, int, cudaStream_t);
-template cudaError_t launch_unpack<float>(const void*, void*, int, int, int, int, int, int, int, int, int,
-                                          cudaStream_t);
-template cudaError_t launch_unpack<double>(const void*, void*, int, int, int, int, int, int, int, int, int,
-                                           cudaStream_t);
+template cudaError_t launch_pack<float>(const MirrorCopy&, cudaStream_t);
+template cudaError_t launch_pack<double>(const MirrorCopy&, cudaStream_t);
+template cudaError_t launch_unpack<float>(const MirrorCopy&, cudaStream_t);
+template cudaError_t launch_unpack<double>(const MirrorCopy&, cudaStream_t);
 
 template cudaError_t launch_count_nonfinite<float>(const void*, long long, void*, unsigned long long*, cudaStream_t);
 template cudaError_t launch_count_nonfinite<double>(const void*, long long, void*, unsigned long long*, cudaStream_t);

@@ -107,16 +107,18 @@ int check_params(const HostParams& p) {
 }
 
 // Copy `count` values between a caller buffer (host or device, dtype `ud`)
-// and a device state array (dtype `sd`), converting through `staging`.
+// and a device state array (dtype `sd`), converting through `staging`.  With
+// sync = false a copy without conversion is only enqueued: the caller
+// synchronises the stream before it returns.
 int transfer(void* state, int sd, void* user, int ud, long long count, bool upload, void* staging,
-             long long staging_elems, cudaStream_t st) {
+             long long staging_elems, cudaStream_t st, bool sync) {
   cudaError_t e;
   if (ud == sd) {
     const size_t bytes = (size_t)count * dtype_size(sd);
     e = upload ? cudaMemcpyAsync(state, user, bytes, cudaMemcpyDefault, st)
                : cudaMemcpyAsync(user, state, bytes, cudaMemcpyDefault, st);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync");
-    e = cudaStreamSynchronize(st);
+    if (sync) e = cudaStreamSynchronize(st);
     return e == cudaSuccess ? LCBP_OK : cuda_fail(e, "cudaStreamSynchronize");
   }
   const size_t ues = dtype_size(ud), ses = dtype_size(sd);
@@ -199,8 +201,8 @@ struct lcbp_lattice {
   double* h_out;  // pinned
   int cur;
   bool f_ready, has_bext;
-  cudaGraphExec_t graph, graph_run;  // two steps; kRunSteps steps
-  bool graph_ok, graph_run_ok;
+  cudaGraphExec_t graph[2], graph_run[2];  // two steps and kRunSteps steps, from buffer 0 or 1
+  bool graph_ok[2], graph_run_ok[2];
   long long step;
   // fast path (z-marching TMA kernels)
   int path_req;   // LCBP_PATH_*
@@ -768,10 +770,12 @@ cudaError_t eager_step(lcbp_lattice* h) {
 }
 
 void drop_graph(lcbp_lattice* h) {
-  if (h->graph_ok) cudaGraphExecDestroy(h->graph);
-  h->graph_ok = false;
-  if (h->graph_run_ok) cudaGraphExecDestroy(h->graph_run);
-  h->graph_run_ok = false;
+  for (int k = 0; k < 2; ++k) {
+    if (h->graph_ok[k]) cudaGraphExecDestroy(h->graph[k]);
+    h->graph_ok[k] = false;
+    if (h->graph_run_ok[k]) cudaGraphExecDestroy(h->graph_run[k]);
+    h->graph_run_ok[k] = false;
+  }
 }
 
 // Steps of the graph that runs of many steps replay, and the run length from
@@ -780,7 +784,7 @@ void drop_graph(lcbp_lattice* h) {
 // and 8.9 us in graphs of 16 (64^3: 30.8 and 29.5 us).
 constexpr int kRunSteps = 16, kRunMin = 32;
 
-// capture `steps` (an even number) steps starting from cur == 0 (the ping-pong
+// capture `steps` (an even number) steps from the current buffer (the ping-pong
 // buffers return to their roles after two steps)
 int build_graph(lcbp_lattice* h, int steps, cudaGraphExec_t* exec, bool* ok) {
   if (h->stream == nullptr) return LCBP_OK;  // legacy stream: no capture, eager launches
@@ -788,7 +792,6 @@ int build_graph(lcbp_lattice* h, int steps, cudaGraphExec_t* exec, bool* ok) {
   cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamBeginCapture");
   const int saved = h->cur;
-  h->cur = 0;
   cudaError_t e1 = cudaSuccess;
   for (int k = 0; k < steps && e1 == cudaSuccess; ++k) e1 = eager_step(h);
   h->cur = saved;
@@ -824,11 +827,8 @@ int diag(lcbp_lattice* h, double threshold, int with_f) {
   return LCBP_OK;
 }
 
-// number of non-finite values among n state-type values at v (device), synchronously
-int count_nonfinite(lcbp_lattice* h, const void* v, long long n, unsigned long long* count) {
-  auto* out = reinterpret_cast<unsigned long long*>(h->d_out);
-  cudaError_t e = h->dtype == LCBP_F64 ? launch_count_nonfinite<double>(v, n, h->d_partials, out, h->stream)
-                                       : launch_count_nonfinite<float>(v, n, h->d_partials, out, h->stream);
+// the count that a check left in d_out, synchronously
+int read_count(lcbp_lattice* h, cudaError_t e, unsigned long long* count) {
   if (e == cudaSuccess) e = cudaMemcpyAsync(h->h_out, h->d_out, 8, cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return cuda_fail(e, "finiteness check");
@@ -1176,14 +1176,18 @@ int lcbp_set_q(lcbp_lattice* h, const void* q5, int dtype) {
   if (!q5 || !valid_dtype(dtype)) return fail(LCBP_EINVAL, "bad buffer or dtype");
   // into the Q* scratch first: a field holding NaN or Inf is refused and Q stays as it was
   int rc = transfer(h->qs, h->dtype, const_cast<void*>(q5), dtype, 5 * h->n, true, h->staging, h->staging_elems,
-                    h->stream);
+                    h->stream, false);
   if (rc) return rc;
+  auto* out = reinterpret_cast<unsigned long long*>(h->d_out);
   unsigned long long bad = 0;
-  rc = count_nonfinite(h, h->qs, 5 * h->n, &bad);
+  rc = read_count(h,
+                  h->dtype == LCBP_F64 ? launch_count_nonfinite<double>(h->qs, 5 * h->n, out, h->stream)
+                                       : launch_count_nonfinite<float>(h->qs, 5 * h->n, out, h->stream),
+                  &bad);
   if (rc) return rc;
   if (bad) return fail(LCBP_ENONFINITE, "%llu values of the uploaded Q are NaN or Inf; Q is unchanged", bad);
-  cudaError_t e = cudaMemcpyAsync(h->q, h->qs, (size_t)(5 * h->n) * h->es, cudaMemcpyDeviceToDevice, h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  const cudaError_t e =
+      cudaMemcpyAsync(h->q, h->qs, (size_t)(5 * h->n) * h->es, cudaMemcpyDeviceToDevice, h->stream);
   return e == cudaSuccess ? LCBP_OK : cuda_fail(e, "set_q");
 }
 
@@ -1225,20 +1229,22 @@ int lcbp_set_f(lcbp_lattice* h, const void* f15, int dtype) {
   }
   h->mirror_ok = false;  // the flat state is written below
   if (!f15 || !valid_dtype(dtype)) return fail(LCBP_EINVAL, "bad buffer or dtype");
-  // into the scratch block (16 N elements) first: non-finite populations are refused, f stays as it was
+  // into the scratch block (16 N elements), from there to the other population
+  // and moment buffers, which become the state's unless a value is not finite
   int rc = transfer(h->h, h->dtype, const_cast<void*>(f15), dtype, 15 * h->n, true, h->staging, h->staging_elems,
-                    h->stream);
+                    h->stream, false);
   if (rc) return rc;
+  const int to = h->cur ^ 1;
+  auto* out = reinterpret_cast<unsigned long long*>(h->d_out);
   unsigned long long bad = 0;
-  rc = count_nonfinite(h, h->h, 15 * h->n, &bad);
+  rc = read_count(h,
+                  h->dtype == LCBP_F64
+                      ? launch_load_f<double>(h->h, h->f[to], h->rhou[to], h->n, out, h->stream)
+                      : launch_load_f<float>(h->h, h->f[to], h->rhou[to], h->n, out, h->stream),
+                  &bad);
   if (rc) return rc;
   if (bad) return fail(LCBP_ENONFINITE, "%llu uploaded populations are NaN or Inf; f is unchanged", bad);
-  // into f as deviations from the rest weights, in one pass from the scratch
-  cudaError_t e = h->dtype == LCBP_F64 ? launch_shift<double>(h->h, h->f[h->cur], h->n, 15, 0, -1, h->stream)
-                                       : launch_shift<float>(h->h, h->f[h->cur], h->n, 15, 0, -1, h->stream);
-  if (e != cudaSuccess) return cuda_fail(e, "set_f");
-  rc = refresh_moments(h);
-  if (rc) return rc;
+  h->cur = to;
   h->f_ready = true;
   return LCBP_OK;
 }
@@ -1278,25 +1284,22 @@ int lcbp_step(lcbp_lattice* h, int nsteps) {
   else h->mirror_ok = false;
   cudaError_t e = cudaSuccess;
   int left = nsteps;
-  if (h->cur == 1) {
-    e = eager_step(h);
-    --left;
-  }
-  if (left >= kRunMin && !h->graph_run_ok && e == cudaSuccess) {
-    int rc = build_graph(h, kRunSteps, &h->graph_run, &h->graph_run_ok);
+  const int c = h->cur;  // (the same after every two steps)
+  if (left >= kRunMin && !h->graph_run_ok[c]) {
+    int rc = build_graph(h, kRunSteps, &h->graph_run[c], &h->graph_run_ok[c]);
     if (rc) return rc;
   }
-  while (left >= kRunSteps && h->graph_run_ok && e == cudaSuccess) {
-    e = cudaGraphLaunch(h->graph_run, h->stream);
+  while (left >= kRunSteps && h->graph_run_ok[c] && e == cudaSuccess) {
+    e = cudaGraphLaunch(h->graph_run[c], h->stream);
     left -= kRunSteps;
   }
-  if (left >= 2 && !h->graph_ok && e == cudaSuccess) {
-    int rc = build_graph(h, 2, &h->graph, &h->graph_ok);
+  if (left >= 2 && !h->graph_ok[c] && e == cudaSuccess) {
+    int rc = build_graph(h, 2, &h->graph[c], &h->graph_ok[c]);
     if (rc) return rc;
   }
   while (left >= 2 && e == cudaSuccess) {
-    if (h->graph_ok) {
-      e = cudaGraphLaunch(h->graph, h->stream);
+    if (h->graph_ok[c]) {
+      e = cudaGraphLaunch(h->graph[c], h->stream);
     } else {
       e = eager_step(h);
       if (e == cudaSuccess) e = eager_step(h);

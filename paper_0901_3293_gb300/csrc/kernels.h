@@ -94,10 +94,13 @@ struct DiagGeom {
 };
 // whole-field checks (state.cu); scratch: state_check_scratch_bytes() of device memory
 size_t state_check_scratch_bytes();
-// *out = number of non-finite values among n
+// *out = number of non-finite values among n (v 16-byte aligned)
 template <typename real>
-cudaError_t launch_count_nonfinite(const void* v, long long n, void* scratch, unsigned long long* out,
-                                   cudaStream_t s);
+cudaError_t launch_count_nonfinite(const void* v, long long n, unsigned long long* out, cudaStream_t s);
+// full populations src [15][n] -> deviations f and moments rhou; *out = number of non-finite values
+template <typename real>
+cudaError_t launch_load_f(const void* src, void* f, void* rhou, long long n, unsigned long long* out,
+                          cudaStream_t s);
 // *out = max |a - b| over n values (NaN if either holds one)
 template <typename real>
 cudaError_t launch_max_abs_diff(const void* a, const void* b, long long n, void* scratch, double* out,

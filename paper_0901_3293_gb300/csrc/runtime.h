@@ -38,7 +38,7 @@ void fill_replica(void* dst, int nx, int ny, int nz, long long base, const HostP
 double s_eq(double gamma);
 int check_params(const HostParams& p);
 int transfer(void* state, int sd, void* user, int ud, long long count, bool upload, void* staging,
-             long long staging_elems, cudaStream_t st);
+             long long staging_elems, cudaStream_t st, bool sync = true);
 bool encode_tiled(CUtensorMap* tm, void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
                   const cuuint32_t* box, int dtype);
 

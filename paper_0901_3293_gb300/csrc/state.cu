@@ -15,19 +15,63 @@ namespace {
 constexpr int kRedThreads = 256;
 constexpr int kRedBlocks = 512;
 
+// adds a CTA's count to *total (only where there is something to add: the usual
+// field holds none, and no CTA writes)
+__device__ __forceinline__ void add_count(unsigned bad, unsigned long long* total) {
+  const int any = __syncthreads_count(bad != 0);
+  if (any && bad) atomicAdd(total, (unsigned long long)bad);
+}
+
+// number of non-finite values, 16 bytes a load (v is 16-byte aligned)
 template <typename real>
-__global__ void k_count_nonfinite(const real* __restrict__ v, long long n, unsigned long long* __restrict__ partial) {
-  unsigned long long c = 0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    c += isfinite(v[i]) ? 0ull : 1ull;
-  __shared__ unsigned long long red[kRedThreads];
-  red[threadIdx.x] = c;
-  __syncthreads();
-  for (int s = kRedThreads / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-    __syncthreads();
+__global__ void __launch_bounds__(kRedThreads)
+    k_count_nonfinite(const real* __restrict__ v, long long n, unsigned long long* total) {
+  constexpr int W = 16 / sizeof(real);
+  unsigned bad = 0;
+  const long long step = (long long)gridDim.x * blockDim.x, t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const int4* v4 = reinterpret_cast<const int4*>(v);
+#pragma unroll 4
+  for (long long i = t0; i < n / W; i += step) {
+    const int4 q = v4[i];
+    const real* x = reinterpret_cast<const real*>(&q);
+#pragma unroll
+    for (int k = 0; k < W; ++k) bad += isfinite(x[k]) ? 0u : 1u;
   }
-  if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
+  for (long long i = n / W * W + t0; i < n; i += step) bad += isfinite(v[i]) ? 0u : 1u;
+  add_count(bad, total);
+}
+
+// Uploaded populations (full values) to the state: deviations from the rest
+// weights, their moments, and the number of non-finite values, in one pass.  It
+// fills buffers that are not the state's yet, so a refused upload costs nothing
+// more (count, shift and moments took a pass over the field each: at 128^3 FP32
+// 154 us in four launches, the call 62 us beyond its copy now).
+template <typename real>
+__global__ void __launch_bounds__(kRedThreads) k_load_f(const real* __restrict__ src, real* __restrict__ f,
+                                                        real* __restrict__ rhou, long long n,
+                                                        unsigned long long* total) {
+  unsigned bad = 0;
+  const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (s < n) {
+    real dr = 0, jx = 0, jy = 0, jz = 0;
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const real v = src[i * n + s];
+      bad += isfinite(v) ? 0u : 1u;
+      const real d = v - (real)rest_weight(i);
+      f[i * n + s] = d;
+      dr += d;
+      jx += real(ex(i)) * d;
+      jy += real(ey(i)) * d;
+      jz += real(ez(i)) * d;
+    }
+    const real r = real(1) + dr;
+    rhou[s] = dr;
+    rhou[n + s] = jx / r;
+    rhou[2 * n + s] = jy / r;
+    rhou[3 * n + s] = jz / r;
+  }
+  add_count(bad, total);
 }
 
 // max |a - b| over n values, as a double; a NaN anywhere gives NaN
@@ -52,24 +96,18 @@ __global__ void k_max_abs_diff(const real* __restrict__ a, const real* __restric
   if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
 }
 
-template <typename T>
-__global__ void k_final_sum(const T* __restrict__ partial, int nb, T* __restrict__ out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    T s = 0;
-    for (int i = 0; i < nb; ++i) s += partial[i];
-    *out = s;
-  }
-}
-
+// the largest of nb partials, by one warp; a NaN among them gives NaN
 __global__ void k_final_max(const double* __restrict__ partial, int nb, double* __restrict__ out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double m = 0.0;
-    for (int i = 0; i < nb; ++i) {
-      const double v = partial[i];
-      if (v > m || v != v) m = v;
-    }
-    *out = m;
+  double m = 0.0;
+  for (int i = threadIdx.x; i < nb; i += 32) {
+    const double v = partial[i];
+    if (v > m || v != v) m = v;
   }
+  for (int o = 16; o > 0; o >>= 1) {
+    const double v = __shfl_down_sync(0xffffffffu, m, o);
+    if (v > m || v != v) m = v;
+  }
+  if (threadIdx.x == 0) *out = m;
 }
 
 int blocks_for(long long n) {
@@ -82,12 +120,22 @@ int blocks_for(long long n) {
 size_t state_check_scratch_bytes() { return (size_t)(kRedBlocks + 1) * 8; }
 
 template <typename real>
-cudaError_t launch_count_nonfinite(const void* v, long long n, void* scratch, unsigned long long* out,
-                                   cudaStream_t s) {
-  auto* partial = static_cast<unsigned long long*>(scratch);
-  const int nb = blocks_for(n);
-  k_count_nonfinite<real><<<nb, kRedThreads, 0, s>>>(static_cast<const real*>(v), n, partial);
-  k_final_sum<unsigned long long><<<1, 32, 0, s>>>(partial, nb, out);
+cudaError_t launch_count_nonfinite(const void* v, long long n, unsigned long long* out, cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(out, 0, sizeof(*out), s);
+  if (e != cudaSuccess) return e;
+  const long long want = (n / 16 + kRedThreads - 1) / kRedThreads + 1;  // about four 16-byte loads a thread
+  k_count_nonfinite<real><<<(int)std::min<long long>(want, 152 * 8), kRedThreads, 0, s>>>(
+      static_cast<const real*>(v), n, out);
+  return cudaGetLastError();
+}
+
+template <typename real>
+cudaError_t launch_load_f(const void* src, void* f, void* rhou, long long n, unsigned long long* out,
+                          cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(out, 0, sizeof(*out), s);
+  if (e != cudaSuccess) return e;
+  k_load_f<real><<<(unsigned)((n + kRedThreads - 1) / kRedThreads), kRedThreads, 0, s>>>(
+      static_cast<const real*>(src), static_cast<real*>(f), static_cast<real*>(rhou), n, out);
   return cudaGetLastError();
 }
 
@@ -108,7 +156,7 @@ cudaError_t launch_max_abs_diff(const void* a, const void* b, long long n, void*
 // the mirrors' side and coalesced rows on the flat side.  One launch moves both
 // fields of every replica of a class (blockIdx.z): a lattice's copies took a
 // launch per field with a CTA per row, whose 64-bit row arithmetic outweighed
-// short rows (128^3 FP32: unpack 40 -> UNPACKFIG us, pack 55 -> PACKFIG us).
+// short rows (128^3 FP32: unpack 40 -> 25 us, pack 55 -> 28 us).
 // ---------------------------------------------------------------------------
 template <typename real>
 __device__ __forceinline__ void put4(real* p, real a, real b, real c, real d) {
@@ -225,8 +273,10 @@ template cudaError_t launch_pack<double>(const MirrorCopy&, cudaStream_t);
 template cudaError_t launch_unpack<float>(const MirrorCopy&, cudaStream_t);
 template cudaError_t launch_unpack<double>(const MirrorCopy&, cudaStream_t);
 
-template cudaError_t launch_count_nonfinite<float>(const void*, long long, void*, unsigned long long*, cudaStream_t);
-template cudaError_t launch_count_nonfinite<double>(const void*, long long, void*, unsigned long long*, cudaStream_t);
+template cudaError_t launch_count_nonfinite<float>(const void*, long long, unsigned long long*, cudaStream_t);
+template cudaError_t launch_count_nonfinite<double>(const void*, long long, unsigned long long*, cudaStream_t);
+template cudaError_t launch_load_f<float>(const void*, void*, void*, long long, unsigned long long*, cudaStream_t);
+template cudaError_t launch_load_f<double>(const void*, void*, void*, long long, unsigned long long*, cudaStream_t);
 template cudaError_t launch_max_abs_diff<float>(const void*, const void*, long long, void*, double*, cudaStream_t);
 template cudaError_t launch_max_abs_diff<double>(const void*, const void*, long long, void*, double*, cudaStream_t);
 

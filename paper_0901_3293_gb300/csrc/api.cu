@@ -807,22 +807,20 @@ int build_graph(lcbp_lattice* h, int steps, cudaGraphExec_t* exec, bool* ok) {
 
 int sync_flat(lcbp_lattice* h);
 
-int diag(lcbp_lattice* h, double threshold, int with_f) {
-  const int rs = sync_flat(h);
-  if (rs) return rs;
-  DiagGeom g{h->nx, h->ny, h->nz, h->n, 0, h->p.A0, h->p.gamma, h->p.K, h->p.q0, h->p.walls_z, {}, 0.0};
+int diag(lcbp_lattice* h, double threshold, int what) {
+  // (from whichever copy of Q is current)
+  DiagGeom g{h->nx, h->ny, h->nz, h->n, h->p.A0, h->p.gamma, h->p.K, h->p.q0, h->mirror_ok, h->p.walls_z, {}, 0.0};
   for (int c = 0; c < 5; ++c) g.qw[c] = h->p.q_wall[c];
   g.c_div = h->p.l2_set ? 0.5 * (h->p.K - h->p.L2) : 0.0;
-  cudaError_t e = h->dtype == LCBP_F64
-                      ? launch_diag_one<double>(g, h->q, h->f[h->cur], with_f, threshold, h->d_partials, h->d_out,
-                                                h->stream)
-                      : launch_diag_one<float>(g, h->q, h->f[h->cur], with_f, threshold, h->d_partials, h->d_out,
-                                               h->stream);
+  const void* q = g.mirror ? h->qm : h->q;
+  cudaError_t e = h->dtype == LCBP_F64 ? launch_diag_one<double>(g, q, h->f[h->cur], what, threshold, h->d_partials,
+                                                                 h->d_err, h->d_out, h->stream)
+                                       : launch_diag_one<float>(g, q, h->f[h->cur], what, threshold, h->d_partials,
+                                                                h->d_err, h->d_out, h->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(h->h_out, h->d_out, 8 * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return cuda_fail(e, "diagnostics");
-  int rc = check_device_error(h);
-  if (rc) return rc;
+  if (h->h_out[7] != 0.0) return check_device_error(h);
   if (h->h_out[6] != 0.0) return fail(LCBP_ENONFINITE, "%.0f sites hold NaN or Inf", h->h_out[6]);
   return LCBP_OK;
 }
@@ -1483,7 +1481,7 @@ int lcbp_read_f(lcbp_lattice* h, void* dst, int dtype) {
 int lcbp_free_energy(lcbp_lattice* h, double* F) {
   CHECK_H(h);
   if (!F) return fail(LCBP_EINVAL, "F is NULL");
-  int rc = diag(h, 0.0, 0);
+  int rc = diag(h, 0.0, kDiagEnergy);
   if (rc) return rc;
   *F = h->h_out[0];
   return LCBP_OK;
@@ -1491,7 +1489,7 @@ int lcbp_free_energy(lcbp_lattice* h, double* F) {
 
 int lcbp_totals(lcbp_lattice* h, double* mass, double momentum[3]) {
   CHECK_H(h);
-  int rc = diag(h, 0.0, 1);
+  int rc = diag(h, 0.0, kDiagTotals);
   if (rc) return rc;
   if (mass) *mass = h->h_out[1];
   if (momentum) {
@@ -1505,7 +1503,7 @@ int lcbp_totals(lcbp_lattice* h, double* mass, double momentum[3]) {
 int lcbp_defect_fraction(lcbp_lattice* h, double threshold, double* fraction) {
   CHECK_H(h);
   if (!fraction) return fail(LCBP_EINVAL, "fraction is NULL");
-  int rc = diag(h, threshold, 0);
+  int rc = diag(h, threshold, kDiagDefects);
   if (rc) return rc;
   *fraction = h->h_out[5] / (double)h->n;
   return LCBP_OK;

@@ -1,9 +1,11 @@
 // Initial states, moments, dtype conversion and FP64 diagnostics.
+#include <algorithm>
 #include <cmath>
 
 #include "common.cuh"
 #include "kernels.h"
 #include "tma.cuh"
+#include "zm.cuh"
 
 namespace lcbp {
 
@@ -363,127 +365,193 @@ __device__ __forceinline__ C chiral_contraction(const Sym5<C>& q, const Sym5<C>&
          qzz * c_zz;
 }
 
-// sums per block: [F_h, mass, Px, Py, Pz, defects, nonfinite, 0].  WALLS: F_h
-// in bond form with the anchored ghost planes (a build of its own, so that the
-// periodic build keeps few registers and many warps per SM).
-template <typename real, bool WALLS>
-// (FP32: four CTAs per SM, 64 registers)
-__global__ void __launch_bounds__(256, sizeof(real) == 4 ? 4 : 2)
-    k_diag(DiagGeom g, const real* __restrict__ Q, const real* __restrict__ f, int with_f, double threshold,
-           double* __restrict__ partials) {
+// Q of a lattice as the diagnostics read it: the flat field, or the padded
+// mirror where a run's state lives, whose 16-byte vectors save three of five loads
+// and whose use saves the copy back to the flat field
+template <typename real, bool MIRROR>
+struct QField {
+  const real* q;
+  long long n;      // flat: component stride
+  int nx, ny;
+  int nxm, nyq;     // mirror: row length, rows per plane
+  long long cq4;    // mirror: start of the yz array
+  __device__ __forceinline__ QField(const DiagGeom& g, const real* base)
+      : q(base), n(g.n), nx(g.nx), ny(g.ny), nxm(zm_mirror_nx(g.nx)), nyq(g.ny + 4),
+        cq4(4LL * zm_mirror_nx(g.nx) * (g.ny + 4) * g.nz) {}
+  // index of site (x, y, z), and the sites a row or a plane further
+  __device__ __forceinline__ long long at(int x, int y, int z) const {
+    if constexpr (MIRROR) return ((long long)z * nyq + y + 2) * nxm + x + kZmMirX;
+    else return ((long long)z * ny + y) * nx + x;
+  }
+  __device__ __forceinline__ Sym5<real> load(long long i) const {
+    if constexpr (MIRROR) {
+      real v[4];
+      ld4(q + 4 * i, 0, v);
+      return {v[0], v[1], v[2], v[3], q[cq4 + i]};
+    } else {
+      return {q[i], q[n + i], q[2 * n + i], q[3 * n + i], q[4 * n + i]};
+    }
+  }
+};
+
+template <typename C>
+__device__ __forceinline__ bool finite5(const Sym5<C>& q) {
+  return isfinite(q.xx) && isfinite(q.xy) && isfinite(q.xz) && isfinite(q.yy) && isfinite(q.yz);
+}
+
+// Sums per block: [F_h, mass, Px, Py, Pz, defects, nonfinite, 0].  Each WHAT does
+// its own work only (kDiagEnergy: the stencil of Q; kDiagTotals: f and a look at
+// Q; kDiagDefects: Q of the site).  WALLS: F_h in bond form with the anchored
+// ghost planes (a build of its own).
+//
+// The FP64 sums bound the energy and the totals (two FP64 lanes per SM: a
+// conversion and an addition per site and sum cost a warp 32 cycles of its SM),
+// so nothing else is done in FP64; the energy's threads march through the planes
+// of a chunk at one (x, y) with the plane's neighbours fetched a plane ahead, as
+// the Heun kernels do.  Three CTAs per SM: 85 registers, which hold the fetched plane.
+// 256^3 FP32, host-timed calls: energy 370 -> 202 us, totals 605 -> 300, defects
+// 369 -> 125; 64 x 64 x 256: 62 -> 39, 87 -> 52, 62 -> 26.
+constexpr int kDiagThreads = 256;
+template <typename real, int WHAT, bool WALLS, bool MIRROR>
+__global__ void __launch_bounds__(kDiagThreads, sizeof(real) == 4 ? 3 : 1)
+    k_diag(DiagGeom g, const real* q, const real* f, double threshold, int planes, double* __restrict__ partials) {
   using C = real;
-  // F_h, then sum(rho - 1), P: FP64; the sites, defects and non-finite sites counted
   double aF = 0.0, aR = 0.0, aJx = 0.0, aJy = 0.0, aJz = 0.0;
-  int sites = 0, defects = 0, bad = 0;
-  const real* qp = Q + 5 * g.base;
-  const real* fp = f ? f + 15 * g.base : nullptr;
-  const long long n = g.n;
+  unsigned sites = 0, defects = 0, bad = 0;
+  const QField<real, MIRROR> Q(g, q);
+  const int nx = g.nx, ny = g.ny, nz = g.nz;
+  const long long n = g.n, np = (long long)nx * ny;
   const C A0 = (C)g.A0, gam = (C)g.gamma, K = (C)g.K, q0 = (C)g.q0;
   const C a2 = C(0.5) * A0 * (C(1) - gam / C(3)), a3 = A0 * gam, a4 = C(0.25) * A0 * gam;
   // the chiral and divergence terms take raw differences: factors 1/2 and 1/4 folded in
   const C kq0h = K * q0, kq0sq = C(2) * K * q0 * q0, cdiv4 = C(0.25) * (C)g.c_div;
-  // decided once: FP64 arithmetic is scarce, so the loop keeps only its FP64 sums
-  const bool has_div = g.c_div != 0.0, small = g.n < (1ll << 31);
+  const bool has_div = g.c_div != 0.0;
   const float tf = (float)threshold;
-  for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
-    int x, y, z;
-    if (small) {  // 32-bit index arithmetic
-      const int si = (int)s, row = si / g.nx;
-      x = si - row * g.nx;
-      z = row / g.ny;
-      y = row - z * g.ny;
-    } else {
-      const long long row = s / g.nx;
-      x = (int)(s - row * g.nx);
-      z = (int)(row / g.ny);
-      y = (int)(row - (long long)z * g.ny);
-    }
-    const int xp = x + 1 == g.nx ? 0 : x + 1, xm = x == 0 ? g.nx - 1 : x - 1;
-    const int yp = y + 1 == g.ny ? 0 : y + 1, ym = y == 0 ? g.ny - 1 : y - 1;
-    const int zp = z + 1 == g.nz ? 0 : z + 1, zm = z == 0 ? g.nz - 1 : z - 1;
-    auto at = [&](int xx, int yy, int zz) { return ((long long)zz * g.ny + yy) * g.nx + xx; };
-    const Sym5<C> qc = load5(qp, n, s);
-    const Sym5<C> qxp = load5(qp, n, at(xp, y, z)), qyp = load5(qp, n, at(x, yp, z)), qzp = load5(qp, n, at(x, y, zp));
-    const bool finite = isfinite(qc.xx) && isfinite(qc.xy) && isfinite(qc.xz) && isfinite(qc.yy) && isfinite(qc.yz);
-    const C qzz = -qc.xx - qc.yy;
-    const C tr2 = qc.xx * qc.xx + qc.yy * qc.yy + qzz * qzz + C(2) * (qc.xy * qc.xy + qc.xz * qc.xz + qc.yz * qc.yz);
-    // Tr Q^3 = 3 det Q for a traceless Q
-    const C det = qc.xx * (qc.yy * qzz - qc.yz * qc.yz) - qc.xy * (qc.xy * qzz - qc.yz * qc.xz) +
-                  qc.xz * (qc.xy * qc.yz - qc.yy * qc.xz);
-    const C bulk = a2 * tr2 - a3 * det + a4 * tr2 * tr2;
-    C Fs;
-    if constexpr (!WALLS) {
-      const C grad2 = dist2(qc, qxp) + dist2(qc, qyp) + dist2(qc, qzp);
-      const Sym5<C> dx = diff5(qxp, load5(qp, n, at(xm, y, z)));
-      const Sym5<C> dy = diff5(qyp, load5(qp, n, at(x, ym, z)));
-      const Sym5<C> dz = diff5(qzp, load5(qp, n, at(x, y, zm)));
-      // 2 K q0 Q:C with C from central derivatives = K q0 (Q:C of the raw differences)
-      Fs = bulk + C(0.5) * K * grad2 + kq0h * chiral_contraction(qc, dx, dy, dz) + kq0sq * tr2;
-      if (has_div) {
-        // div_a = sum_b D0_b Q_ab; raw differences carry twice it
-        const C vx = dx.xx + dy.xy + dz.xz, vy = dx.xy + dy.yy + dz.yz, vz = dx.xz + dy.yz + dz.zz();
-        Fs -= cdiv4 * (vx * vx + vy * vy + vz * vz);
+  // items: kDiagThreads positions of a plane times `planes` planes
+  const long long blocks = (np + kDiagThreads - 1) / kDiagThreads;
+  const long long items = blocks * ((nz + planes - 1) / planes);
+  for (long long it = blockIdx.x; it < items; it += gridDim.x) {
+    const long long pos = it % blocks * kDiagThreads + threadIdx.x;
+    if (pos >= np) continue;
+    const int y = (int)(pos / nx), x = (int)(pos - (long long)y * nx);
+    const int z0 = (int)(it / blocks) * planes, z1 = min(z0 + planes, nz);
+    const int xp = x + 1 == nx ? 0 : x + 1, xm = x == 0 ? nx - 1 : x - 1;
+    const int yp = y + 1 == ny ? 0 : y + 1, ym = y == 0 ? ny - 1 : y - 1;
+    auto above = [&](int z) { return z + 1 == nz ? 0 : z + 1; };
+    if constexpr (WHAT == kDiagEnergy) {
+      // plane z's site, its z neighbours, and its neighbours in the plane (fetched a plane ahead)
+      Sym5<C> qc = Q.load(Q.at(x, y, z0)), qzm = Q.load(Q.at(x, y, z0 == 0 ? nz - 1 : z0 - 1));
+      Sym5<C> fzp, fxp, fyp, fxm, fym;
+      auto fetch = [&](int z) {
+        fzp = Q.load(Q.at(x, y, above(z)));
+        fxp = Q.load(Q.at(xp, y, z));
+        fyp = Q.load(Q.at(x, yp, z));
+        if constexpr (!WALLS) {
+          fxm = Q.load(Q.at(xm, y, z));
+          fym = Q.load(Q.at(x, ym, z));
+        }
+      };
+      fetch(z0);
+      for (int z = z0; z < z1; ++z) {
+        const Sym5<C> qzp = fzp, qxp = fxp, qyp = fyp, qxm = fxm, qym = fym;
+        if (z + 1 < z1) fetch(z + 1);
+        const C qzz = -qc.xx - qc.yy;
+        const C tr2 =
+            qc.xx * qc.xx + qc.yy * qc.yy + qzz * qzz + C(2) * (qc.xy * qc.xy + qc.xz * qc.xz + qc.yz * qc.yz);
+        // Tr Q^3 = 3 det Q for a traceless Q
+        const C det = qc.xx * (qc.yy * qzz - qc.yz * qc.yz) - qc.xy * (qc.xy * qzz - qc.yz * qc.xz) +
+                      qc.xz * (qc.xy * qc.yz - qc.yy * qc.xz);
+        const C bulk = a2 * tr2 - a3 * det + a4 * tr2 * tr2;
+        C Fs;
+        if constexpr (!WALLS) {
+          const C grad2 = dist2(qc, qxp) + dist2(qc, qyp) + dist2(qc, qzp);
+          const Sym5<C> dx = diff5(qxp, qxm), dy = diff5(qyp, qym), dz = diff5(qzp, qzm);
+          // 2 K q0 Q:C with C from central derivatives = K q0 (Q:C of the raw differences)
+          Fs = bulk + C(0.5) * K * grad2 + kq0h * chiral_contraction(qc, dx, dy, dz) + kq0sq * tr2;
+          if (has_div) {
+            // div_a = sum_b D0_b Q_ab; raw differences carry twice it
+            const C vx = dx.xx + dy.xy + dz.xz, vy = dx.xy + dy.yy + dz.yz, vz = dx.xz + dy.yz + dz.zz();
+            Fs -= cdiv4 * (vx * vx + vy * vy + vz * vz);
+          }
+        } else {
+          // bond form: this site's three forward bonds (the z bond of the top plane
+          // ends on the anchored ghost) and, on the bottom plane, the bond from the
+          // ghost below; every bond touching the lattice is counted once
+          const Sym5<C> qw = {(C)g.qw[0], (C)g.qw[1], (C)g.qw[2], (C)g.qw[3], (C)g.qw[4]};
+          C Fb = bond_energy(qc, qxp, 0, K, q0) + bond_energy(qc, qyp, 1, K, q0);
+          Fb += bond_energy(qc, z == nz - 1 ? qw : qzp, 2, K, q0);
+          if (z == 0) Fb += bond_energy(qw, qc, 2, K, q0);
+          Fs = bulk + Fb + kq0sq * tr2;
+        }
+        aF += (double)Fs;
+        bad += finite5(qc) ? 0u : 1u;
+        qzm = qc;
+        qc = qzp;
       }
     } else {
-      // bond form: this site's three forward bonds (the z bond of the top plane
-      // ends on the anchored ghost) and, on the bottom plane, the bond from the
-      // ghost below; every bond touching the lattice is counted once
-      const Sym5<C> qw = {(C)g.qw[0], (C)g.qw[1], (C)g.qw[2], (C)g.qw[3], (C)g.qw[4]};
-      C Fb = bond_energy(qc, qxp, 0, K, q0) + bond_energy(qc, qyp, 1, K, q0);
-      Fb += bond_energy(qc, z == g.nz - 1 ? qw : qzp, 2, K, q0);
-      if (z == 0) Fb += bond_energy(qw, qc, 2, K, q0);
-      Fs = bulk + Fb + kq0sq * tr2;
-    }
-    aF += (double)Fs;
-    defects += finite && top_eigenvalue_below(qc, threshold, tf) ? 1 : 0;
-    ++sites;
-    bool ffin = true;
-    if (with_f) {
-      // deviation storage: rho = 1 + sum df_i; the per-site sums of the small
-      // deviations in the state's precision, the sum over sites in FP64
-      C r = C(0), jx = C(0), jy = C(0), jz = C(0);
+#pragma unroll 2
+      for (int z = z0; z < z1; ++z) {
+        const Sym5<C> qc = Q.load(Q.at(x, y, z));
+        bool fin = finite5(qc);
+        if constexpr (WHAT == kDiagDefects) defects += fin && top_eigenvalue_below(qc, threshold, tf) ? 1u : 0u;
+        if constexpr (WHAT == kDiagTotals) {
+          // deviation storage: rho = 1 + sum df_i; the per-site sums of the small
+          // deviations in the state's precision, the sum over sites in FP64
+          const real* fs = f + (long long)z * np + pos;
+          C r = C(0), jx = C(0), jy = C(0), jz = C(0);
 #pragma unroll
-      for (int i = 0; i < NV; ++i) {
-        const C fi = fp[i * n + s];
-        ffin = ffin && isfinite(fi);
-        r += fi;
-        if (ex(i) > 0) jx += fi; else if (ex(i) < 0) jx -= fi;
-        if (ey(i) > 0) jy += fi; else if (ey(i) < 0) jy -= fi;
-        if (ez(i) > 0) jz += fi; else if (ez(i) < 0) jz -= fi;
+          for (int i = 0; i < NV; ++i) {
+            const C fi = fs[i * n];
+            fin = fin && isfinite(fi);
+            r += fi;
+            if (ex(i) > 0) jx += fi; else if (ex(i) < 0) jx -= fi;
+            if (ey(i) > 0) jy += fi; else if (ey(i) < 0) jy -= fi;
+            if (ez(i) > 0) jz += fi; else if (ez(i) < 0) jz -= fi;
+          }
+          aR += (double)r;
+          aJx += (double)jx;
+          aJy += (double)jy;
+          aJz += (double)jz;
+          ++sites;
+        }
+        bad += fin ? 0u : 1u;
       }
-      aR += (double)r;
-      aJx += (double)jx;
-      aJy += (double)jy;
-      aJz += (double)jz;
     }
-    bad += finite && ffin ? 0 : 1;
   }
   // mass = sites + sum(rho - 1).  Block reduction in a fixed order: a shuffle
-  // tree within each warp, then warp 0 adds the eight warps' sums in order.
-  double acc[7] = {aF, with_f ? aR + (double)sites : 0.0, aJx, aJy, aJz, (double)defects, (double)bad};
-#pragma unroll
-  for (int k = 0; k < 7; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_down_sync(0xffffffffu, acc[k], o);
-  __shared__ double red[8][8];
+  // tree within each warp, then the first lanes add the warps' sums in order.
+  double acc[7] = {aF, aR + (double)sites, aJx, aJy, aJz, (double)defects, (double)bad};
+  __shared__ double red[kDiagThreads / 32][8];
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  if (lane == 0)
 #pragma unroll
-    for (int k = 0; k < 7; ++k) red[warp][k] = acc[k];
+  for (int k = 0; k < 7; ++k) {
+    const bool used = k == 6 || (WHAT == kDiagEnergy ? k == 0 : WHAT == kDiagDefects ? k == 5 : k >= 1 && k <= 4);
+    if (!used) acc[k] = 0.0;
+    else
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_down_sync(0xffffffffu, acc[k], o);
+    if (lane == 0) red[warp][k] = acc[k];
+  }
   __syncthreads();
   if (threadIdx.x < 8) {
     const int k = threadIdx.x;
     double t = 0.0;
     if (k < 7)
-      for (int w = 0; w < (int)blockDim.x / 32; ++w) t += red[w][k];
+      for (int w = 0; w < kDiagThreads / 32; ++w) t += red[w][k];
     partials[blockIdx.x * 8 + k] = t;
   }
 }
 
 // the block partials summed per quantity: warp k sums quantity k, lanes
-// striding over the blocks, then a shuffle tree (a fixed order)
-__global__ void k_diag_final(const double* __restrict__ partials, int nblocks, double* __restrict__ out) {
+// striding over the blocks, then a shuffle tree (a fixed order); out[7] takes the
+// error flag of the step's kernels, so that one copy brings both to the host
+__global__ void k_diag_final(const double* __restrict__ partials, int nblocks, const int* err,
+                             double* __restrict__ out) {
   const int k = threadIdx.x / 32, lane = threadIdx.x % 32;
+  if (k == 7) {
+    if (lane == 0) out[7] = err ? (double)*err : 0.0;
+    return;
+  }
   double s = 0.0;
   for (int b = lane; b < nblocks; b += 32) s += partials[b * 8 + k];
   for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
@@ -511,24 +579,44 @@ cudaError_t launch_wait_probe(uint64_t limit_ns, int* flag, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-constexpr int kDiagBlocks = 512;
+// CTAs of k_diag: three per SM of the 152; fewer where there is less work
+constexpr int kDiagBlocks = 456;
+static_assert(kDiagBlocks * 8 <= kDiagPartials, "the partials buffer holds 8 values per block");
+
+template <typename real, int WHAT, bool WALLS, bool MIRROR>
+void diag_launch(const DiagGeom& g, const void* q, const void* f, double threshold, double* partials, const int* err,
+                 double* out, cudaStream_t s) {
+  const long long blocks = ((long long)g.nx * g.ny + kDiagThreads - 1) / kDiagThreads;
+  // planes per item: the fewer the shorter the last wave, up to 16 for the energy's marches
+  const long long share = (blocks * g.nz + kDiagBlocks - 1) / kDiagBlocks;
+  const int planes = (int)std::max<long long>(1, std::min<long long>(16, share));
+  const long long items = blocks * ((g.nz + planes - 1) / planes);
+  const int grid = (int)std::min<long long>(items, kDiagBlocks);
+  k_diag<real, WHAT, WALLS, MIRROR><<<grid, kDiagThreads, 0, s>>>(
+      g, static_cast<const real*>(q), static_cast<const real*>(f), threshold, planes, partials);
+  k_diag_final<<<1, 256, 0, s>>>(partials, grid, err, out);
+}
+
+template <typename real, bool MIRROR>
+void diag_what(const DiagGeom& g, const void* q, const void* f, int what, double threshold, double* partials,
+               const int* err, double* out, cudaStream_t s) {
+  if (what == kDiagTotals) diag_launch<real, kDiagTotals, false, MIRROR>(g, q, f, threshold, partials, err, out, s);
+  else if (what == kDiagDefects)
+    diag_launch<real, kDiagDefects, false, MIRROR>(g, q, f, threshold, partials, err, out, s);
+  else if (g.walls) diag_launch<real, kDiagEnergy, true, MIRROR>(g, q, f, threshold, partials, err, out, s);
+  else diag_launch<real, kDiagEnergy, false, MIRROR>(g, q, f, threshold, partials, err, out, s);
+}
 
 template <typename real>
-cudaError_t launch_diag_one(const DiagGeom& g, const void* q, const void* f, int with_f, double threshold,
-                            double* partials, double* out, cudaStream_t s) {
-  static_assert(kDiagBlocks * 8 == kDiagPartials, "the partials buffer holds 8 values per block");
-  if (g.walls)
-    k_diag<real, true><<<kDiagBlocks, 256, 0, s>>>(g, static_cast<const real*>(q), static_cast<const real*>(f),
-                                                    with_f, threshold, partials);
-  else
-    k_diag<real, false><<<kDiagBlocks, 256, 0, s>>>(g, static_cast<const real*>(q), static_cast<const real*>(f),
-                                                     with_f, threshold, partials);
-  k_diag_final<<<1, 256, 0, s>>>(partials, kDiagBlocks, out);
+cudaError_t launch_diag_one(const DiagGeom& g, const void* q, const void* f, int what, double threshold,
+                            double* partials, const int* err, double* out, cudaStream_t s) {
+  if (g.mirror) diag_what<real, true>(g, q, f, what, threshold, partials, err, out, s);
+  else diag_what<real, false>(g, q, f, what, threshold, partials, err, out, s);
   return cudaGetLastError();
 }
-template cudaError_t launch_diag_one<float>(const DiagGeom&, const void*, const void*, int, double, double*, double*,
-                                            cudaStream_t);
-template cudaError_t launch_diag_one<double>(const DiagGeom&, const void*, const void*, int, double, double*, double*,
-                                             cudaStream_t);
+template cudaError_t launch_diag_one<float>(const DiagGeom&, const void*, const void*, int, double, double*,
+                                            const int*, double*, cudaStream_t);
+template cudaError_t launch_diag_one<double>(const DiagGeom&, const void*, const void*, int, double, double*,
+                                             const int*, double*, cudaStream_t);
 
 }  // namespace lcbp

@@ -32,6 +32,7 @@ struct lcbp_batch {
   int device;
   std::vector<int> nx, ny, nz;
   std::vector<long long> n, base;
+  std::vector<long long> qm_off;  // first element of each replica's Q mirror (fast path)
   long long ntot;
   std::vector<HostParams> p;
   int flow_on, coupling;
@@ -516,19 +517,18 @@ int moments_all(lcbp_batch* b) {
   return e == cudaSuccess ? LCBP_OK : cuda_fail(e, "moments");
 }
 
-int diag(lcbp_batch* b, int r, double threshold, int with_f) {
-  const int rs = sync_flat(b);
-  if (rs) return rs;
-  DiagGeom g{b->nx[r], b->ny[r], b->nz[r], b->n[r], b->base[r], b->p[r].A0, b->p[r].gamma, b->p[r].K, b->p[r].q0};
-  cudaError_t e = b->dtype == LCBP_F64 ? launch_diag_one<double>(g, b->q, b->f[b->cur], with_f, threshold,
-                                                                 b->d_partials, b->d_out, b->stream)
-                                       : launch_diag_one<float>(g, b->q, b->f[b->cur], with_f, threshold,
-                                                                b->d_partials, b->d_out, b->stream);
+int diag(lcbp_batch* b, int r, double threshold, int what) {
+  DiagGeom g{b->nx[r], b->ny[r], b->nz[r], b->n[r], b->p[r].A0, b->p[r].gamma, b->p[r].K, b->p[r].q0, b->mirror_ok};
+  const void* q = field(b, b->q, 5, r);
+  if (b->mirror_ok) q = static_cast<char*>(b->qm) + (size_t)b->qm_off[r] * b->es;
+  const void* f = field(b, b->f[b->cur], 15, r);
+  cudaError_t e = b->dtype == LCBP_F64
+                      ? launch_diag_one<double>(g, q, f, what, threshold, b->d_partials, b->d_err, b->d_out, b->stream)
+                      : launch_diag_one<float>(g, q, f, what, threshold, b->d_partials, b->d_err, b->d_out, b->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->h_out, b->d_out, 64, cudaMemcpyDeviceToHost, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return cuda_fail(e, "diagnostics");
-  int rc = check_error_flag(b);
-  if (rc) return rc;
+  if (b->h_out[7] != 0.0) return check_error_flag(b);
   if (b->h_out[6] != 0.0) return fail(LCBP_ENONFINITE, "replica %d: %.0f sites hold NaN or Inf", r, b->h_out[6]);
   return LCBP_OK;
 }
@@ -596,6 +596,7 @@ int lcbp_batch_create(int R, const int* dims, const lcbp_params* params, int dty
     members[cls[r]].push_back(r);
   }
   b->base.assign(R, 0);
+  b->qm_off.assign(R, 0);
   for (int k = 0; k < (int)members.size(); ++k) {
     const int q = members[k][0];
     if (k < kZmMaxClasses) {
@@ -634,6 +635,7 @@ int lcbp_batch_create(int R, const int* dims, const lcbp_params* params, int dty
     const long long nxm = zm_mirror_nx(c.G.nx), cq = nxm * (c.G.ny + 4) * c.G.nz, cu = nxm * (c.G.ny + 2) * c.G.nz;
     c.qm0 = qm_tot;
     qm_tot += ((long long)c.count * 5 * cq + 63) / 64 * 64;
+    for (int j = 0; j < c.count; ++j) b->qm_off[b->order[c.rep0 + j]] = c.qm0 + j * 5 * cq;
     c.um0 = um_tot;
     um_tot += ((long long)c.count * 4 * cu + 63) / 64 * 64;
   }
@@ -911,7 +913,7 @@ int lcbp_batch_free_energy(lcbp_batch* b, int r, double* F) {
   if (!rc) rc = check_r(b, r);
   if (rc) return rc;
   if (!F) return fail(LCBP_EINVAL, "F is NULL");
-  rc = diag(b, r, 0.0, 0);
+  rc = diag(b, r, 0.0, kDiagEnergy);
   if (rc) return rc;
   *F = b->h_out[0];
   return LCBP_OK;
@@ -921,7 +923,7 @@ int lcbp_batch_totals(lcbp_batch* b, int r, double* mass, double momentum[3]) {
   int rc = check_b(b);
   if (!rc) rc = check_r(b, r);
   if (rc) return rc;
-  rc = diag(b, r, 0.0, 1);
+  rc = diag(b, r, 0.0, kDiagTotals);
   if (rc) return rc;
   if (mass) *mass = b->h_out[1];
   if (momentum) {
@@ -937,7 +939,7 @@ int lcbp_batch_defect_fraction(lcbp_batch* b, int r, double threshold, double* f
   if (!rc) rc = check_r(b, r);
   if (rc) return rc;
   if (!fraction) return fail(LCBP_EINVAL, "fraction is NULL");
-  rc = diag(b, r, threshold, 0);
+  rc = diag(b, r, threshold, kDiagDefects);
   if (rc) return rc;
   *fraction = b->h_out[5] / (double)b->n[r];
   return LCBP_OK;

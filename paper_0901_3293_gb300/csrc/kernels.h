@@ -83,11 +83,15 @@ cudaError_t launch_convert(const void* src, int src_dtype, void* dst, int dst_dt
 
 // Diagnostics of one lattice (replica), accumulated in FP64 with a fixed
 // reduction order: out[0..6] = [F_h, mass, Px, Py, Pz, #sites with
-// lambda_max(Q) < threshold, #non-finite sites].  partials holds 512 * 8 doubles.
+// lambda_max(Q) < threshold, #non-finite sites], of which a call forms the
+// quantities of its kind and the last; out[7] = *err (0 if err is null).
+// partials holds kDiagPartials doubles; q and f are the lattice's (replica's) own.
+enum DiagWhat { kDiagEnergy, kDiagTotals, kDiagDefects };
 struct DiagGeom {
   int nx, ny, nz;
-  long long n, base;
+  long long n;
   double A0, gamma, K, q0;
+  int mirror;      // q is the padded mirror of Q, not the flat field
   int walls;       // solid walls in z: F_h in bond form with the anchored ghost planes
   double qw[5];    // anchored Q (q5 order)
   double c_div;    // (K - L2) / 2: F_h gains -c_div |div Q|^2 per site
@@ -109,8 +113,8 @@ cudaError_t launch_max_abs_diff(const void* a, const void* b, long long n, void*
 // one CTA waits on a barrier nothing arrives on, for at most limit_ns; *flag = 1 if it gave up
 cudaError_t launch_wait_probe(uint64_t limit_ns, int* flag, cudaStream_t s);
 template <typename real>
-cudaError_t launch_diag_one(const DiagGeom& g, const void* q, const void* f, int with_f, double threshold,
-                            double* partials, double* out, cudaStream_t s);
+cudaError_t launch_diag_one(const DiagGeom& g, const void* q, const void* f, int what, double threshold,
+                            double* partials, const int* err, double* out, cudaStream_t s);
 constexpr int kDiagPartials = 512 * 8;
 
 // ---------------------------------------------------------------------------

@@ -108,11 +108,11 @@ extern "C" int lcbp_free_energy_noalloc(const void* q5, int dtype, int nx, int n
   int rc = scratch_for_current_device(&scratch);
   if (rc) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  DiagGeom g{nx, ny, nz, n, 0, A0, gamma, K, q0};
+  DiagGeom g{nx, ny, nz, n, A0, gamma, K, q0};
   double* partials = scratch;
   double* out = scratch + kDiagPartials;
-  cudaError_t e = dtype == LCBP_F64 ? launch_diag_one<double>(g, q5, nullptr, 0, 0.0, partials, out, st)
-                                    : launch_diag_one<float>(g, q5, nullptr, 0, 0.0, partials, out, st);
+  cudaError_t e = dtype == LCBP_F64 ? launch_diag_one<double>(g, q5, nullptr, kDiagEnergy, 0.0, partials, nullptr, out, st)
+                                    : launch_diag_one<float>(g, q5, nullptr, kDiagEnergy, 0.0, partials, nullptr, out, st);
   double res[8];
   if (e == cudaSuccess) e = cudaMemcpyAsync(res, out, sizeof(res), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);

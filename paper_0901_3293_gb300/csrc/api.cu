@@ -1675,18 +1675,14 @@ int lcbp_reequilibrate_f(lcbp_lattice* h) {
 }  // extern "C"
 
 namespace lcbp {
-// Enqueue the Beris-Edwards rate of a lattice into its predictor scratch on
-// the lattice's stream and record `done` after it; returns that scratch
-// (5 * N floats, valid until the lattice's next step)
-int lattice_rate(lcbp_lattice* h, const float** rate, cudaEvent_t done) {
+// Enqueue on stream s (ordered after the lattice's work by the caller) the
+// Beris-Edwards rate of a lattice into its predictor scratch, and the network
+// input from it; returns that scratch (5 * N floats, valid until the lattice's
+// next step)
+int lattice_rate_input(lcbp_lattice* h, const RateInput& in, cudaStream_t s, const float** rate) {
   if (!h) return fail(LCBP_EINVAL, "null lattice handle");
   if (h->dtype != LCBP_F32) return fail(LCBP_EINVAL, "the surrogate works on FP32 lattice state");
-  cudaSetDevice(h->device);
-  const int rs = sync_flat(h);
-  if (rs) return rs;
-  StepArgs a = step_args(h);
-  cudaError_t e = launch_rate<float>(a, h->stream);
-  if (e == cudaSuccess) e = cudaEventRecord(done, h->stream);
+  const cudaError_t e = launch_rate_input(step_args(h), in, s);
   if (e != cudaSuccess) return cuda_fail(e, "rate");
   *rate = static_cast<const float*>(h->qs);
   return LCBP_OK;

@@ -300,15 +300,18 @@ __device__ __forceinline__ Sym5<real> molecular_field(const Stencil7<real>& st, 
   }
   const real qzz = q.zz();
   // Q.Q (symmetric)
-  // (Tr Q = 0 turns Q_ab (Q_aa + Q_bb) of the off-diagonal entries into -Q_ab Q_cc)
+  // RAW (the stepping kernels): Tr Q = 0 turns Q_ab (Q_aa + Q_bb) of the
+  // off-diagonal entries into -Q_ab Q_cc, and shared terms are formed once.  The
+  // plain form stays for the rate that the surrogate extrapolates: an unjudged
+  // run of its calls amplifies the last bit of R to 3e-4 of Q in eight calls.
   const real qq_xx = q.xx * q.xx + q.xy * q.xy + q.xz * q.xz;
-  const real qq_xy = q.xz * q.yz - q.xy * qzz;
-  const real qq_xz = q.xy * q.yz - q.xz * q.yy;
+  const real qq_xy = RAW ? q.xz * q.yz - q.xy * qzz : q.xx * q.xy + q.xy * q.yy + q.xz * q.yz;
+  const real qq_xz = RAW ? q.xy * q.yz - q.xz * q.yy : q.xx * q.xz + q.xy * q.yz + q.xz * qzz;
   const real qq_yy = q.xy * q.xy + q.yy * q.yy + q.yz * q.yz;
-  const real qq_yz = q.xy * q.xz - q.yz * q.xx;
+  const real qq_yz = RAW ? q.xy * q.xz - q.yz * q.xx : q.xy * q.xz + q.yy * q.yz + q.yz * qzz;
   const real qq_zz = q.xz * q.xz + q.yz * q.yz + qzz * qzz;
   const real trq2 = qq_xx + qq_yy + qq_zz;
-  const real tr3 = (m.b_bulk * LCBP_Q(1, 3)) * trq2;
+  const real third = LCBP_Q(1, 3);
   // 7-point Laplacian
   auto lap = [&](real c, real a, real b, real cc, real d, real e, real f) {
     return (a + b) + (cc + d) + (e + f) - real(6) * c;
@@ -336,11 +339,16 @@ __device__ __forceinline__ Sym5<real> molecular_field(const Stencil7<real>& st, 
   const real bulk_iso = m.a_bulk + m.b_bulk * trq2 + m.kq0sq4;  // coefficient of -Q
   const real kc = RAW ? real(0.5) * m.kq0x2 : m.kq0x2;           // of C + C^T
   Sym5<real> H;
-  const real kc2 = kc + kc;
-  H.xx = (m.b_bulk * qq_xx - (bulk_iso * q.xx + tr3)) + m.K * l_xx - kc2 * c_xx;
+  if constexpr (RAW) {
+    const real tr3 = (m.b_bulk * third) * trq2, kc2 = kc + kc;
+    H.xx = (m.b_bulk * qq_xx - (bulk_iso * q.xx + tr3)) + m.K * l_xx - kc2 * c_xx;
+    H.yy = (m.b_bulk * qq_yy - (bulk_iso * q.yy + tr3)) + m.K * l_yy - kc2 * c_yy;
+  } else {
+    H.xx = -bulk_iso * q.xx + m.b_bulk * (qq_xx - third * trq2) + m.K * l_xx - kc * (c_xx + c_xx);
+    H.yy = -bulk_iso * q.yy + m.b_bulk * (qq_yy - third * trq2) + m.K * l_yy - kc * (c_yy + c_yy);
+  }
   H.xy = -bulk_iso * q.xy + m.b_bulk * qq_xy + m.K * l_xy - kc * (c_xy + c_yx);
   H.xz = -bulk_iso * q.xz + m.b_bulk * qq_xz + m.K * l_xz - kc * (c_xz + c_zx);
-  H.yy = (m.b_bulk * qq_yy - (bulk_iso * q.yy + tr3)) + m.K * l_yy - kc2 * c_yy;
   H.yz = -bulk_iso * q.yz + m.b_bulk * qq_yz + m.K * l_yz - kc * (c_yz + c_zy);
   return H;
 }

@@ -21,6 +21,7 @@
 #include "common.cuh"
 #include "conv.h"
 #include "tc.cuh"
+#include "zm.cuh"
 
 namespace lcbp {
 
@@ -388,6 +389,10 @@ __global__ void __launch_bounds__(kWinThreads) k_conv_win(const void* __restrict
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot + (uint32_t)pipe * L::PIPE_COLS;
+  // the input comes from the kernel before; the next kernel's CTAs may follow as
+  // this one's leave their SMs (every CTA holds its tensor memory by now)
+  grid_wait();
+  grid_launch_dependents();
 
   auto bounded_wait = [&](uint64_t* bar, uint32_t parity) {
     if (*abort_flag) return false;
@@ -712,7 +717,7 @@ cudaError_t conv_launch_win_t(const void* base, const CUtensorMap& tmW, const Co
   const long long items = (long long)g.ntiles * ((a.nz + 1) / 2);
   const int tmem_per_sm = std::max(1, 512 / (int)WinSmem<CIN, COUT>::TMEM_COLS);
   const int grid = (int)std::min<long long>(items, (long long)std::min(per_sm, tmem_per_sm) * sms);
-  k_conv_win<CIN, COUT, EPI><<<grid, kWinThreads, smem, s>>>(base, tmW, a, g);
+  launch_dependent(k_conv_win<CIN, COUT, EPI>, grid, kWinThreads, smem, s, base, tmW, a, g);
   return cudaGetLastError();
 }
 

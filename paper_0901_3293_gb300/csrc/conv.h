@@ -77,7 +77,7 @@ cudaError_t conv_launch(int cin, int cout, int epi, const ConvMaps& m, bool allo
                         const ConvArgs& a, int sms, cudaStream_t s);
 
 // Weight and bias gradients of one convolution on tcgen05 (dw.cu):
-// dW[t][ci][co] += sum_r X(r + o_t)[ci] dY(r)[co], db[co] += sum_r dY(r)[co]
+// dW[t][ci][co] = sum_r X(r + o_t)[ci] dY(r)[co], db[co] = sum_r dY(r)[co]
 // over the interior sites, X and dY padded BF16 (C_in, C_out in {16, 32}),
 // deterministic.  partial: dw_partial_floats(sms) floats of scratch.
 // dw_fits: whether the staged plane windows fit shared memory (planes up to

@@ -37,6 +37,7 @@
 
 #include "conv.h"
 #include "tc.cuh"
+#include "zm.cuh"
 
 namespace lcbp {
 
@@ -110,6 +111,8 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_dw_tc(const __nv_bfloat16* __
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  grid_wait();
+  grid_launch_dependents();
 
   auto bounded_wait = [&](uint64_t* bar, uint32_t parity) {
     if (*abort_flag) return false;
@@ -235,7 +238,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_dw_tc(const __nv_bfloat16* __
   }
 }
 
-// dW += sum over parts of the partials, db likewise, in a fixed order: a
+// dW = sum over parts of the partials, db likewise, in a fixed order: a
 // block takes 32 consecutive values; warp w adds parts w, w + 8, w + 16, ...
 // in turn (coalesced 128-byte rows), then thread l of warp 0 adds the eight
 // warps' sums in warp order.  A CTA's partial holds the weight gradients as
@@ -249,8 +252,10 @@ __global__ void __launch_bounds__(32 * kRedWarps) k_dw_reduce(const float* __res
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int i = blockIdx.x * 32 + lane;
   float s = 0.f;
+  grid_wait();
+  grid_launch_dependents();
   if (i < count) {
-#pragma unroll 4
+#pragma unroll 8
     for (int p = warp; p < nparts; p += kRedWarps) s += partial[(size_t)p * count + i];
   }
   red[warp][lane] = s;
@@ -261,9 +266,9 @@ __global__ void __launch_bounds__(32 * kRedWarps) k_dw_reduce(const float* __res
     for (int w = 1; w < kRedWarps; ++w) t += red[w][lane];
     if (i < nw) {
       const int tap = i / (cin * cout), r = i % (cin * cout), co = r / cin, ci = r % cin;
-      dW[((size_t)tap * cin + ci) * cout + co] += t;
+      dW[((size_t)tap * cin + ci) * cout + co] = t;
     } else {
-      db[i - nw] += t;
+      db[i - nw] = t;
     }
   }
 }
@@ -316,9 +321,9 @@ static cudaError_t dw_launch_t(const __nv_bfloat16* X, const __nv_bfloat16* dY, 
   cudaError_t e = cudaFuncSetAttribute(k_dw_tc<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int grid = g.items < sms ? g.items : sms;
-  k_dw_tc<CIN, COUT><<<grid, kDwThreads, smem, s>>>(X, dY, g, partial, err);
+  launch_dependent(k_dw_tc<CIN, COUT>, grid, kDwThreads, smem, s, X, dY, g, partial, err);
   const int nw = 27 * CIN * COUT;
-  k_dw_reduce<<<(nw + COUT + 31) / 32, 32 * kRedWarps, 0, s>>>(partial, grid, CIN, COUT, dW, db);
+  launch_dependent(k_dw_reduce, (nw + COUT + 31) / 32, 32 * kRedWarps, 0, s, partial, grid, CIN, COUT, dW, db);
   return cudaGetLastError();
 }
 

@@ -3,6 +3,7 @@
 
 #include <cstdint>
 #include <cuda.h>
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include "../../include/lcbp.h"
@@ -49,6 +50,14 @@ cudaError_t launch_field(const StepArgs& a, cudaStream_t s);
 // Beris-Edwards rate R(Q, u) (u = 0 with flow off) written to a.qs
 template <typename real>
 cudaError_t launch_rate(const StepArgs& a, cudaStream_t s);
+
+// network input of the surrogate beside the rate (FP32 lattices without walls)
+struct RateInput {
+  __nv_bfloat16* x;    // padded chunk-planar activations, 16 channels
+  float su, sr;        // input scales of u and R
+  float kappa, tau;
+};
+cudaError_t launch_rate_input(const StepArgs& a, const RateInput& in, cudaStream_t s);
 
 // initial Q (kinds as in lcbp.h); per-replica q0 is in q0s[rep] (device array)
 struct InitQArgs {

@@ -591,10 +591,11 @@ __device__ __forceinline__ void qside_body(const CUtensorMap* tmQ, const CUtenso
           const real g3[4] = {L(qs[0]), L(qs[1]), L(qs[2]), L(qs[3])};
           scratch_positions(nx, ny, gx, gy, [&](int xx, int yy) {
             real* d = pq + ((z * kZmPQG * nyp + yy) * nxp + xx) * 4;
-            st4g(d, g0[0], g0[1], g0[2], g0[3]);
-            st4g(d + gs, g1[0], g1[1], g1[2], g1[3]);
-            st4g(d + 2 * gs, g2[0], g2[1], g2[2], g2[3]);
-            if constexpr (!LBO) st4g(d + 3 * gs, g3[0], g3[1], g3[2], g3[3]);
+            // (not streaming: the next kernel reads them)
+            st4(d, g0[0], g0[1], g0[2], g0[3]);
+            st4(d + gs, g1[0], g1[1], g1[2], g1[3]);
+            st4(d + 2 * gs, g2[0], g2[1], g2[2], g2[3]);
+            if constexpr (!LBO) st4(d + 3 * gs, g3[0], g3[1], g3[2], g3[3]);
           });
         }
       };

@@ -137,8 +137,8 @@ constexpr int kDiagPartials = 512 * 8;
 // periodically padded scratch ("LB-ready" scratch) of 16 values per site in
 // four groups of four, interleaved per site ([z][group][Y][X][4], one 16-byte
 // vector per site and group):
-//   G0 = [C, V_x, V_y, V_z], G1 = [W_xy, W_xz, W_yz, F_x],
-//   G2 = [F_y, F_z, Q*_yz, rho - 1], G3 = [Q*_xx, Q*_xy, Q*_xz, Q*_yy],
+//   G0 = [C, V_x, V_y, V_z], G1 = [W_xy, W_xz, W_yz, rho - 1],
+//   G2 = [F_x, F_y, F_z, Q*_yz], G3 = [Q*_xx, Q*_xy, Q*_xz, Q*_yy],
 // over an (nx + 4) x (ny + 2) x nz array in which site (x, y, z) sits at
 // (X, Y) = (x + 1, y + 1) and the columns x = -1, nx and rows y = -1, ny hold
 // the periodic images.  The second kernel then stages them by TMA with no halo
@@ -146,7 +146,8 @@ constexpr int kDiagPartials = 512 * 8;
 // pre-collision terms (f^eq_i / tau_f + p_i of Sec. 2.2 Eq. feq, coeff, eq4):
 // a face direction +-e_a has F_a +- V_a, a corner direction s has
 // C + (s . V) / 8 + s_x s_y W_xy + s_x s_z W_xz + s_y s_z W_yz.  A corner
-// thus reads G0 and G1 of its source site, and the Q* stencil G3 and G2.
+// thus reads G0 and G1 of its source site; a face neighbour's G2 gives its F for
+// the face direction and its Q*_yz for the Q* stencil (G2 and G3).
 // ---------------------------------------------------------------------------
 constexpr int kZmPadX = 4;   // padded scratch: columns added to nx (one left, three right)
 constexpr int kZmPQ = 16;    // values per site of the padded scratch (four groups of four)

@@ -576,7 +576,7 @@ __device__ __forceinline__ void qside_body(const CUtensorMap* tmQ, const CUtenso
         qv[3] = q.yy + r.yy;
         qv[4] = q.yz + r.yz;
       }
-      // The site's 16 values (four groups; rho - 1 in the last place) of the
+      // The site's 16 values (four groups) of the
       // padded scratch for lane k, at the site's position and its images
       const int nxp = G.nxp, nyp = G.nyp, gs = 4 * G.nxp * G.nyp;  // gs: group stride
       auto put = [&](const V* P, const V* qs, const V& dr) {
@@ -586,8 +586,8 @@ __device__ __forceinline__ void qside_body(const CUtensorMap* tmQ, const CUtenso
           if (gy >= ny) continue;
           auto L = [&](const V& v) { return lane<SPT, real>(v, k); };
           const real g0[4] = {L(P[6]), L(P[3]), L(P[4]), L(P[5])};
-          const real g1[4] = {L(P[7]), L(P[8]), L(P[9]), L(P[0])};
-          const real g2[4] = {L(P[1]), L(P[2]), L(qs[4]), L(dr)};
+          const real g1[4] = {L(P[7]), L(P[8]), L(P[9]), L(dr)};
+          const real g2[4] = {L(P[0]), L(P[1]), L(P[2]), L(qs[4])};
           const real g3[4] = {L(qs[0]), L(qs[1]), L(qs[2]), L(qs[3])};
           scratch_positions(nx, ny, gx, gy, [&](int xx, int yy) {
             real* d = pq + ((z * kZmPQG * nyp + yy) * nxp + xx) * 4;
@@ -724,8 +724,8 @@ __device__ __forceinline__ void qsite_body(const ZmGeom& G, const Model<real>& m
   scratch_positions(G.nx, G.ny, x, y, [&](int X, int Y) {
     real* d = pq + ((z * kZmPQG * G.nyp + Y) * G.nxp + X) * 4;
     st4(d, P[6], P[3], P[4], P[5]);
-    st4(d + gs, P[7], P[8], P[9], P[0]);
-    st4(d + 2 * gs, P[1], P[2], qs[4], c[0]);
+    st4(d + gs, P[7], P[8], P[9], c[0]);
+    st4(d + 2 * gs, P[0], P[1], P[2], qs[4]);
     if constexpr (!LBO) st4(d + 3 * gs, qs[0], qs[1], qs[2], qs[3]);
   });
 }
@@ -1031,7 +1031,7 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
   auto fill = [&](int p) {
     real* sl = slot(p);
     for (int t = threadIdx.x; t < L::GS / 4; t += blockDim.x) {  // Q*_yz in G2, the rest in G3
-      sl[2 * L::GS + 4 * t + 2] = qw.yz;
+      sl[2 * L::GS + 4 * t + 3] = qw.yz;
       st4(sl + 3 * L::GS + 4 * t, qw.xx, qw.xy, qw.xz, qw.yy);
     }
   };
@@ -1143,12 +1143,12 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
         if constexpr (SPT == 1) fin[i] = fin_l[0][i];
         else fin[i] = V(fin_l[0][i], fin_l[SPT - 1][i], 0);
       }
-      // the site's G0 .. G2 of the scratch: [C V], [W F_x], [F_y F_z Q*_yz rho-1]
+      // the site's G0 .. G2 of the scratch: [C V], [W rho-1], [F Q*_yz]
       V c0[4], c1[4], c2[4];
       PG(nc, 0, ca, c0);
       PG(nc, 1, ca, c1);
       PG(nc, 2, ca, c2);
-      const V drho_y = c2[3];
+      const V drho_y = c1[3];
       V u_y[3];
       U3(nc, cu, u_y);
       const V rho_y = V(1) + drho_y;
@@ -1159,24 +1159,93 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
       // term of the opposite direction (all signs flipped)
       V pre[NV];
       pre[0] = (drho_y * LCBP_Q(8, 15) - rusq_n * LCBP_Q(2, 3)) * inv_tau;
+      // the six face neighbours: one vector of G2 gives F and Q*_yz of each, so the
+      // Q* stencil and the faces' terms are read together, and the Heun corrector
+      // comes before the collision, while the pulled populations arrive (256^3:
+      // 0.709 -> 0.694 ms, 64 x 64 x 256: 58.2 -> 56.5 us against the faces' terms as
+      // scalars of two groups and the corrector last)
+      Stencil7<V> st;
+      {
+        Sym5<V>* const nb[6] = {&st.xm, &st.xp, &st.ym, &st.yp, &st.zm, &st.zp};  // the sources of directions 1 .. 6
 #pragma unroll
-      for (int i = 1; i < NV; ++i) {
-        const bool bb = (ez(i) > 0 && wl) || (ez(i) < 0 && wh);
-        const real* sl = bb ? nc : (ez(i) > 0 ? nm : ez(i) < 0 ? np : nc);
-        const int idx = bb ? ca : ca - ey(i) * AW - ex(i);
-        if (i <= 6) {
+        for (int i = 1; i <= 6; ++i) {
           const int a = (i - 1) / 2;
-          // F_a: G1.3 (x), G2.0 (y), G2.1 (z); V_a: G0.(1 + a)
-          const V Fa = a == 0 ? PS(sl, 1, 3, idx) : PS(sl, 2, a - 1, idx), Va = PS(sl, 0, 1 + a, idx);
+          const bool bb = (ez(i) > 0 && wl) || (ez(i) < 0 && wh);
+          const real* sl = ez(i) > 0 ? nm : ez(i) < 0 ? np : nc;
+          const int idx = ca - ey(i) * AW - ex(i);
+          V g2[4];
+          PG(sl, 2, idx, g2);
+          const V Fa = bb ? c2[a] : g2[a], Va = bb ? c0[1 + a] : PS(sl, 0, 1 + a, idx);
           pre[i] = ((i & 1) != 0) != bb ? Fa + Va : Fa - Va;  // odd i: the + direction
-        } else {
-          V g0[4], g1[4];  // [C, V_x, V_y, V_z], [W_xy, W_xz, W_yz, F_x]
-          PG(sl, 0, idx, g0);
-          PG(sl, 1, idx, g1);
-          const V vs = signed_sum(ex(i), g0[1], ey(i), g0[2], ez(i), g0[3]);
-          const V ws = signed_sum(ex(i) * ey(i), g1[0], ex(i) * ez(i), g1[1], ey(i) * ez(i), g1[2]);
-          pre[i] = bb ? (g0[0] + ws) - LCBP_Q(1, 8) * vs : (g0[0] + ws) + LCBP_Q(1, 8) * vs;
+          if constexpr (!LBO) {
+            V g3[4];
+            PG(sl, 3, idx, g3);
+            *nb[i - 1] = Sym5<V>{g3[0], g3[1], g3[2], g3[3], g2[3]};
+          }
         }
+      }
+      if constexpr (!LBO) {
+        // Heun corrector with u^n
+        V g3c[4];
+        PG(nc, 3, ca, g3c);
+        st.c = Sym5<V>{g3c[0], g3c[1], g3c[2], g3c[3], c2[3]};
+        Sym5<V> dq[3];
+        const Sym5<V> h = molecular_field<true>(st, mv, dq);
+        V w[3][3];
+        const V half = V(0.5);
+        V uxp[3], uxm[3], uyp[3], uym[3], uzp[3], uzm[3];
+        U3(nc, cu + 1, uxp);
+        U3(nc, cu - 1, uxm);
+        U3(nc, cu + B::UW, uyp);
+        U3(nc, cu - B::UW, uym);
+        U3(np, cu, uzp);
+        U3(nm, cu, uzm);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          w[a][0] = uxp[a] - uxm[a];  // twice the central derivatives
+          w[a][1] = uyp[a] - uym[a];
+          V upz = uzp[a], umz = uzm[a];
+          if (wl) umz = -u_y[a];  // no slip half a spacing beyond the wall
+          if (wh) upz = -u_y[a];
+          w[a][2] = upz - umz;
+        }
+        const Sym5<V> r = be_rate<true>(st.c, h, dq, u_y, w, mv, true);
+        // Q^n of the site from the Q mirror ([xx xy xz yy] vectors, then the yz array)
+        int sq[SPT];
+#pragma unroll
+        for (int k = 0; k < SPT; ++k) sq[k] = (z * G.nyq + gy[k] + B::QPY) * G.nxm + gx + B::QPX;
+        const int cq = (int)G.cq;
+        V qa[4];
+        ld4v<SPT>(Qin, 4 * sq[0], 4 * sq[SPT - 1], qa);
+        const Sym5<V> q0 = {qa[0], qa[1], qa[2], qa[3], vld<SPT>(Qin, 4 * cq + sq[0], 4 * cq + sq[SPT - 1])};
+        const Sym5<V> q1 = {half * (q0.xx + st.c.xx + r.xx), half * (q0.xy + st.c.xy + r.xy),
+                            half * (q0.xz + st.c.xz + r.xz), half * (q0.yy + st.c.yy + r.yy),
+                            half * (q0.yz + st.c.yz + r.yz)};
+#pragma unroll
+        for (int k = 0; k < SPT; ++k) {
+          if (!lane_ok[k]) continue;
+          const real a = lane<SPT, real>(q1.xx, k), b = lane<SPT, real>(q1.xy, k), c = lane<SPT, real>(q1.xz, k),
+                     d = lane<SPT, real>(q1.yy, k), e = lane<SPT, real>(q1.yz, k);
+          const int nxm = G.nxm, nyq = G.nyq, cq4 = 4 * (int)G.cq;
+          mirror_positions(B::QPX, 2, nx, ny, gx, gy[k], [&](int X, int Y) {
+            const int o = (z * nyq + Y) * nxm + X;
+            st4g(Qout + 4 * o, a, b, c, d);
+            __stcs(&Qout[cq4 + o], e);
+          });
+        }
+      }
+      // the corners
+#pragma unroll
+      for (int i = 7; i < NV; ++i) {
+        const bool bb = (ez(i) > 0 && wl) || (ez(i) < 0 && wh);
+        const real* sl = bb ? nc : (ez(i) > 0 ? nm : np);
+        const int idx = bb ? ca : ca - ey(i) * AW - ex(i);
+        V g0[4], g1[4];  // [C, V_x, V_y, V_z], [W_xy, W_xz, W_yz, rho - 1]
+        PG(sl, 0, idx, g0);
+        PG(sl, 1, idx, g1);
+        const V vs = signed_sum(ex(i), g0[1], ey(i), g0[2], ez(i), g0[3]);
+        const V ws = signed_sum(ex(i) * ey(i), g1[0], ex(i) * ez(i), g1[1], ey(i) * ez(i), g1[2]);
+        pre[i] = bb ? (g0[0] + ws) - LCBP_Q(1, 8) * vs : (g0[0] + ws) + LCBP_Q(1, 8) * vs;
       }
       // C_i = (f^eq - f_i) / tau_f + p_i; predictor f* = f + C, and f + C / 2
       // (FP64 keeps f itself: see the corrector below)
@@ -1202,7 +1271,7 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
       // at the site's step-n values.  P(y) holds them for (rho^n, u^n), so
       // each takes the change of its moment part.
       const V dd = (drs - drho_y) * LCBP_Q(1, 30) - (rusq_s - rusq_n) * LCBP_Q(1, 12);
-      const V Fn[3] = {c1[3], c2[0], c2[1]};
+      const V Fn[3] = {c2[0], c2[1], c2[2]};
       V Fs[3], Vs[3];
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
@@ -1268,69 +1337,6 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
                          [&](int X, int Y) { st4g(rhou_new + 4 * ((z * nyu + Y) * nxm + X), a, b, c, d); });
       }
 
-      if constexpr (LBO) return;
-      // Heun corrector with u^n
-      // Q* at a box index: G3 = [xx xy xz yy] and G2.2 = yz
-      auto QS = [&](const real* sl, int idx) {
-        V g3[4];
-        PG(sl, 3, idx, g3);
-        return Sym5<V>{g3[0], g3[1], g3[2], g3[3], PS(sl, 2, 2, idx)};
-      };
-      Stencil7<V> st;
-      V g3c[4];
-      PG(nc, 3, ca, g3c);
-      st.c = Sym5<V>{g3c[0], g3c[1], g3c[2], g3c[3], c2[2]};
-      st.xm = QS(nc, ca - 1);
-      st.xp = QS(nc, ca + 1);
-      st.ym = QS(nc, ca - AW);
-      st.yp = QS(nc, ca + AW);
-      st.zm = QS(nm, ca);
-      st.zp = QS(np, ca);
-      Sym5<V> dq[3];
-      const Sym5<V> h = molecular_field<true>(st, mv, dq);
-      V w[3][3];
-      const V half = V(0.5);
-      V uxp[3], uxm[3], uyp[3], uym[3], uzp[3], uzm[3];
-      U3(nc, cu + 1, uxp);
-      U3(nc, cu - 1, uxm);
-      U3(nc, cu + B::UW, uyp);
-      U3(nc, cu - B::UW, uym);
-      U3(np, cu, uzp);
-      U3(nm, cu, uzm);
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        w[a][0] = uxp[a] - uxm[a];  // twice the central derivatives
-        w[a][1] = uyp[a] - uym[a];
-        V upz = uzp[a], umz = uzm[a];
-        if (wl) umz = -u_y[a];  // no slip half a spacing beyond the wall
-        if (wh) upz = -u_y[a];
-        w[a][2] = upz - umz;
-      }
-      const Sym5<V> r = be_rate<true>(st.c, h, dq, u_y, w, mv, true);
-      // Q^n of the site: the flat field, or the Q mirror ([xx xy xz yy]
-      // vectors, then the yz array)
-      int sq[SPT];
-#pragma unroll
-      for (int k = 0; k < SPT; ++k) sq[k] = (z * G.nyq + gy[k] + B::QPY) * G.nxm + gx + B::QPX;
-      const int cq = (int)G.cq;
-      V qa[4];
-      ld4v<SPT>(Qin, 4 * sq[0], 4 * sq[SPT - 1], qa);
-      const Sym5<V> q0 = {qa[0], qa[1], qa[2], qa[3], vld<SPT>(Qin, 4 * cq + sq[0], 4 * cq + sq[SPT - 1])};
-      const Sym5<V> q1 = {half * (q0.xx + st.c.xx + r.xx), half * (q0.xy + st.c.xy + r.xy),
-                          half * (q0.xz + st.c.xz + r.xz), half * (q0.yy + st.c.yy + r.yy),
-                          half * (q0.yz + st.c.yz + r.yz)};
-#pragma unroll
-      for (int k = 0; k < SPT; ++k) {
-        if (!lane_ok[k]) continue;
-        const real a = lane<SPT, real>(q1.xx, k), b = lane<SPT, real>(q1.xy, k), c = lane<SPT, real>(q1.xz, k),
-                   d = lane<SPT, real>(q1.yy, k), e = lane<SPT, real>(q1.yz, k);
-        const int nxm = G.nxm, nyq = G.nyq, cq4 = 4 * (int)G.cq;
-        mirror_positions(B::QPX, 2, nx, ny, gx, gy[k], [&](int X, int Y) {
-          const int o = (z * nyq + Y) * nxm + X;
-          st4g(Qout + 4 * o, a, b, c, d);
-          __stcs(&Qout[cq4 + o], e);
-        });
-      }
     };
     if (valid) {
       if (WALLS && (wlo || whi)) plane_work(std::true_type{});

@@ -186,7 +186,7 @@ struct QsideSmem {
   // own cells of a plane: H (5 components) then sigma_LC (5)
   static constexpr int TSLOT = 3 * TROWS * TCOLS, HSLOT = 10 * TY * TX;
   static constexpr int OFF_U = QSLOTS * QSLOT, OFF_T = OFF_U + USLOTS * USLOT;
-  static constexpr int OFF_H = OFF_T + 3 * TSLOT, OFF_BAR = align_elems(OFF_H + 2 * HSLOT, sizeof(real));
+  static constexpr int OFF_H = OFF_T + 4 * TSLOT, OFF_BAR = align_elems(OFF_H + 2 * HSLOT, sizeof(real));
   // barriers, then the abort flag
   static constexpr size_t bytes = sizeof(real) * (size_t)OFF_BAR + 16 * 8 + 16;
 };
@@ -253,6 +253,8 @@ __device__ __forceinline__ void qside_body(const CUtensorMap* tmQ, const CUtenso
   // plane p of Q lives in slot (p - (z0-2)) % 5, of rho u in slot (p - (z0-1)) % 4
   // (the plane offsets below are never negative: unsigned arithmetic keeps the ring
   // index a plain multiply-shift or mask)
+  // the lattice plane of p in [z0 - 2, z1 + 1]: no remainder but for the thinnest lattices
+  auto wz = [&](int p) { return nz >= 4 ? (p < 0 ? p + nz : p >= nz ? p - nz : p) : wrap(p, nz); };
   auto qslot = [&](int p) { return qring + ((unsigned)(p - (z0 - 2)) % L::QSLOTS) * L::QSLOT; };
   auto uslot = [&](int p) { return uring + ((unsigned)(p - (z0 - 1)) % L::USLOTS) * L::USLOT; };
   auto issue_q = [&](int p) {
@@ -262,11 +264,11 @@ __device__ __forceinline__ void qside_body(const CUtensorMap* tmQ, const CUtenso
     // the mirror's [xx xy xz yy] vectors, then its yz array (replica rc of a batch class)
     const int X = x0 - B::QX + B::QPX, Y = y0 - 2 + B::QPY;
     if constexpr (BATCH) {
-      tma_load_4d(qslot(p), tmQ, 4 * X, Y, wrap(p, nz), rc, bar);
-      tma_load_4d(qslot(p) + 4 * L::QCS, tmQ1, X, Y, wrap(p, nz), rc, bar);
+      tma_load_4d(qslot(p), tmQ, 4 * X, Y, wz(p), rc, bar);
+      tma_load_4d(qslot(p) + 4 * L::QCS, tmQ1, X, Y, wz(p), rc, bar);
     } else {
-      tma_load_3d(qslot(p), tmQ, 4 * X, Y, wrap(p, nz), bar);
-      tma_load_3d(qslot(p) + 4 * L::QCS, tmQ1, X, Y, wrap(p, nz), bar);
+      tma_load_3d(qslot(p), tmQ, 4 * X, Y, wz(p), bar);
+      tma_load_3d(qslot(p) + 4 * L::QCS, tmQ1, X, Y, wz(p), bar);
     }
   };
   auto issue_u = [&](int p) {
@@ -274,9 +276,9 @@ __device__ __forceinline__ void qside_body(const CUtensorMap* tmQ, const CUtenso
     uint64_t* bar = &bars[L::QSLOTS + k % L::USLOTS];
     mbar_arrive_expect_tx(bar, ubytes);
     if constexpr (BATCH)
-      tma_load_4d(uslot(p), tmU, 4 * (x0 - B::UX + B::UPX), y0 - 1 + B::UPY, wrap(p, nz), rc, bar);
+      tma_load_4d(uslot(p), tmU, 4 * (x0 - B::UX + B::UPX), y0 - 1 + B::UPY, wz(p), rc, bar);
     else
-      tma_load_3d(uslot(p), tmU, 4 * (x0 - B::UX + B::UPX), y0 - 1 + B::UPY, wrap(p, nz), bar);
+      tma_load_3d(uslot(p), tmU, 4 * (x0 - B::UX + B::UPX), y0 - 1 + B::UPY, wz(p), bar);
   };
   // Q and rho u at box index i0 (lane 0) and i1 (lane 1) of a staged slot:
   // the mirrors stage [row][col][4] vectors (Q: then its yz as [row][col])
@@ -311,7 +313,7 @@ __device__ __forceinline__ void qside_body(const CUtensorMap* tmQ, const CUtenso
       sl[4 * L::QCS + t] = qw.yz;
     }
   };
-  auto tslot = [&](int p) { return tring + ((unsigned)(p - z0 + 3) % 3u) * L::TSLOT; };
+  auto tslot = [&](int p) { return tring + ((unsigned)(p - z0 + 3) & 3u) * L::TSLOT; };
   auto hslot = [&](int p) { return hbuf + ((unsigned)(p - z0 + 2) & 1u) * L::HSLOT; };
 
   // H and tau of plane p on the tile plus a one-site ring (Q planes p-1..p+1);
@@ -972,6 +974,7 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
   grid_wait();  // the scratch comes from the kernel before this one
   grid_launch_dependents();
 
+  auto wz = [&](int p) { return nz >= 4 ? (p < 0 ? p + nz : p >= nz ? p - nz : p) : wrap(p, nz); };
   auto slot = [&](int p) { return ring + ((unsigned)(p - (z0 - 1)) % L::SLOTS) * L::SLOT; };
   // plane p: the padded P / Q* box (site (x, y) at padded (x + 1, y + 1), so the
   // box starting at padded (x0, y0) covers x0-1 .. x0+TX) and the u box of rho u
@@ -979,7 +982,7 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
     const unsigned k = p - (z0 - 1);
     uint64_t* bar = &bars[k % L::SLOTS];
     real* sl = slot(p);
-    const int zz = wrap(p, nz);
+    const int zz = wz(p);
     mbar_arrive_expect_tx(bar, L::TX_BYTES);
     // the scratch as (4 X, Y, group, z): x coordinate in elements of 4 per site
     if constexpr (BATCH) tma_load_5d(sl, tmPQ, 4 * x0, y0, 0, zz, rc, bar);
@@ -1001,8 +1004,8 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
       tma_prefetch_l2_5d(tmF1, xf, yb, zz, 4, rc);
       tma_prefetch_l2_5d(tmF2, xf, yb, zz, 9, rc);
       tma_prefetch_l2_5d(tmF2, xf, yb, zz, 13, rc);
-      tma_prefetch_l2_4d(tmQ, 4 * X, Y, wrap(p - 1, nz), rc);
-      tma_prefetch_l2_4d(tmQ1, X, Y, wrap(p - 1, nz), rc);
+      tma_prefetch_l2_4d(tmQ, 4 * X, Y, wz(p - 1), rc);
+      tma_prefetch_l2_4d(tmQ1, X, Y, wz(p - 1), rc);
     } else {
       tma_load_3d(sl + L::OFF_U, tmU3, 4 * (x0 - B::UX + B::UPX), y0 - 1 + B::UPY, zz, bar);
       if (G.pf) {
@@ -1015,8 +1018,8 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
         tma_prefetch_l2_4d(tmF2, xf, yb, zz, 13);
       }
       if constexpr (!LBO) {
-        tma_prefetch_l2_3d(tmQ, 4 * X, Y, wrap(p - 1, nz));
-        tma_prefetch_l2_3d(tmQ1, X, Y, wrap(p - 1, nz));
+        tma_prefetch_l2_3d(tmQ, 4 * X, Y, wz(p - 1));
+        tma_prefetch_l2_3d(tmQ1, X, Y, wz(p - 1));
       }
     }
   };
@@ -1115,7 +1118,7 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
     // the tile prefetches its row of plane z+2
     if (!BATCH && !G.pf && z + 2 <= z1 && (int)threadIdx.x < NV * TY) {
       const int i = threadIdx.x / TY, yy = min(y0 + (int)threadIdx.x % TY, ny - 1);
-      const real* row = f + (i * n + (wrap(z + 2, nz) * ny + yy) * nx);
+      const real* row = f + (i * n + (wz(z + 2) * ny + yy) * nx);
       for (int k = 0; k <= TX; k += 128 / (int)sizeof(real)) prefetch_l2(row + min(x0 + min(k, TX - 1), nx - 1));
     }
     // a wall's ghost plane: the anchored Q*

@@ -942,8 +942,16 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
   const int n = (int)G.n;  // (32-bit element offsets, as in k_qside)
   const int x0 = (bt % G.tiles_x) * TX;
   const int y0 = ((bt / G.tiles_x) % G.tiles_y) * TY;
-  const int z0 = (bt / (G.tiles_x * G.tiles_y)) * G.zc;
-  const int z1 = min(z0 + G.zc, nz);
+  // The CTA marches down its chunk of planes, marching plane p being lattice plane
+  // ztop - p, and the first CTAs take the highest chunk.  k_qside marches up, so the
+  // scratch that it wrote last, still in L2, is read first, and the next k_qside
+  // starts where this kernel ends: 128^3 173.4 -> 169.4 us a step, walls 128x96x64
+  // 72.8 -> 71.5, slab 64x64x256 88.5 -> 87.0; 256^3, whose scratch is far above L2,
+  // unchanged at 1144.  The short chunk stays last: leading with it left a tail of
+  // full ones (101x75x67: k_lbq 37.4 -> 41.2 us).
+  const int full = nz / G.zc, ci = bt / (G.tiles_x * G.tiles_y);  // full chunks; a short one goes last
+  const int zlow = (ci < full ? full - 1 - ci : ci) * G.zc, ztop = min(zlow + G.zc, nz) - 1;
+  const int z0 = 0, z1 = ztop - zlow + 1;
   const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
   const int gx = x0 + tx;
   int gy[SPT];
@@ -975,6 +983,7 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
   grid_launch_dependents();
 
   auto wz = [&](int p) { return nz >= 4 ? (p < 0 ? p + nz : p >= nz ? p - nz : p) : wrap(p, nz); };
+  auto plane = [&](int p) { return wz(ztop - p); };
   auto slot = [&](int p) { return ring + ((unsigned)(p - (z0 - 1)) % L::SLOTS) * L::SLOT; };
   // plane p: the padded P / Q* box (site (x, y) at padded (x + 1, y + 1), so the
   // box starting at padded (x0, y0) covers x0-1 .. x0+TX) and the u box of rho u
@@ -982,7 +991,7 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
     const unsigned k = p - (z0 - 1);
     uint64_t* bar = &bars[k % L::SLOTS];
     real* sl = slot(p);
-    const int zz = wz(p);
+    const int zz = plane(p), zb = plane(p - 1);
     mbar_arrive_expect_tx(bar, L::TX_BYTES);
     // the scratch as (4 X, Y, group, z): x coordinate in elements of 4 per site
     if constexpr (BATCH) tma_load_5d(sl, tmPQ, 4 * x0, y0, 0, zz, rc, bar);
@@ -1004,8 +1013,8 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
       tma_prefetch_l2_5d(tmF1, xf, yb, zz, 4, rc);
       tma_prefetch_l2_5d(tmF2, xf, yb, zz, 9, rc);
       tma_prefetch_l2_5d(tmF2, xf, yb, zz, 13, rc);
-      tma_prefetch_l2_4d(tmQ, 4 * X, Y, wz(p - 1), rc);
-      tma_prefetch_l2_4d(tmQ1, X, Y, wz(p - 1), rc);
+      tma_prefetch_l2_4d(tmQ, 4 * X, Y, zb, rc);
+      tma_prefetch_l2_4d(tmQ1, X, Y, zb, rc);
     } else {
       tma_load_3d(sl + L::OFF_U, tmU3, 4 * (x0 - B::UX + B::UPX), y0 - 1 + B::UPY, zz, bar);
       if (G.pf) {
@@ -1018,8 +1027,8 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
         tma_prefetch_l2_4d(tmF2, xf, yb, zz, 13);
       }
       if constexpr (!LBO) {
-        tma_prefetch_l2_3d(tmQ, 4 * X, Y, wz(p - 1));
-        tma_prefetch_l2_3d(tmQ1, X, Y, wz(p - 1));
+        tma_prefetch_l2_3d(tmQ, 4 * X, Y, zb);
+        tma_prefetch_l2_3d(tmQ1, X, Y, zb);
       }
     }
   };
@@ -1030,7 +1039,7 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
     return ok;
   };
   // a staged plane beyond a wall: only its Q* is read (the anchored qw)
-  auto ghost = [&](int p) { return WALLS && (p < 0 || p >= nz); };
+  auto ghost = [&](int p) { return WALLS && (ztop - p < 0 || ztop - p >= nz); };
   auto fill = [&](int p) {
     real* sl = slot(p);
     for (int t = threadIdx.x; t < L::GS / 4; t += blockDim.x) {  // Q*_yz in G2, the rest in G3
@@ -1075,7 +1084,8 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
   // One CTA barrier per plane, after the wait: past it every thread has
   // finished plane z-1, the last reader of the slot that the load of plane
   // z+2 overwrites (plane z-2), so that load is issued right after it.
-  for (int z = z0; z < z1; ++z) {
+  for (int zl = z0; zl < z1; ++zl) {
+    const int z = ztop - zl;  // the lattice plane
     // populations f_i(y - e_i) and the site's rho - 1, issued before the
     // barrier wait so that they overlap it
     real fin_l[SPT][NV];
@@ -1104,7 +1114,7 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
       if (WALLS && (wlo || whi)) pull(std::true_type{});
       else pull(std::false_type{});
     }
-    wait(z + 1);
+    wait(zl + 1);
     __syncthreads();
     if (*abort_flag) {
       aborted = true;
@@ -1112,19 +1122,19 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
     }
     if (threadIdx.x == 0) {
       fence_proxy_async();
-      if (z + 2 <= z1) issue(z + 2);
+      if (zl + 2 <= z1) issue(zl + 2);
     }
     // rows of f that no tensor map describes: a thread per population and row of
-    // the tile prefetches its row of plane z+2
-    if (!BATCH && !G.pf && z + 2 <= z1 && (int)threadIdx.x < NV * TY) {
+    // the tile prefetches its row of the plane after the next
+    if (!BATCH && !G.pf && zl + 2 <= z1 && (int)threadIdx.x < NV * TY) {
       const int i = threadIdx.x / TY, yy = min(y0 + (int)threadIdx.x % TY, ny - 1);
-      const real* row = f + (i * n + (wz(z + 2) * ny + yy) * nx);
+      const real* row = f + (i * n + (plane(zl + 2) * ny + yy) * nx);
       for (int k = 0; k <= TX; k += 128 / (int)sizeof(real)) prefetch_l2(row + min(x0 + min(k, TX - 1), nx - 1));
     }
     // a wall's ghost plane: the anchored Q*
-    if (WALLS && (ghost(z + 1) || (z == z0 && ghost(z0 - 1)))) {
-      if (ghost(z + 1)) fill(z + 1);
-      if (z == z0 && ghost(z0 - 1)) fill(z0 - 1);
+    if (WALLS && (ghost(zl + 1) || (zl == z0 && ghost(z0 - 1)))) {
+      if (ghost(zl + 1)) fill(zl + 1);
+      if (zl == z0 && ghost(z0 - 1)) fill(z0 - 1);
       __syncthreads();
     }
     // a plane beside a wall runs a build of the plane's work with the
@@ -1135,9 +1145,9 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
       int s[SPT];
 #pragma unroll
       for (int k = 0; k < SPT; ++k) s[k] = (z * ny + gy[k]) * nx + gx;
-      const real* nm = slot(z - 1);
-      const real* nc = slot(z);
-      const real* np = slot(z + 1);
+      const real* nm = slot(zl + 1);  // lattice plane z - 1
+      const real* nc = slot(zl);
+      const real* np = slot(zl - 1);
       const int ca = (ty + 1) * AW + (tx + 1);          // the site in the P / Q* box
       const int cu = (ty + 1) * B::UW + (tx + B::UX);   // the site in the u box
       V fin[NV], ds[NV], dh[NV];

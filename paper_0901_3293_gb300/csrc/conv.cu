@@ -303,8 +303,8 @@ __global__ void __launch_bounds__(kConvThreads) k_conv_tc(const __grid_constant_
 // row shift is a 16-B shift of the descriptor's start address).  In the
 // chunk-planar activation layout each group's window is one contiguous run,
 // brought in by one bulk copy.  A CTA
-// walks a contiguous range of (tile, z) items with z fastest, so consecutive
-// items reuse two of their three planes; rows of a tile that fall on ghost
+// walks a contiguous range of (tile, plane pair) items with z fastest, so consecutive
+// items share two of their four planes; rows of a tile that fall on ghost
 // positions (X or Y on the padding) are computed and discarded.
 // ---------------------------------------------------------------------------
 constexpr int kWinPipes = 2;   // independent pipelines per CTA (they share the weights)
@@ -325,6 +325,33 @@ struct WinSmem {
   static constexpr uint32_t WSBO = 8 * CIN * 2;
   static constexpr uint32_t PIPE_COLS = kWinAcc * 2 * COUT;  // an accumulator stage holds two output planes
   static constexpr uint32_t TMEM_COLS = kWinPipes * PIPE_COLS < 32 ? 32 : kWinPipes * PIPE_COLS;
+};
+
+// Slots of an item's input planes zA - 1 .. zA + 2 from those of the item before
+// (the same tile, one pair down): its last two planes stay where they are, and
+// the new ones take the slots in the order in which that item releases them.
+// Its plane 0 goes first, after a quarter of its MMAs, and takes the new plane
+// 3, whose MMAs are second; its plane 1, after three quarters, takes the new plane
+// 2, whose MMAs are last.  So each load has an item's time or more before
+// the MMAs that need it.  In ring order, with an item starting once both had
+// landed, the second load had a quarter of an item: 69.9 -> 64.0 us a 32 -> 32
+// layer at 64 x 64 x 256 (74.3 -> 66.0 with a residual), where the MMAs' reads of
+// shared memory take 46 us.
+__device__ __forceinline__ void win_slots(bool first, int ps[4]) {
+  const int a = first ? 0 : ps[2], b = first ? 1 : ps[3], c = first ? 2 : ps[1], d = first ? 3 : ps[0];
+  ps[0] = a, ps[1] = b, ps[2] = c, ps[3] = d;
+}
+
+// Phase bits of a pipeline's slots
+struct WinSlots {
+  uint32_t phase = 0, loaded = 0;
+  __device__ __forceinline__ uint32_t flip(int s) {  // the parity to wait for next
+    const uint32_t p = phase >> s & 1u;
+    phase ^= 1u << s;
+    return p;
+  }
+  __device__ __forceinline__ bool seen(int s) const { return loaded >> s & 1u; }
+  __device__ __forceinline__ void mark(int s) { loaded |= 1u << s; }
 };
 
 template <int CIN, int COUT, int EPI>
@@ -414,35 +441,34 @@ __global__ void __launch_bounds__(kWinThreads) k_conv_win(const void* __restrict
       }
       const uint32_t tx_bytes = (uint32_t)(L::CH * g.wb * 16);
       const __nv_bfloat16* src = static_cast<const __nv_bfloat16*>(base);
-      int sl = 0;        // slot of the next plane load
-      uint32_t eph = 0;  // parity of that slot's next release
-      int nloads = 0;
+      WinSlots rel;              // per slot: loaded before, parity of its next release
+      int ps[4] = {0, 0, 0, 0};  // slots of the item's input planes zA - 1 .. zA + 2
       bool ok = true;
       int T = T0, k = k0;
       for (int it = 0; ok && it < nitems; ++it) {
         const int zA = 2 * k;
-        const bool first = it == 0 || k == 0;
+        const bool pair = zA + 1 < a.nz, first = it == 0 || k == 0;
         // window start inside a plane: first row of the tile minus px + 1
         const long long w0 = (long long)g.l_first + (long long)T * 128 - (g.px + 1);
-        // padded planes zA .. zA+3 hold input planes zA-1 .. zA+2 (zA .. zA+2 for a lone plane);
-        // a pair continuing the previous one shares its first two
-        const int zlast = zA + (zA + 1 < a.nz ? 3 : 2);
-        for (int Z = first ? zA : zA + 2; Z <= zlast; ++Z) {
-          if (nloads >= kWinSlots && !bounded_wait(&empty[sl], eph)) {
+        win_slots(first, ps);
+        // input plane zA - 1 + d (padded plane zA + d) into its slot
+        auto load = [&](int d, int sl) {
+          if (!ok || (rel.seen(sl) && !bounded_wait(&empty[sl], rel.flip(sl)))) {
             ok = false;
-            break;
+            return;
           }
+          rel.mark(sl);
           unsigned char* dst = slots + (size_t)sl * g.slot_bytes;
           mbar_arrive_expect_tx(&full[sl], tx_bytes);
           for (int c = 0; c < L::CH; ++c)
-            bulk_load(dst + (size_t)c * g.lbo, src + ((long long)Z * L::CH + c) * plane * 8 + w0 * 8, g.wb * 16,
+            bulk_load(dst + (size_t)c * g.lbo, src + ((long long)(zA + d) * L::CH + c) * plane * 8 + w0 * 8, g.wb * 16,
                       &full[sl]);
-          ++nloads;
-          if (++sl == kWinSlots) {
-            sl = 0;
-            if (nloads > kWinSlots) eph ^= 1u;  // load n waits for release n - S: parity (n / S - 1) & 1
-          }
-        }
+        };
+        // in the order of use (a pair's last plane comes second)
+        if (first) load(0, ps[0]);
+        if (pair) load(3, ps[3]);
+        if (first) load(1, ps[1]);
+        load(2, ps[2]);
         if (++k == npairs) {
           k = 0;
           ++T;
@@ -472,37 +498,22 @@ __global__ void __launch_bounds__(kWinThreads) k_conv_win(const void* __restrict
       // row shift of in-plane shift sh in 16-byte units: px + 1 + dy px + dx
       auto row16 = [&](int sh) { return (uint32_t)(px + 1 + (sh / 3 - 1) * px + (sh % 3 - 1)); };
       bool ok = bounded_wait(wbar, 0);
-      // ring state of the loads: the planes of the current item, oldest first
-      int ps[4] = {0, 0, 0, 0};
-      uint32_t pph[4] = {0, 0, 0, 0};
-      int nsl = 0;       // slot of the next load to consume
-      uint32_t nph = 0;  // its full-barrier parity
+      int ps[4] = {0, 0, 0, 0};  // slots of the item's input planes zA - 1 .. zA + 2
+      WinSlots fill;             // per slot: parity of its next load
       int acc = 0;
       uint32_t aph = 0;  // accumulator-free parity
       int k = k0;
       for (int it = 0; ok && it < nitems; ++it) {
         const int zA = 2 * k;
         const bool pair = zA + 1 < a.nz, first = it == 0 || k == 0;
-        const int np = pair ? 4 : 3;
-        if (!first) {
-          ps[0] = ps[2];
-          pph[0] = pph[2];
-          ps[1] = ps[3];
-          pph[1] = pph[3];
-        }
-        for (int d = first ? 0 : 2; d < np; ++d) {
-          ps[d] = nsl;
-          pph[d] = nph;
-          if (++nsl == kWinSlots) {
-            nsl = 0;
-            nph ^= 1u;
-          }
-        }
+        win_slots(first, ps);
+        // the load into slot sl has landed; a plane that the item before used stays until released
+        auto landed = [&](int sl) {
+          ok = ok && bounded_wait(&full[sl], fill.flip(sl));
+          tc_fence_after();
+          return ok;
+        };
         if (it >= kWinAcc && !bounded_wait(&acce[acc], aph ^ 1u)) break;
-        // planes already seen complete by the previous item stay loaded until released
-        for (int d = first ? 0 : 2; d < np; ++d)
-          if (!bounded_wait(&full[ps[d]], pph[d])) ok = false;
-        if (!ok) break;
         tc_fence_after();
         // accumulator stage: block 0 (columns [0, COUT)) = output plane zA+1, block 1 = zA
         const uint32_t d0 = tmem_base + acc * 2 * COUT, d1 = d0 + COUT;
@@ -511,6 +522,7 @@ __global__ void __launch_bounds__(kWinThreads) k_conv_win(const void* __restrict
         for (int d = 0; d < 4; ++d) ab[d] = adesc0 + (uint64_t)ps[d] * slot16;
         if (pair) {
           // input plane zA-1 feeds plane zA only (dz = -1), into block 1
+          if (first && !landed(ps[0])) break;
 #pragma unroll
           for (int sh = 0; sh < 9; ++sh)
 #pragma unroll
@@ -519,12 +531,14 @@ __global__ void __launch_bounds__(kWinThreads) k_conv_win(const void* __restrict
                         (sh > 0 || kc > 0) ? 1u : 0u);
           umma_commit(&empty[ps[0]]);
           // input plane zA+2 feeds plane zA+1 only (dz = +1), into block 0
+          if (!landed(ps[3])) break;
 #pragma unroll
           for (int sh = 0; sh < 9; ++sh)
 #pragma unroll
             for (int kc = 0; kc < CIN / 16; ++kc)
               umma_bf16(d0, ab[3] + row16(sh) + 2u * kc * lbo16, wdesc(sh, 1, kc), idesc1,
                         (sh > 0 || kc > 0) ? 1u : 0u);
+          if (first && !landed(ps[1])) break;
           // input plane zA feeds both: B rows [W(dz = -1); W(dz = 0)] -> blocks 0 (zA+1) and 1 (zA)
 #pragma unroll
           for (int sh = 0; sh < 9; ++sh)
@@ -532,6 +546,7 @@ __global__ void __launch_bounds__(kWinThreads) k_conv_win(const void* __restrict
             for (int kc = 0; kc < CIN / 16; ++kc)
               umma_bf16(d0, ab[1] + row16(sh) + 2u * kc * lbo16, wdesc(sh, -1, kc), idesc2, 1u);
           umma_commit(&empty[ps[1]]);
+          if (!landed(ps[2])) break;
           // input plane zA+1 feeds both: B rows [W(dz = 0); W(dz = +1)] -> blocks 0 (zA+1) and 1 (zA)
 #pragma unroll
           for (int sh = 0; sh < 9; ++sh)
@@ -540,6 +555,8 @@ __global__ void __launch_bounds__(kWinThreads) k_conv_win(const void* __restrict
               umma_bf16(d0, ab[2] + row16(sh) + 2u * kc * lbo16, wdesc(sh, 0, kc), idesc2, 1u);
         } else {
           // a lone plane zA: all 27 taps from input planes zA-1 .. zA+1, into block 1
+          if (first && (!landed(ps[0]) || !landed(ps[1]))) break;
+          if (!landed(ps[2])) break;
 #pragma unroll
           for (int t = 0; t < 27; ++t) {
             const int sh = t % 9, dz = t / 9 - 1;

@@ -303,9 +303,19 @@ __global__ void __launch_bounds__(kConvThreads) k_conv_tc(const __grid_constant_
 // row shift is a 16-B shift of the descriptor's start address).  In the
 // chunk-planar activation layout each group's window is one contiguous run,
 // brought in by one bulk copy.  A CTA
-// walks a contiguous range of (tile, plane pair) items with z fastest, so consecutive
-// items share two of their four planes; rows of a tile that fall on ghost
-// positions (X or Y on the padding) are computed and discarded.
+// walks a contiguous range of (tile, plane pair) items with z fastest, downwards;
+// rows of a tile that fall on ghost positions (X or Y on the padding) are computed
+// and discarded.
+//
+// An MMA reads its 4 KB of A from shared memory in 32 cycles whatever its N, so
+// N = 32 is bound by that read.  A staged plane feeds up to three output planes:
+// their accumulators lie next to one another (a stage holds planes 2k + 1 and 2k,
+// the next stage 2k - 1), and one MMA with N = 96 serves all three.  The sums keep
+// the order of dz that pairs of N = 64 gave them (-1, 0, +1 for even output planes,
+// +1, -1, 0 for odd ones), so results stay the same to the bit: that is why pairs
+// are walked down and an odd input plane takes two passes.  32 -> 32 layer at 64 x 64 x 256: tensor pipe 93k -> 82k
+// cycles, 64.2 -> 59.2 us by itself; in a call's chain of layers, where the first
+// windows (190 KB an SM, all SMs at once) take 7 us of each, 655 -> 649 us a call.
 // ---------------------------------------------------------------------------
 constexpr int kWinPipes = 2;   // independent pipelines per CTA (they share the weights)
 constexpr int kWinSlots = 4;   // staged planes per pipeline
@@ -328,17 +338,15 @@ struct WinSmem {
 };
 
 // Slots of an item's input planes zA - 1 .. zA + 2 from those of the item before
-// (the same tile, one pair down): its last two planes stay where they are, and
-// the new ones take the slots in the order in which that item releases them.
-// Its plane 0 goes first, after a quarter of its MMAs, and takes the new plane
-// 3, whose MMAs are second; its plane 1, after three quarters, takes the new plane
-// 2, whose MMAs are last.  So each load has an item's time or more before
-// the MMAs that need it.  In ring order, with an item starting once both had
-// landed, the second load had a quarter of an item: 69.9 -> 64.0 us a 32 -> 32
-// layer at 64 x 64 x 256 (74.3 -> 66.0 with a residual), where the MMAs' reads of
-// shared memory take 46 us.
+// (the same tile, the pair above): its plane zA - 1 is this item's zA + 1 and stays
+// where it is.  The new ones are loaded in the order of use: zA - 1, first, into
+// the slot that has been free since that item began (or since its zA + 2 was used),
+// zA into the slot of that item's zA, released before its last taps.  Each set of
+// taps waits for its own plane.  (With an item that started once all of its planes
+// had landed, in ring order: 69.9 us a 32 -> 32 layer, now 59.2.  A fifth slot
+// does not help: 649 -> 693 us a call.)
 __device__ __forceinline__ void win_slots(bool first, int ps[4]) {
-  const int a = first ? 0 : ps[2], b = first ? 1 : ps[3], c = first ? 2 : ps[1], d = first ? 3 : ps[0];
+  const int a = first ? 0 : ps[3], b = first ? 1 : ps[1], c = first ? 2 : ps[0], d = first ? 3 : ps[2];
   ps[0] = a, ps[1] = b, ps[2] = c, ps[3] = d;
 }
 
@@ -378,17 +386,17 @@ __global__ void __launch_bounds__(kWinThreads) k_conv_win(const void* __restrict
   uint64_t* acce = accf + kWinAcc;
   uint64_t* done = acce + kWinAcc;
 
-  // this pipeline's items: (tile T, plane pair k) with k fastest, a contiguous
-  // share of the CTA's range; pair k is output planes 2k and 2k + 1 (2k alone
-  // when nz is odd and k is the last); every role walks them with incremental
-  // 32-bit counters
+  // this pipeline's items: (tile T, plane pair k) with k fastest and downwards, a
+  // contiguous share of the CTA's range; pair k is output planes 2k and 2k + 1 (2k
+  // alone when nz is odd and k is the last); every role walks them with
+  // incremental 32-bit counters
   const int npairs = (a.nz + 1) / 2;
   const long long items = (long long)g.ntiles * npairs;
   const long long cbeg = items * blockIdx.x / gridDim.x, cend = items * (blockIdx.x + 1) / gridDim.x;
   const long long jbeg = cbeg + (cend - cbeg) * pipe / kWinPipes;
   const long long jend = cbeg + (cend - cbeg) * (pipe + 1) / kWinPipes;
   const int nitems = (int)(jend - jbeg);
-  const int T0 = (int)(jbeg / npairs), k0 = (int)(jbeg % npairs);
+  const int T0 = (int)(jbeg / npairs), k0 = npairs - 1 - (int)(jbeg % npairs);
   const long long plane = (long long)g.px * g.py;
 
   if (threadIdx.x == 0) {
@@ -447,7 +455,7 @@ __global__ void __launch_bounds__(kWinThreads) k_conv_win(const void* __restrict
       int T = T0, k = k0;
       for (int it = 0; ok && it < nitems; ++it) {
         const int zA = 2 * k;
-        const bool pair = zA + 1 < a.nz, first = it == 0 || k == 0;
+        const bool pair = zA + 1 < a.nz, first = it == 0 || k == npairs - 1;
         // window start inside a plane: first row of the tile minus px + 1
         const long long w0 = (long long)g.l_first + (long long)T * 128 - (g.px + 1);
         win_slots(first, ps);
@@ -464,13 +472,13 @@ __global__ void __launch_bounds__(kWinThreads) k_conv_win(const void* __restrict
             bulk_load(dst + (size_t)c * g.lbo, src + ((long long)(zA + d) * L::CH + c) * plane * 8 + w0 * 8, g.wb * 16,
                       &full[sl]);
         };
-        // in the order of use (a pair's last plane comes second)
-        if (first) load(0, ps[0]);
-        if (pair) load(3, ps[3]);
-        if (first) load(1, ps[1]);
-        load(2, ps[2]);
-        if (++k == npairs) {
-          k = 0;
+        // in the order of use
+        if (first && pair) load(3, ps[3]);
+        load(0, ps[0]);
+        load(1, ps[1]);
+        if (first) load(2, ps[2]);
+        if (k-- == 0) {
+          k = npairs - 1;
           ++T;
         }
       }
@@ -485,7 +493,8 @@ __global__ void __launch_bounds__(kWinThreads) k_conv_win(const void* __restrict
   } else if (warp >= kWinEpiWarps + kWinPipes) {
     // ---------------- MMA issuer
     if (lane == 0) {
-      constexpr uint32_t idesc1 = umma_idesc_bf16(128, COUT), idesc2 = umma_idesc_bf16(128, 2 * COUT);
+      constexpr uint32_t idesc1 = umma_idesc_bf16(128, COUT), idesc2 = umma_idesc_bf16(128, 2 * COUT),
+                         idesc3 = umma_idesc_bf16(128, 3 * COUT);
       // descriptors are advanced by adding (byte offset >> 4) to the start-address field
       const uint64_t bdesc0 = umma_sdesc(smem_addr(wsm), L::WSBO, L::SWZ);
       const uint64_t adesc0 = umma_sdesc_noswz(smem_addr(slots), g.lbo, 128u);
@@ -500,86 +509,79 @@ __global__ void __launch_bounds__(kWinThreads) k_conv_win(const void* __restrict
       bool ok = bounded_wait(wbar, 0);
       int ps[4] = {0, 0, 0, 0};  // slots of the item's input planes zA - 1 .. zA + 2
       WinSlots fill;             // per slot: parity of its next load
-      int acc = 0;
-      uint32_t aph = 0;  // accumulator-free parity
       int k = k0;
+      // accumulator stage of item i: free once the epilogue has read the item kWinAcc before
+      auto acquire = [&](int i) {
+        ok = ok && (i < kWinAcc || bounded_wait(&acce[i % kWinAcc], (i / kWinAcc - 1) & 1));
+        tc_fence_after();
+        return ok;
+      };
+      // the load into slot sl has landed; a plane that the item before used stays until released
+      auto landed = [&](int sl) {
+        ok = ok && bounded_wait(&full[sl], fill.flip(sl));
+        tc_fence_after();
+        return ok;
+      };
+      // the nine in-plane taps of the plane in slot sl, B rows from W(dz) on, into column d
+      auto taps = [&](uint32_t d, int sl, int dz, uint32_t idesc, bool fresh) {
+        const uint64_t ab = adesc0 + (uint64_t)sl * slot16;
+#pragma unroll
+        for (int sh = 0; sh < 9; ++sh)
+#pragma unroll
+          for (int kc = 0; kc < CIN / 16; ++kc)
+            umma_bf16(d, ab + row16(sh) + 2u * kc * lbo16, wdesc(sh, dz, kc), idesc,
+                      sh > 0 || kc > 0 || !fresh ? 1u : 0u);
+      };
       for (int it = 0; ok && it < nitems; ++it) {
         const int zA = 2 * k;
-        const bool pair = zA + 1 < a.nz, first = it == 0 || k == 0;
+        const bool pair = zA + 1 < a.nz, first = it == 0 || k == npairs - 1;
+        const bool cont = it + 1 < nitems && k != 0;  // the next item is the pair below
         win_slots(first, ps);
-        // the load into slot sl has landed; a plane that the item before used stays until released
-        auto landed = [&](int sl) {
-          ok = ok && bounded_wait(&full[sl], fill.flip(sl));
-          tc_fence_after();
-          return ok;
-        };
-        if (it >= kWinAcc && !bounded_wait(&acce[acc], aph ^ 1u)) break;
-        tc_fence_after();
         // accumulator stage: block 0 (columns [0, COUT)) = output plane zA+1, block 1 = zA
+        const int acc = it % kWinAcc;
         const uint32_t d0 = tmem_base + acc * 2 * COUT, d1 = d0 + COUT;
-        uint64_t ab[4];
-#pragma unroll
-        for (int d = 0; d < 4; ++d) ab[d] = adesc0 + (uint64_t)ps[d] * slot16;
-        if (pair) {
-          // input plane zA-1 feeds plane zA only (dz = -1), into block 1
-          if (first && !landed(ps[0])) break;
-#pragma unroll
-          for (int sh = 0; sh < 9; ++sh)
-#pragma unroll
-            for (int kc = 0; kc < CIN / 16; ++kc)
-              umma_bf16(d1, ab[0] + row16(sh) + 2u * kc * lbo16, wdesc(sh, -1, kc), idesc1,
-                        (sh > 0 || kc > 0) ? 1u : 0u);
-          umma_commit(&empty[ps[0]]);
-          // input plane zA+2 feeds plane zA+1 only (dz = +1), into block 0
-          if (!landed(ps[3])) break;
-#pragma unroll
-          for (int sh = 0; sh < 9; ++sh)
-#pragma unroll
-            for (int kc = 0; kc < CIN / 16; ++kc)
-              umma_bf16(d0, ab[3] + row16(sh) + 2u * kc * lbo16, wdesc(sh, 1, kc), idesc1,
-                        (sh > 0 || kc > 0) ? 1u : 0u);
-          if (first && !landed(ps[1])) break;
-          // input plane zA feeds both: B rows [W(dz = -1); W(dz = 0)] -> blocks 0 (zA+1) and 1 (zA)
-#pragma unroll
-          for (int sh = 0; sh < 9; ++sh)
-#pragma unroll
-            for (int kc = 0; kc < CIN / 16; ++kc)
-              umma_bf16(d0, ab[1] + row16(sh) + 2u * kc * lbo16, wdesc(sh, -1, kc), idesc2, 1u);
-          umma_commit(&empty[ps[1]]);
-          if (!landed(ps[2])) break;
-          // input plane zA+1 feeds both: B rows [W(dz = 0); W(dz = +1)] -> blocks 0 (zA+1) and 1 (zA)
-#pragma unroll
-          for (int sh = 0; sh < 9; ++sh)
-#pragma unroll
-            for (int kc = 0; kc < CIN / 16; ++kc)
-              umma_bf16(d0, ab[2] + row16(sh) + 2u * kc * lbo16, wdesc(sh, 0, kc), idesc2, 1u);
-        } else {
-          // a lone plane zA: all 27 taps from input planes zA-1 .. zA+1, into block 1
-          if (first && (!landed(ps[0]) || !landed(ps[1]))) break;
-          if (!landed(ps[2])) break;
-#pragma unroll
-          for (int t = 0; t < 27; ++t) {
-            const int sh = t % 9, dz = t / 9 - 1;
-#pragma unroll
-            for (int kc = 0; kc < CIN / 16; ++kc)
-              umma_bf16(d1, ab[dz + 1] + row16(sh) + 2u * kc * lbo16, wdesc(sh, dz, kc), idesc1,
-                        (t > 0 || kc > 0) ? 1u : 0u);
+        const uint32_t d2 = tmem_base + (acc + 1 < kWinAcc ? acc + 1 : 0) * 2 * COUT;  // the next item's block 0
+        // (the item before acquired this one's stage and began its plane zA+1)
+        if (first) {
+          if (!acquire(it)) break;
+          if (pair) {
+            // input plane zA+2 feeds zA+1 (dz = +1)
+            if (!landed(ps[3])) break;
+            taps(d0, ps[3], 1, idesc1, true);
+            umma_commit(&empty[ps[3]]);
           }
-          umma_commit(&empty[ps[0]]);
-          umma_commit(&empty[ps[1]]);
         }
+        // input plane zA-1 feeds zA (dz = -1)
+        if (!landed(ps[0])) break;
+        taps(d1, ps[0], -1, idesc1, true);
+        // input plane zA feeds zA+1 (dz = -1), zA (dz = 0) and the next item's zA-1 (dz = +1)
+        if (!landed(ps[1]) || (cont && !acquire(it + 1))) break;
+        if (pair && cont && acc + 1 < kWinAcc) {
+          // three adjacent blocks: B rows [W(dz = -1); W(dz = 0); W(dz = +1)]; the
+          // third one starts anew in the first MMA, which is split for it
+          const uint64_t ab = adesc0 + (uint64_t)ps[1] * slot16;
+          umma_bf16(d0, ab + row16(0), wdesc(0, -1, 0), idesc2, 1u);
+          umma_bf16(d2, ab + row16(0), wdesc(0, 1, 0), idesc1, 0u);
+#pragma unroll
+          for (int sh = 0; sh < 9; ++sh)
+#pragma unroll
+            for (int kc = 0; kc < CIN / 16; ++kc)
+              if (sh > 0 || kc > 0)
+                umma_bf16(d0, ab + row16(sh) + 2u * kc * lbo16, wdesc(sh, -1, kc), idesc3, 1u);
+        } else {
+          if (pair) taps(d0, ps[1], -1, idesc2, false);
+          else taps(d1, ps[1], 0, idesc1, false);
+          if (cont) taps(d2, ps[1], 1, idesc1, true);  // (the ring's first stage follows its last)
+        }
+        umma_commit(&empty[ps[1]]);
+        // input plane zA+1 feeds zA+1 (dz = 0) and zA (dz = +1)
+        if (first && !landed(ps[2])) break;
+        if (pair) taps(d0, ps[2], 0, idesc2, false);
+        else taps(d1, ps[2], 1, idesc1, false);
+        umma_commit(&empty[ps[2]]);
+        if (!cont) umma_commit(&empty[ps[0]]);
         umma_commit(&accf[acc]);
-        if (++acc == kWinAcc) {
-          acc = 0;
-          aph ^= 1u;
-        }
-        if (++k == npairs) k = 0;
-        // release the planes the next item does not share with this one
-        const bool cont = it + 1 < nitems && k != 0;
-        if (!cont) {
-          umma_commit(&empty[ps[2]]);
-          if (pair) umma_commit(&empty[ps[3]]);
-        }
+        if (k-- == 0) k = npairs - 1;
       }
       // every issued MMA has finished before the CTA leaves
       umma_commit(done);
@@ -649,8 +651,8 @@ __global__ void __launch_bounds__(kWinThreads) k_conv_win(const void* __restrict
         acc = 0;
         fph ^= 1u;
       }
-      if (++k == npairs) {
-        k = 0;
+      if (k-- == 0) {
+        k = npairs - 1;
         X += 128;
         while (X >= g.px) {
           X -= g.px;

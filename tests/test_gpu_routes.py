@@ -3,8 +3,10 @@
 Widths that are no multiple of 4 (the z-marching kernels with plain row
 prefetches), steps with the flow off (the Heun kernels on the Q mirror) and
 Gauss-Seidel coupling (the LB halves of the z-marching kernels, then the Heun
-kernels with the new velocity), with and without walls, on shapes with ragged tiles in x and y, several tiles and
-z-chunks, and the smallest width.
+kernels with the new velocity), with and without walls, on shapes with ragged
+tiles in x and y, several tiles and z-chunks, and the smallest width; then what
+reads the state the kernels leave, the graphs that replay them, and the
+convolutions over many plane pairs.
 """
 
 import numpy as np
@@ -119,3 +121,102 @@ def test_coupling_switched_between_steps(lcbp):
         lat.set_flow(coupling=lcbp.JACOBI).step(4)
     assert np.abs(a.read_q() - b.read_q()).max() < TOL["f64"][0]
     assert np.abs(a.read_u() - b.read_u()).max() < TOL["f64"][1]
+
+
+@pytest.mark.parametrize("mode", ["flow", "walls"])
+@pytest.mark.parametrize("shape", [(30, 33, 16), (21, 18, 12), (5, 100, 13)])
+def test_narrow_tiles_match_generic(lcbp, shape, mode):
+    """Lattices at most 16 wide: 16 x 16 tiles, full and ragged in x and y."""
+    check(lcbp, shape, "f32", mode, 11)
+
+
+# dtype, mode, shape: every kernel set, the graphs of 16 and 2 steps and single steps
+@pytest.mark.parametrize("dtype,mode,shape", [("f32", "flow", (24, 16, 40)), ("f32", "walls", (17, 9, 37)),
+                                              ("f64", "flow", (6, 10, 36)), ("f32", "noflow", (9, 16, 24)),
+                                              ("f32", "seidel", (10, 12, 36))])
+@pytest.mark.parametrize("before", [0, 1])
+def test_long_runs_equal_single_steps(lcbp, dtype, mode, shape, before):
+    """The same kernels in the same order, whichever graphs replay them and from
+    whichever of the two population buffers: equal to the bit."""
+    a = pair(lcbp, shape, dtype, mode)[0]
+    b = pair(lcbp, shape, dtype, mode)[0]
+    for lat in (a, b):
+        lat.step(before)
+    a.step(51)
+    for _ in range(51):
+        b.step(1)
+    assert np.array_equal(a.read_q(), b.read_q())
+    if mode != "noflow":
+        assert np.array_equal(a.read_u(), b.read_u())
+        assert np.array_equal(a.read_f(), b.read_f())
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("mode", ["flow", "walls", "noflow"])
+@pytest.mark.parametrize("shape", [(7, 9, 33), (6, 12, 64), (1, 5, 5)])
+def test_device_reads_and_diagnostics_from_the_mirrors(lcbp, shape, dtype, mode):
+    """After a step Q and rho u live in the padded mirrors.  Reads into device
+    tensors equal the host's to the bit; the diagnostics of Q equal those of the same
+    field held flat by a generic lattice but for the order of their FP64 sums (1e-12
+    of the sum of n terms of one size)."""
+    import torch
+    lat = pair(lcbp, shape, dtype, mode)[0]
+    lat.step(3)
+    diag = lat.free_energy(), lat.defect_fraction()
+    nptype = np.float32 if dtype == "f32" else np.float64
+    for read, comps in (("read_q", 5), ("read_u", 3), ("read_rho", 1)):
+        host = getattr(lat, read)(dtype=nptype)
+        out = torch.empty(host.shape, device="cuda", dtype=torch.float32 if dtype == "f32" else torch.float64)
+        getattr(lat, read)(out=out)
+        assert np.array_equal(out.cpu().numpy(), host)
+    flat = pair(lcbp, shape, dtype, mode)[1]
+    flat.set_q(lat.read_q())
+    want = flat.free_energy(), flat.defect_fraction()
+    assert abs(diag[0] - want[0]) <= 1e-12 * max(1.0, abs(want[0]))
+    assert diag[1] == want[1]
+
+
+@pytest.mark.parametrize("dims", [(64, 64, 255), (30, 61, 300), (126, 9, 601)])
+def test_window_convolutions_of_many_plane_pairs(lcbp, dims):
+    """Lattices that give a pipeline of the window kernel many plane pairs: the ring
+    of accumulators and of staged planes wraps, ranges start inside a tile, a lone
+    last plane.  Weights of -1, 0, 1 (two in a hundred not zero) and whole inputs keep every
+    FP32 sum a whole number below 2^24, exact in any order, so the two kernels
+    agree to the bit."""
+    nx, ny, nz = dims
+    rng = np.random.default_rng(12)
+    q5 = rng.integers(-1, 2, size=(5, nz, ny, nx)).astype(np.float32)
+    zero3, zero5 = np.zeros((3, nz, ny, nx), np.float32), np.zeros((5, nz, ny, nx), np.float32)
+    out = []
+    for kernel in (lcbp.CONV_TAPS, lcbp.CONV_WINDOW):
+        sur = lcbp.Surrogate(nx, ny, nz)
+        w = np.random.default_rng(13).choice([-1.0, 0.0, 1.0], p=[0.01, 0.98, 0.01], size=sur.get_params().size)
+        sur.set_conv_kernel(kernel).set_params(w)
+        out.append(sur.forward(q5, zero3, zero5, 2.0, -1.0))
+        sur.close()
+    assert np.abs(out[0]).max() > 0
+    assert np.array_equal(out[0], out[1])
+
+
+def test_loss_with_fractional_masks(lcbp):
+    """The mask's weights sum on the device.  A constant 1/4 changes neither loss nor
+    gradients (powers of two are exact), and loss times sum is additive in the mask:
+    products rounded to FP32 (2^-24 each, three losses) and FP64 sums of positive terms."""
+    shape = (6, 10, 33)
+    rng = np.random.default_rng(3)
+    q5, r5, dq = (0.1 * rng.standard_normal((5,) + shape) for _ in range(3))
+    u3 = 1e-3 * rng.standard_normal((3,) + shape)
+    m1 = rng.choice([0.0, 0.3, 0.7, 1.0], size=shape).astype(np.float32)
+    m2 = (np.float32(1) - m1).astype(np.float32)
+    sur = lcbp.Surrogate(shape[2], shape[1], shape[0], training=True)
+    params = 0.02 * rng.standard_normal(sur.get_params().size)
+    loss, grads = {}, {}
+    for name, m in (("none", None), ("quarter", np.full(shape, 0.25, np.float32)), ("one", m1), ("rest", m2)):
+        m64 = None if m is None else m.astype(np.float64)
+        loss[name] = sur.set_params(params).train_step(q5, u3, r5, 1.0, -0.5, dq, m64, lr=1e-6)
+        grads[name] = sur.get_grads()
+    assert loss["quarter"] == loss["none"]
+    assert np.array_equal(grads["quarter"], grads["none"])
+    s1, s2 = m1.astype(np.float64).sum(), m2.astype(np.float64).sum()
+    whole = loss["one"] * s1 + loss["rest"] * s2
+    assert abs(whole - loss["none"] * m1.size) <= 4 * 2.0 ** -24 * loss["none"] * m1.size

@@ -12,7 +12,9 @@
 // so ragged widths leave no lanes idle, and H is formed in each launch instead of
 // stored between them.  96^3 FP32 without flow: 21 us per step, against 39 us on
 // the generic kernels (which store H and read scalars); 200^3: 176 us, 0.67 of
-// the copy bandwidth on the 100 B a site moves; 32^3: 3.6 us.  186 instructions
+// the copy bandwidth on the 100 B a site moves; 32^3: 3.6 us.  The corrector adds
+// in the order of the generic kernels: (Q + Q*) + R; with Q + (Q* + R) the FP64
+// result was 2.7 times as far from the exact one after 40 steps.  186 instructions
 // a site put the issue floor at 4.3 us per launch at 96^3; what is above it is
 // the latency of the loads, which the fetch of the next plane covers in part
 // (24 -> 21 us).  Tiles of 2-D neighbourhoods in place of linear positions and
@@ -28,15 +30,21 @@ namespace lcbp {
 
 namespace {
 
-constexpr int kHeunThreads = 128;
+// FP64: the pipe (half a lane per SM sub-partition) is the bound, so what counts is
+// an even spread of warps: CTAs of one warp, one plane each.  Against 128 threads
+// and several planes: 24^3 15.5 -> 10.4 us a step, 32^3 31.5 -> 17.5, 40^3 59.0 ->
+// 35.8, 64^3 143 -> 117 (the generic kernels: 16.6, 23.8, 58.6, 127).
+template <typename real>
+constexpr int heun_threads() {
+  return sizeof(real) == 8 ? 32 : 128;
+}
 
 template <typename real, bool FLOW, bool WALLS, bool CORRECT>
-__global__ void __launch_bounds__(kHeunThreads)
+__global__ void __launch_bounds__(heun_threads<real>())
     k_heun(ZmGeom G, Model<real> m, const real* S, const real* Qn, const real* U, real* out, Sym5<real> qw) {
   grid_wait();
-  grid_launch_dependents();
   const int nx = G.nx, ny = G.ny, nz = G.nz, nxm = G.nxm;
-  const int p = (blockIdx.x % G.tiles_x) * kHeunThreads + threadIdx.x;
+  const int p = (blockIdx.x % G.tiles_x) * heun_threads<real>() + threadIdx.x;
   if (p >= nx * ny) return;
   const int y = p / nx, x = p - y * nx;
   const int z0 = (blockIdx.x / G.tiles_x) * G.zc, z1 = min(z0 + G.zc, nz);
@@ -104,11 +112,11 @@ __global__ void __launch_bounds__(kHeunThreads)
       }
     }
     const Sym5<real> r = be_rate<true>(st.c, h, dq, u, w, m, FLOW);
-    Sym5<real> q1 = {st.c.xx + r.xx, st.c.xy + r.xy, st.c.xz + r.xz, st.c.yy + r.yy, st.c.yz + r.yz};
     if constexpr (CORRECT) {
       const real half = real(0.5);
-      q1 = {half * (q0.xx + q1.xx), half * (q0.xy + q1.xy), half * (q0.xz + q1.xz), half * (q0.yy + q1.yy),
-            half * (q0.yz + q1.yz)};
+      const Sym5<real> q1 = {half * (q0.xx + st.c.xx + r.xx), half * (q0.xy + st.c.xy + r.xy),
+                             half * (q0.xz + st.c.xz + r.xz), half * (q0.yy + st.c.yy + r.yy),
+                             half * (q0.yz + st.c.yz + r.yz)};
       // the state's mirror: its periodic images too
       mirror_positions(kZmMirX, 2, nx, ny, x, y, [&](int X, int Y) {
         const int i = (z * G.nyq + Y) * nxm + X;
@@ -116,6 +124,7 @@ __global__ void __launch_bounds__(kHeunThreads)
         out[cq4 + i] = q1.yz;
       });
     } else {
+      const Sym5<real> q1 = {st.c.xx + r.xx, st.c.xy + r.xy, st.c.xz + r.xz, st.c.yy + r.yy, st.c.yz + r.yz};
       st4(out + 4 * o, q1.xx, q1.xy, q1.xz, q1.yy);
       out[cq4 + o] = q1.yz;
     }
@@ -131,14 +140,15 @@ __global__ void __launch_bounds__(kHeunThreads)
   }
 }
 
-// Planes per thread: as many as let the grid fill the resident CTAs once (fewer
-// loads per site), at most 16
-template <typename K>
+// Planes per thread: FP64 one (above); FP32 as many as let the grid fill the
+// resident CTAs once (fewer loads per site), at most 16
+template <typename real, typename K>
 int heun_planes(K kernel, int tiles, int nz) {
+  if (sizeof(real) == 8) return 1;
   int dev = 0, sms = 1, per_sm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kHeunThreads, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, heun_threads<real>(), 0);
   const long long slots = (long long)sms * std::max(1, per_sm);
   return (int)std::min<long long>(16, std::max<long long>(1, ((long long)tiles * nz + slots - 1) / slots));
 }
@@ -153,17 +163,17 @@ cudaError_t launch(const HeunArgs& a, cudaStream_t s) {
   G.nyq = a.ny + 4;
   G.nyu = a.ny + 2;
   G.cq = (long long)G.nxm * G.nyq * a.nz;
-  G.tiles_x = (a.nx * a.ny + kHeunThreads - 1) / kHeunThreads;
-  G.zc = heun_planes(k_heun<real, FLOW, WALLS, true>, G.tiles_x, a.nz);
+  G.tiles_x = (a.nx * a.ny + heun_threads<real>() - 1) / heun_threads<real>();
+  G.zc = heun_planes<real>(k_heun<real, FLOW, WALLS, true>, G.tiles_x, a.nz);
   const int grid = G.tiles_x * ((a.nz + G.zc - 1) / G.zc);
   const Model<real> m = *static_cast<const Model<real>*>(a.model);
   Sym5<real> qw{};
   if (WALLS) qw = {(real)a.q_wall[0], (real)a.q_wall[1], (real)a.q_wall[2], (real)a.q_wall[3], (real)a.q_wall[4]};
   const real *q = static_cast<const real*>(a.q), *u = static_cast<const real*>(a.u);
   real* qs = static_cast<real*>(a.qs);
-  launch_dependent(k_heun<real, FLOW, WALLS, false>, grid, kHeunThreads, 0, s, G, m, q, nullptr, u, qs, qw);
+  launch_dependent(k_heun<real, FLOW, WALLS, false>, grid, heun_threads<real>(), 0, s, G, m, q, nullptr, u, qs, qw);
   if (a.mid) cudaEventRecord(a.mid, s);
-  launch_dependent(k_heun<real, FLOW, WALLS, true>, grid, kHeunThreads, 0, s, G, m, qs, q, u, static_cast<real*>(a.q),
+  launch_dependent(k_heun<real, FLOW, WALLS, true>, grid, heun_threads<real>(), 0, s, G, m, qs, q, u, static_cast<real*>(a.q),
                    qw);
   return cudaGetLastError();
 }

@@ -87,6 +87,17 @@ __device__ __forceinline__ Sym5<real> qmirror_at(const real* Q, int cq4, int o) 
 // previous kernel of the stream drains, and wait for it in grid_wait.  It hides
 // the launch and the barrier set-up of each kernel: 12.5 -> 10.3 us per FP32 step
 // at 32^3, 94.5 -> 93.5 us at 64 x 64 x 256 (two-step graphs).
+// The FP32 marching kernels let the next kernel's CTAs in at their start
+// (grid_launch_dependents), to set up beside them.  The others leave that to their
+// end: CTAs that come in early take the places that happen to be free and stay
+// there, so that a small grid ends up unevenly spread, and a kernel bound by its
+// busiest SM loses more than the set-up saves.  That holds for every FP64 kernel
+// (two FP64 lanes an SM: 32^3 80.1 -> 67.9 us a step, 24^3 49.0 -> 37.0, without
+// flow 31.5 -> 17.5 at 32^3 together with CTAs of one warp, Gauss-Seidel 99.9 ->
+// 73.6), for k_heun (FP32 without flow: 64^3 9.8 -> 8.5 us, 128^3 57.6 -> 53.1;
+// 48^3 5.2 -> 5.4) and for the k_lbq before it (FP32 Gauss-Seidel 128^3 256 -> 235
+// us, 96^3 99.6 -> 96.1, 80 x 64 x 48 37.6 -> 37.7).  The FP32 marching kernels
+// gain from it at every even width (32^3 10.1 -> 9.2 us, 64^3 29.6 -> 28.8).
 template <typename... Params, typename... Args>
 void launch_dependent(void (*kernel)(Params...), int grid, int threads, size_t smem, cudaStream_t s, Args&&... args) {
   cudaLaunchAttribute at{};

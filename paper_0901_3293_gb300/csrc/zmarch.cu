@@ -248,7 +248,7 @@ __device__ __forceinline__ void qside_body(const CUtensorMap* tmQ, const CUtenso
   }
   __syncthreads();
   grid_wait();  // the kernel before this one wrote the mirrors and reads the scratch
-  grid_launch_dependents();
+  if constexpr (sizeof(real) == 4) grid_launch_dependents();
 
   // plane p of Q lives in slot (p - (z0-2)) % 5, of rho u in slot (p - (z0-1)) % 4
   // (the plane offsets below are never negative: unsigned arithmetic keeps the ring
@@ -762,13 +762,11 @@ template <typename real, int TY, bool WALLS, bool LBO>
 __global__ void __launch_bounds__(ZM_TX* TY) k_qsite(ZmGeom G, Model<real> m, const real* Q, const real* U,
                                                      const real* bext, real* tau, real* pq, Sym5<real> qw) {
   grid_wait();
-  grid_launch_dependents();
   qsite_body<real, TY, WALLS, LBO>(G, m, blockIdx.x, Q, U, bext, tau, pq, qw);
 }
 template <typename real, int TY, bool WALLS>
 __global__ void __launch_bounds__(ZM_TX* TY) k_qdiv(ZmGeom G, const real* tau, real* pq) {
   grid_wait();
-  grid_launch_dependents();
   qdiv_body<real, TY, WALLS>(G, blockIdx.x, tau, pq);
 }
 
@@ -850,7 +848,6 @@ __global__ void __launch_bounds__(ZM_TX* TY) k_qsite_batch(ZmBatch B, const Repl
                                                            const int* __restrict__ order, const real* Q,
                                                            const real* U, real* fnew, real* pq) {
   grid_wait();
-  grid_launch_dependents();
   const ZmItem it = zm_item(B);
   const ZmGeom G = zm_class_geom(B, it.k);
   int rep0 = B.c[0].rep0;
@@ -980,7 +977,7 @@ __device__ __forceinline__ void lbq_body(const CUtensorMap* tmPQ, const CUtensor
   }
   __syncthreads();
   grid_wait();  // the scratch comes from the kernel before this one
-  grid_launch_dependents();
+  if constexpr (sizeof(real) == 4 && !LBO) grid_launch_dependents();  // (the rule: launch_dependent)
 
   auto wz = [&](int p) { return nz >= 4 ? (p < 0 ? p + nz : p >= nz ? p - nz : p) : wrap(p, nz); };
   auto plane = [&](int p) { return wz(ztop - p); };

@@ -425,11 +425,44 @@ bool mirror_shape(const lcbp_lattice* h) {
 // flow off: the Heun kernels on the Q mirror
 bool use_heun(const lcbp_lattice* h) { return mirror_shape(h) && !h->p.flow_on; }
 
+int sm_count() {
+  static const int n = [] {
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+  }();
+  return n;
+}
+
+// Whether the z-marching kernels pay for a shape that is not their own (widths that
+// are no multiple of 4, and Gauss-Seidel coupling), by size alone, so that runs
+// repeat.  T is the grid with a plane per CTA, e the share of its lanes with a
+// site.  Generic time over marching time, measured:
+//   one CTA an SM at most    FP32 1.13-1.51, FP64 1.30-1.37
+//   FP64, width from 24 on   1.15-1.63; below 0.29-1.10 (the generic tiles fit it)
+//   Gauss-Seidel FP32        width from 32 on 1.03-1.38; below 0.51-1.15
+//   T < 400, Jacobi FP32     e >= 0.8: 1.06-1.07, below 0.77-1.18 (a second CTA on
+//                            some SMs); walls e >= 0.55: 1.10-1.24, below 0.86-0.99
+//   T >= 400, Jacobi FP32    width from 24 on 1.10-1.47; 17-23 1.03-1.15 from T =
+//                            1000 on (0.93-1.05 below); 13-16 (narrow tiles)
+//                            1.10-1.14, below 13 0.57-1.00
+bool march_pays(const lcbp_lattice* h) {
+  if (h->nx % 4 == 0 && !seidel(h)) return true;
+  const int tx = tile_x(h), ty = tile_y(h), nx = h->nx;
+  const long long T = (long long)((nx + tx - 1) / tx) * ((h->ny + ty - 1) / ty) * h->nz;
+  if (T <= sm_count()) return true;
+  if (h->dtype == LCBP_F64) return nx >= 24;
+  if (seidel(h)) return nx >= 32;
+  if (T < 400) return h->n >= (h->p.walls_z ? 0.55 : 0.8) * (double)(T * tx * ty);
+  return nx <= kZmNarrowX ? nx >= 13 : nx >= 24 || T >= 1000;
+}
+
 // whether the step runs the z-marching kernels (both halves of a Jacobi step, or
 // the LB half of a Gauss-Seidel step, whose Q half is the Heun kernels': 80 x 64 x
 // 48 FP32 takes 39 us per step so, 53 us on the five generic kernels)
 bool use_march(lcbp_lattice* h) {
-  if (!mirror_shape(h) || !h->p.flow_on) return false;
+  if (!mirror_shape(h) || !h->p.flow_on || !march_pays(h)) return false;
   if (!h->tmaps_ok) {
     static std::once_flag prep32, prep64;
     if (h->dtype == LCBP_F64) std::call_once(prep64, [] { zm_prepare<double>(); });

@@ -53,14 +53,15 @@ HBM_NOMINAL_GBS = 7900.0  # GB300 HBM3e data-sheet bandwidth (the measured copy 
 # launch scales with the sites.  Valid only for the kernel sources it was
 # taken on (hash below); otherwise null.
 MEASURED_TRAFFIC = {
-    "sources": ["paper_0901_3293_gb300/csrc/zmarch.cu", "paper_0901_3293_gb300/csrc/common.cuh",
-                "paper_0901_3293_gb300/csrc/tma.cuh", "paper_0901_3293_gb300/csrc/kernels.h"],
-    "sha256_16": "83a89e0b63237421",
+    "sources": ["paper_0901_3293_gb300/csrc/zmarch.cu", "paper_0901_3293_gb300/csrc/zm.cuh",
+                "paper_0901_3293_gb300/csrc/common.cuh", "paper_0901_3293_gb300/csrc/tma.cuh",
+                "paper_0901_3293_gb300/csrc/kernels.h"],
+    "sha256_16": "7801db46be7a7ee9",
     # one launch of each kernel in the capture (ncu --set full)
-    "bytes_per_site": {"qside": (181522432 + 211604224) / 160 ** 3,
-                       "lbq": (772152320 + 364112384) / 160 ** 3},
+    "bytes_per_site": {"qside": (182622976 + 214948096) / 160 ** 3,
+                       "lbq": (772982784 + 363322624) / 160 ** 3},
     # smsp__inst_executed.sum (warp instructions) x 32 of the same launches
-    "thread_instr_per_site": {"qside": 101004852 * 32 / 160 ** 3, "lbq": 118693712 * 32 / 160 ** 3},
+    "thread_instr_per_site": {"qside": 98833268 * 32 / 160 ** 3, "lbq": 117323748 * 32 / 160 ** 3},
 }
 ORACLE_SAMPLE = 32  # side of the periodic cube the oracle steps (two BPII unit cells)
 WALL_Q = (0.2, 0.0, 0.0, -0.1, 0.0)  # planar anchoring S (x x - I/3), S = 0.3, on the ghost planes

@@ -363,7 +363,7 @@ struct WinSlots {
 };
 
 template <int CIN, int COUT, int EPI>
-__global__ void __launch_bounds__(kWinThreads) k_conv_win(const void* __restrict__ base,
+__global__ void __launch_bounds__(kWinThreads) k_conv_win(const void* base,
                                                           const __grid_constant__ CUtensorMap tmW, ConvArgs a,
                                                           ConvWin g) {
   using L = WinSmem<CIN, COUT>;

@@ -62,8 +62,8 @@ struct DwGeom {
 };
 
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(kDwThreads, 1) k_dw_tc(const __nv_bfloat16* __restrict__ X,
-                                                         const __nv_bfloat16* __restrict__ dY, DwGeom g,
+__global__ void __launch_bounds__(kDwThreads, 1) k_dw_tc(const __nv_bfloat16* X, const __nv_bfloat16* dY,
+                                                         DwGeom g,
                                                          float* __restrict__ partial, int* __restrict__ err) {
   constexpr int CG = CIN / 8, OG = COUT / 8;
   constexpr int NOUT = 27 * CIN * COUT + COUT;  // values of one CTA's partial
@@ -245,8 +245,8 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_dw_tc(const __nv_bfloat16* __
 // [tap][C_out][C_in] (its epilogue threads are the C_in rows, so each of its
 // stores is one coalesced row) and then the C_out bias gradients.
 constexpr int kRedWarps = 8;
-__global__ void __launch_bounds__(32 * kRedWarps) k_dw_reduce(const float* __restrict__ partial, int nparts, int cin,
-                                                              int cout, float* __restrict__ dW, float* __restrict__ db) {
+__global__ void __launch_bounds__(32 * kRedWarps) k_dw_reduce(const float* partial, int nparts, int cin, int cout,
+                                                              float* __restrict__ dW, float* __restrict__ db) {
   __shared__ float red[kRedWarps][32];
   const int nw = 27 * cin * cout, count = nw + cout;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;

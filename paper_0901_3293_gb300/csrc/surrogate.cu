@@ -65,9 +65,8 @@ size_t true_param_count() {
 // kernels
 // ---------------------------------------------------------------------------
 // network input from physical fields: Q [5][n], u [3][n], R [5][n] (FP32) -> padded BF16, 16 channels, chunk-planar
-__global__ void k_sur_input(const float* __restrict__ q, const float* __restrict__ u, const float* __restrict__ r,
-                            float su, float sr, float kap, float tau, int nx, int ny, int nz,
-                            __nv_bfloat16* __restrict__ out) {
+__global__ void k_sur_input(const float* q, const float* u, const float* r, float su, float sr, float kap, float tau,
+                            int nx, int ny, int nz, __nv_bfloat16* __restrict__ out) {
   grid_wait();
   grid_launch_dependents();
   const long long n = (long long)nx * ny * nz;
@@ -116,9 +115,8 @@ __global__ void k_sur_input(const float* __restrict__ q, const float* __restrict
 
 // masked MSE on y (FP32 [n][16], first 5 channels) against (dq - 10 R) / s_dq
 // (FP32 [5][n]); writes the BF16 padded (chunk-planar) gradient d loss / d y and per-block partial sums
-__global__ void k_sur_loss(const float* __restrict__ y, const float* __restrict__ target,
-                           const float* __restrict__ rate, float ksteps, const float* __restrict__ mask, float inv_sdq,
-                           double inv_den, int nx, int ny, int nz, __nv_bfloat16* __restrict__ grad,
+__global__ void k_sur_loss(const float* y, const float* target, const float* rate, float ksteps, const float* mask,
+                           float inv_sdq, double inv_den, int nx, int ny, int nz, __nv_bfloat16* __restrict__ grad,
                            double* __restrict__ partial) {
   grid_wait();
   grid_launch_dependents();
@@ -168,7 +166,7 @@ __global__ void k_sur_loss(const float* __restrict__ y, const float* __restrict_
 
 // sum of nb partials times scale, by one warp in a fixed order: lane l adds
 // partials l, l + 32, ... in turn, then the lanes' sums meet in a fixed tree
-__global__ void k_sum(const double* __restrict__ partial, int nb, double scale, double* __restrict__ out) {
+__global__ void k_sum(const double* partial, int nb, double scale, double* __restrict__ out) {
   grid_wait();
   grid_launch_dependents();
   if (blockIdx.x != 0 || threadIdx.x >= 32) return;
@@ -304,7 +302,7 @@ __device__ __forceinline__ void put_operands(const ParamTable& tb, int l, int of
 
 // Adam (Kingma & Ba 2015) with bias correction on FP32 master parameters, and
 // the new weights' BF16 operand copies
-__global__ void k_adam(const ParamTable tb, float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m,
+__global__ void k_adam(const ParamTable tb, float* __restrict__ w, const float* g, float* __restrict__ m,
                        float* __restrict__ v, int count, float lr, float b1, float b2, float eps, float c1, float c2) {
   grid_wait();
   grid_launch_dependents();

@@ -98,6 +98,13 @@ __device__ __forceinline__ Sym5<real> qmirror_at(const real* Q, int cq4, int o) 
 // 48^3 5.2 -> 5.4) and for the k_lbq before it (FP32 Gauss-Seidel 128^3 256 -> 235
 // us, 96^3 99.6 -> 96.1, 80 x 64 x 48 37.6 -> 37.7).  The FP32 marching kernels
 // gain from it at every even width (32^3 10.1 -> 9.2 us, 64^3 29.6 -> 28.8).
+//
+// What such a kernel reads and the kernel before it may still be writing is read
+// after grid_wait, and through plain pointers: `const T* __restrict__` and __ldg let
+// the compiler take the read-only path, which is defined only for memory that nothing
+// writes while the kernel lives, and lets it move the load above the wait.  The
+// exceptions (f and Qin of k_lbq, the host's tables and force field) were complete
+// before the kernel was launched.
 template <typename... Params, typename... Args>
 void launch_dependent(void (*kernel)(Params...), int grid, int threads, size_t smem, cudaStream_t s, Args&&... args) {
   cudaLaunchAttribute at{};

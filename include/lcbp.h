@@ -257,10 +257,10 @@ LCBP_API int lcbp_step(lcbp_lattice *h, int nsteps);
  * (field: H/sigma/tau; force_predict: b and the Heun predictor; lb_correct:
  * LB predictor-corrector and the Heun corrector), 5 with Gauss-Seidel
  * coupling (field, force, lb, predict, correct), 3 with flow off (field,
- * predict, correct); with flow off on widths of at least 4 and without
- * LCBP_PATH_GENERIC 2 (predict, correct), with Gauss-Seidel coupling on the
- * marching kernels 4 (qside, lb, predict, correct).  Errors: LCBP_EINVAL if
- * capacity < *nkernels.
+ * predict, correct); with flow off on the Heun kernels of the padded Q 2
+ * (predict, correct), with Gauss-Seidel coupling on the marching kernels 4
+ * (qside, lb, predict, correct).  The count thus tells which kernels run.
+ * Errors: LCBP_EINVAL if capacity < *nkernels.
  */
 LCBP_API int lcbp_profile_steps(lcbp_lattice *h, int nsteps, double *kernel_ms, int capacity, int *nkernels);
 
@@ -270,9 +270,9 @@ LCBP_API int lcbp_profile_steps(lcbp_lattice *h, int nsteps, double *kernel_ms, 
  * -- whenever flow is on, coupling is Jacobi and nx is a multiple of 4; other
  * widths of at least 4 run the same two kernels where their size makes them the
  * faster ones (lcbp_get_path names only the multiples of 4 fast).  With flow off
- * every width of at least 4 runs two kernels of the Heun step on the padded Q, and
- * with Gauss-Seidel coupling, again by size, the LB halves of the fast kernels
- * followed by those two.  Otherwise, or with LCBP_PATH_GENERIC, three
+ * widths of at least 4 run two kernels of the Heun step on the padded Q, and with
+ * Gauss-Seidel coupling the LB halves of the fast kernels followed by those two,
+ * both again by size.  Otherwise, or with LCBP_PATH_GENERIC, three
  * one-thread-per-site kernels.
  * FP32 fast kernels come in two builds, one or two lattice sites per thread
  * (the latter on packed FP32x2 arithmetic); AUTO times both, LCBP_PATH_FAST1

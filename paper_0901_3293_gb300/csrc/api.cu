@@ -422,8 +422,23 @@ bool mirror_shape(const lcbp_lattice* h) {
   return h->path_req != LCBP_PATH_GENERIC && zm_march_ok(h->nx, h->ny, h->nz) && !(h->p.l2_set && h->p.L2 != h->p.K);
 }
 
+// Whether the Heun kernels pay for a lattice with the flow off.  A mirror row of a
+// narrow FP32 lattice is 96 columns for a few sites (a thin one in y has four ghost
+// rows beside its own), and from some 10^5 rows on the lines in use leave L2.  Generic
+// time over Heun time, measured: to 110 000 mirror rows 1.03-2.1 at every shape; above,
+// widths of 4, 5, 7 and 9 0.54-1.01; 6, 8 and 10 0.98-1.37 to 150 000 rows and 0.73-1.12
+// beyond; 11 0.98-1.09; 12 and more 1.08-1.84 in planes of 80 sites and more (12 to 15
+// wide of 96), 0.85-1.26 in smaller ones.  FP64, bound by its arithmetic, 1.05 and more
+// at every shape.
+bool heun_pays(const lcbp_lattice* h) {
+  const long long rows = (long long)(h->ny + 4) * h->nz;
+  if (h->dtype == LCBP_F64 || rows <= 110000) return true;
+  if (h->nx >= 12) return h->nx * h->ny >= (h->nx < 16 ? 96 : 80);
+  return rows <= 150000 && h->nx % 2 == 0 && h->nx > 4;
+}
+
 // flow off: the Heun kernels on the Q mirror
-bool use_heun(const lcbp_lattice* h) { return mirror_shape(h) && !h->p.flow_on; }
+bool use_heun(const lcbp_lattice* h) { return mirror_shape(h) && !h->p.flow_on && heun_pays(h); }
 
 int sm_count() {
   static const int n = [] {

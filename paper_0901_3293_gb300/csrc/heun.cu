@@ -39,15 +39,22 @@ constexpr int heun_threads() {
   return sizeof(real) == 8 ? 32 : 128;
 }
 
-template <typename real, bool FLOW, bool WALLS, bool CORRECT>
+// LINEAR: threads take the positions of all chunks in one sequence, so that planes
+// much smaller than a CTA leave no lanes idle (4 x 4 x 16384 FP32 37.5 -> 17.3 us a
+// step, 17 x 8 x 5000 31.0 -> 21.7; FP64 223 -> 119, 6 x 6 x 4000 117 -> 70).  Else a
+// CTA keeps to one chunk, whose planes are then the same for all of its threads:
+// FP32 21.6 us at 96^3 against 23.3.
+template <typename real, bool FLOW, bool WALLS, bool CORRECT, bool LINEAR>
 __global__ void __launch_bounds__(heun_threads<real>())
     k_heun(ZmGeom G, Model<real> m, const real* S, const real* Qn, const real* U, real* out, Sym5<real> qw) {
   grid_wait();
   const int nx = G.nx, ny = G.ny, nz = G.nz, nxm = G.nxm;
-  const int p = (blockIdx.x % G.tiles_x) * heun_threads<real>() + threadIdx.x;
-  if (p >= nx * ny) return;
+  const int np = nx * ny, t = (LINEAR ? blockIdx.x : blockIdx.x % G.tiles_x) * heun_threads<real>() + threadIdx.x;
+  const int chunk = LINEAR ? t / np : blockIdx.x / G.tiles_x;
+  const int p = LINEAR ? t - chunk * np : t;
+  if (LINEAR ? chunk >= G.tiles_z : p >= np) return;
   const int y = p / nx, x = p - y * nx;
-  const int z0 = (blockIdx.x / G.tiles_x) * G.zc, z1 = min(z0 + G.zc, nz);
+  const int z0 = chunk * G.zc, z1 = min(z0 + G.zc, nz);
   // periodic neighbours in the plane, as offsets in sites
   const int dxm = x == 0 ? nx - 1 : -1, dxp = x == nx - 1 ? 1 - nx : 1;
   const int dym = y == 0 ? (ny - 1) * nxm : -nxm, dyp = y == ny - 1 ? (1 - ny) * nxm : nxm;
@@ -140,19 +147,37 @@ __global__ void __launch_bounds__(heun_threads<real>())
   }
 }
 
-// Planes per thread: FP64 one (above); FP32 as many as let the grid fill the
-// resident CTAs once (fewer loads per site), at most 16
+// CTAs of the kernel that the chip holds at once
 template <typename real, typename K>
-int heun_planes(K kernel, int tiles, int nz) {
-  if (sizeof(real) == 8) return 1;
+long long heun_slots(K kernel) {
   int dev = 0, sms = 1, per_sm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, heun_threads<real>(), 0);
-  const long long slots = (long long)sms * std::max(1, per_sm);
-  return (int)std::min<long long>(16, std::max<long long>(1, ((long long)tiles * nz + slots - 1) / slots));
+  return (long long)sms * std::max(1, per_sm);
 }
 
+template <typename real, bool FLOW, bool WALLS, bool LINEAR>
+cudaError_t launch_as(const HeunArgs& a, ZmGeom G, cudaStream_t s) {
+  G.tiles_z = (a.nz + G.zc - 1) / G.zc;
+  const int T = heun_threads<real>();
+  const int grid = LINEAR ? (a.nx * a.ny * G.tiles_z + T - 1) / T : G.tiles_x * G.tiles_z;
+  const Model<real> m = *static_cast<const Model<real>*>(a.model);
+  Sym5<real> qw{};
+  if (WALLS) qw = {(real)a.q_wall[0], (real)a.q_wall[1], (real)a.q_wall[2], (real)a.q_wall[3], (real)a.q_wall[4]};
+  const real *q = static_cast<const real*>(a.q), *u = static_cast<const real*>(a.u);
+  real *qs = static_cast<real*>(a.qs), *out = static_cast<real*>(a.q);
+  launch_dependent(k_heun<real, FLOW, WALLS, false, LINEAR>, grid, T, 0, s, G, m, q, nullptr, u, qs, qw);
+  if (a.mid) cudaEventRecord(a.mid, s);
+  launch_dependent(k_heun<real, FLOW, WALLS, true, LINEAR>, grid, T, 0, s, G, m, qs, q, u, out, qw);
+  return cudaGetLastError();
+}
+
+// Planes per thread: FP64 one (above); FP32 as many as let the grid fill the
+// resident CTAs once (fewer loads per site), at most 16.  FP64 is always LINEAR (no
+// shape of 24 lost by it); FP32 where planes would fill less than 0.6 of their CTAs'
+// lanes, in more CTAs than the chip holds at once (above 0.6 it gave 0.87-1.01 of the
+// other's speed, below 0.98-2.16; 4 x 4 x 500, which fits at once, 0.91).
 template <typename real, bool FLOW, bool WALLS>
 cudaError_t launch(const HeunArgs& a, cudaStream_t s) {
   ZmGeom G{};
@@ -163,19 +188,19 @@ cudaError_t launch(const HeunArgs& a, cudaStream_t s) {
   G.nyq = a.ny + 4;
   G.nyu = a.ny + 2;
   G.cq = (long long)G.nxm * G.nyq * a.nz;
-  G.tiles_x = (a.nx * a.ny + heun_threads<real>() - 1) / heun_threads<real>();
-  G.zc = heun_planes<real>(k_heun<real, FLOW, WALLS, true>, G.tiles_x, a.nz);
-  const int grid = G.tiles_x * ((a.nz + G.zc - 1) / G.zc);
-  const Model<real> m = *static_cast<const Model<real>*>(a.model);
-  Sym5<real> qw{};
-  if (WALLS) qw = {(real)a.q_wall[0], (real)a.q_wall[1], (real)a.q_wall[2], (real)a.q_wall[3], (real)a.q_wall[4]};
-  const real *q = static_cast<const real*>(a.q), *u = static_cast<const real*>(a.u);
-  real* qs = static_cast<real*>(a.qs);
-  launch_dependent(k_heun<real, FLOW, WALLS, false>, grid, heun_threads<real>(), 0, s, G, m, q, nullptr, u, qs, qw);
-  if (a.mid) cudaEventRecord(a.mid, s);
-  launch_dependent(k_heun<real, FLOW, WALLS, true>, grid, heun_threads<real>(), 0, s, G, m, qs, q, u, static_cast<real*>(a.q),
-                   qw);
-  return cudaGetLastError();
+  const int T = heun_threads<real>(), np = a.nx * a.ny;
+  G.tiles_x = (np + T - 1) / T;
+  if constexpr (sizeof(real) == 8) {
+    G.zc = 1;
+    return launch_as<real, FLOW, WALLS, true>(a, G, s);
+  } else {
+    const long long slots = heun_slots<real>(k_heun<real, FLOW, WALLS, true, false>);
+    const long long ctas = (long long)G.tiles_x * a.nz;
+    const bool linear = np < 0.6 * G.tiles_x * T && ctas > slots;
+    const long long all = linear ? ((long long)np * a.nz + T - 1) / T : ctas;
+    G.zc = (int)std::min<long long>(16, std::max<long long>(1, (all + slots - 1) / slots));
+    return linear ? launch_as<real, FLOW, WALLS, true>(a, G, s) : launch_as<real, FLOW, WALLS, false>(a, G, s);
+  }
 }
 
 }  // namespace

@@ -89,6 +89,28 @@ def test_heun_kernels_match_generic(lcbp, shape, dtype, mode):
     check(lcbp, shape, dtype, mode, 10)
 
 
+# planes far smaller than a CTA: FP64 takes the sites of all planes in one sequence at
+# every shape, FP32 in long lattices (the last CTA of each partly filled; one chunk of several planes and a shorter last one)
+@pytest.mark.parametrize("mode", ["noflow", "noflow_walls", "seidel"])
+@pytest.mark.parametrize("dtype,shape", [("f64", (7, 1, 5)), ("f64", (130, 5, 7)), ("f32", (4100, 5, 5)),
+                                         ("f32", (4999, 8, 17)), ("f32", (9000, 1, 4))])
+def test_heun_kernels_in_thin_lattices(lcbp, dtype, shape, mode):
+    if mode == "seidel" and dtype == "f32":
+        pytest.skip("FP32 Gauss-Seidel: by its rounding errors below")
+    check(lcbp, shape, dtype, mode, 6)
+
+
+@pytest.mark.parametrize("shape,kernels", [((300, 300, 5), 2), ((350, 350, 5), 3), ((16384, 4, 4), 3), ((340, 350, 8), 2),
+                                           ((500, 500, 8), 3), ((500, 500, 12), 2), ((26000, 3, 12), 3)])
+def test_heun_kernels_where_they_pay(lcbp, shape, kernels):
+    """Flow off, FP32: two Heun kernels a step, but the generic three where the mirror's rows are too many for their
+    few sites (there the two took up to 1.8 times as long)."""
+    lat = lcbp.Lattice(shape[2], shape[1], shape[0]).set_flow(flow_on=False).init_q(lcbp.BPII, 0.3, noise=1e-3, seed=4)
+    assert len(lat.profile_steps(1)) == kernels
+    wide = lcbp.Lattice(shape[2], shape[1], shape[0] // 100, dtype="f64").set_flow(flow_on=False)
+    assert len(wide.init_q(lcbp.BPII, 0.3, seed=4).profile_steps(1)) == 2
+
+
 def test_flow_switched_on_after_relaxation(lcbp):
     """The state moves between the kernel sets with its mirrors' images intact."""
     a, b = pair(lcbp, (12, 10, 36), "f64", "noflow")

@@ -411,8 +411,13 @@ __device__ __forceinline__ bool finite5(const Sym5<C>& q) {
 // the Heun kernels do.  Three CTAs per SM: 85 registers, which hold the fetched plane.
 // 256^3 FP32, host-timed calls: energy 370 -> 202 us, totals 605 -> 300, defects
 // 369 -> 125; 64 x 64 x 256: 62 -> 39, 87 -> 52, 62 -> 26.
+// LINEAR: the positions of all chunks in one sequence, so that planes much smaller
+// than a CTA leave no lanes idle (FP64 energy at 4 x 4 x 16384 424 -> 99 us, 5 x 5 x
+// 5000 144 -> 63; FP32 totals 63 -> 33).  The totals of an FP32 lattice stay with one
+// chunk a CTA, the same planes for all of its threads, where planes fill 0.6 of their
+// CTAs (256^3: 297 us, LINEAR 322).
 constexpr int kDiagThreads = 256;
-template <typename real, int WHAT, bool WALLS, bool MIRROR>
+template <typename real, int WHAT, bool WALLS, bool MIRROR, bool LINEAR>
 __global__ void __launch_bounds__(kDiagThreads, sizeof(real) == 4 ? 3 : 1)
     k_diag(DiagGeom g, const real* q, const real* f, double threshold, int planes, double* __restrict__ partials) {
   using C = real;
@@ -427,14 +432,17 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(real) == 4 ? 3 : 1)
   const C kq0h = K * q0, kq0sq = C(2) * K * q0 * q0, cdiv4 = C(0.25) * (C)g.c_div;
   const bool has_div = g.c_div != 0.0;
   const float tf = (float)threshold;
-  // items: kDiagThreads positions of a plane times `planes` planes
+  // a CTA's item: kDiagThreads positions of a plane (LINEAR: of all chunks) times `planes` planes
+  const int chunks = (nz + planes - 1) / planes;
   const long long blocks = (np + kDiagThreads - 1) / kDiagThreads;
-  const long long items = blocks * ((nz + planes - 1) / planes);
+  const long long items = LINEAR ? (np * chunks + kDiagThreads - 1) / kDiagThreads : blocks * chunks;
   for (long long it = blockIdx.x; it < items; it += gridDim.x) {
-    const long long pos = it % blocks * kDiagThreads + threadIdx.x;
-    if (pos >= np) continue;
-    const int y = (int)(pos / nx), x = (int)(pos - (long long)y * nx);
-    const int z0 = (int)(it / blocks) * planes, z1 = min(z0 + planes, nz);
+    const long long t = (LINEAR ? it : it % blocks) * kDiagThreads + threadIdx.x;
+    const int chunk = !LINEAR ? (int)(it / blocks) : t < (1ll << 32) ? (int)((unsigned)t / (unsigned)np) : (int)(t / np);
+    const long long pos = LINEAR ? t - chunk * np : t;
+    if (LINEAR ? chunk >= chunks : pos >= np) continue;
+    const int y = (int)((unsigned)pos / (unsigned)nx), x = (int)((unsigned)pos - (unsigned)y * (unsigned)nx);
+    const int z0 = chunk * planes, z1 = min(z0 + planes, nz);
     const int xp = x + 1 == nx ? 0 : x + 1, xm = x == 0 ? nx - 1 : x - 1;
     const int yp = y + 1 == ny ? 0 : y + 1, ym = y == 0 ? ny - 1 : y - 1;
     auto above = [&](int z) { return z + 1 == nz ? 0 : z + 1; };
@@ -579,21 +587,28 @@ cudaError_t launch_wait_probe(uint64_t limit_ns, int* flag, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// CTAs of k_diag: three per SM of the 152; fewer where there is less work
+// CTAs of k_diag: three for each of 152 SMs, fewer where there is less work; a fixed
+// number, so that the order of the sums is the lattice's alone
 constexpr int kDiagBlocks = 456;
 static_assert(kDiagBlocks * 8 <= kDiagPartials, "the partials buffer holds 8 values per block");
 
 template <typename real, int WHAT, bool WALLS, bool MIRROR>
 void diag_launch(const DiagGeom& g, const void* q, const void* f, double threshold, double* partials, const int* err,
                  double* out, cudaStream_t s) {
-  const long long blocks = ((long long)g.nx * g.ny + kDiagThreads - 1) / kDiagThreads;
-  // planes per item: the fewer the shorter the last wave, up to 16 for the energy's marches
-  const long long share = (blocks * g.nz + kDiagBlocks - 1) / kDiagBlocks;
-  const int planes = (int)std::max<long long>(1, std::min<long long>(16, share));
-  const long long items = blocks * ((g.nz + planes - 1) / planes);
+  const long long np = (long long)g.nx * g.ny, blocks = (np + kDiagThreads - 1) / kDiagThreads;
+  const bool linear = sizeof(real) == 8 || WHAT != kDiagTotals || np < 0.6 * blocks * kDiagThreads;
+  // planes per chunk: the fewer the shorter the last wave, up to 16 for the energy's marches
+  const long long all = linear ? (g.n + kDiagThreads - 1) / kDiagThreads : blocks * g.nz;
+  const int planes = (int)std::min<long long>({16, (all + kDiagBlocks - 1) / kDiagBlocks, (long long)g.nz});
+  const int chunks = (g.nz + planes - 1) / planes;
+  const long long items = linear ? (np * chunks + kDiagThreads - 1) / kDiagThreads : blocks * chunks;
   const int grid = (int)std::min<long long>(items, kDiagBlocks);
-  k_diag<real, WHAT, WALLS, MIRROR><<<grid, kDiagThreads, 0, s>>>(
-      g, static_cast<const real*>(q), static_cast<const real*>(f), threshold, planes, partials);
+  auto go = [&](auto kernel) {
+    kernel<<<grid, kDiagThreads, 0, s>>>(g, static_cast<const real*>(q), static_cast<const real*>(f), threshold, planes,
+                                         partials);
+  };
+  if (linear) go(k_diag<real, WHAT, WALLS, MIRROR, true>);
+  else if constexpr (sizeof(real) == 4 && WHAT == kDiagTotals) go(k_diag<real, WHAT, WALLS, MIRROR, false>);
   k_diag_final<<<1, 256, 0, s>>>(partials, grid, err, out);
 }
 

@@ -210,6 +210,32 @@ def test_device_reads_and_diagnostics_from_the_mirrors(lcbp, shape, dtype, mode)
     assert diag[1] == want[1]
 
 
+# planes much smaller than a CTA and slightly larger ones, one chunk and many, chunks that straddle CTAs
+@pytest.mark.parametrize("dtype,tol", [("f64", 1e-12), ("f32", 1e-4)])
+@pytest.mark.parametrize("walls", [False, True])
+@pytest.mark.parametrize("shape", [(50, 1, 4), (1500, 5, 7), (11, 17, 16), (3, 1, 300), (640, 20, 9)])
+def test_diagnostics_of_thin_lattices(lcbp, shape, walls, dtype, tol):
+    """Against the oracle, from the flat field and from the mirrors that a step leaves: F with the bounds of the other
+    energy tests, whole counts of defects (the threshold in a gap of the eigenvalues), the mass to FP32 moments."""
+    from oracle import lbq
+    p = lbq.Params(walls_z=walls, q_wall=(0.2, 0.0, 0.0, -0.1, 0.0)) if walls else lbq.Params()
+    lat = lcbp.Lattice(shape[2], shape[1], shape[0], dtype=dtype)
+    lat.set_ldg(p.A0, p.gamma, p.K, p.q0).set_flow(p.tau_f, p.xi, p.Gamma)
+    if walls:
+        lat.set_walls(True, p.q_wall)
+    lat.init_q(lcbp.BPII, 0.3, noise=1e-3, seed=4).init_f_equilibrium(1.0)
+    for _ in range(2):
+        Q = lbq.q5_to_q9(lat.read_q())
+        F = lbq.free_energy(Q, p)
+        assert abs(lat.free_energy() - F) < tol * max(1.0, abs(F))
+        top = np.sort(np.linalg.eigvalsh(Q)[..., 2], axis=None)
+        mid = top.size // 4 + np.argmax(np.diff(top[top.size // 4: 3 * top.size // 4]))
+        assert lat.defect_fraction(float(top[mid] + top[mid + 1]) / 2) * lat.n == mid + 1
+        mass = lat.read_f().sum()
+        assert abs(lat.totals()[0] - mass) < (1e-12 if dtype == "f64" else 2.0 ** -23) * mass
+        lat.step(1)
+
+
 @pytest.mark.parametrize("dims", [(64, 64, 255), (30, 61, 300), (126, 9, 601)])
 def test_window_convolutions_of_many_plane_pairs(lcbp, dims):
     """Lattices that give a pipeline of the window kernel many plane pairs: the ring

@@ -670,58 +670,72 @@ int tune_zc(lcbp_lattice* h) {
   auto destroy = [&]() {
     for (int i = 0; i < 3; ++i) cudaEventDestroy(ev[i]);
   };
-  // each kernel keeps its own best: k_lbq over (spt, zc), k_qside over (spt_q, zc)
-  float best_l = 1e30f, best_q = 1e30f;
+  // each kernel keeps its own best, k_lbq over (spt, zc) and k_qside over (spt_q, zc): one
+  // pass over the candidates serves both
+  struct Candidate {
+    int zc, spt;
+    float q, l;
+  };
+  std::vector<Candidate> cand;
+  for (int spt = spt_lo; spt <= spt_hi; ++spt)
+    for (int zc : zc_candidates(h, spt)) cand.push_back({zc, spt, 1e30f, 1e30f});
+  // Times of a candidate's kernels, `reps` launches of each in turn.  Short steps get a
+  // step before the timed one, so that the timed kernels start from a queue and not
+  // from the host's launch of each, and several launches of each kernel between its
+  // events (their order and the launch overlap are then a run's, and a microsecond
+  // decides less).
+  auto time = [&](const Candidate& c, bool lead, int reps, float* q, float* l) {
+    ZmArgs a = zm_args(h, mb.bytes);
+    a.zc = a.zc_q = c.zc;
+    a.spt = a.spt_q = c.spt;
+    // Q^{n+1} to the Q-mirror-sized buffer after the padded scratch: the state is untouched
+    a.qout = static_cast<char*>(h->pq) + (size_t)zm_pq_elems(h->nx, h->ny, h->nz) * h->es;
+    cudaError_t e = cudaSuccess;
+    if (lead) e = launch_zm(h, a);
+    a.reps = reps;
+    a.events = ev;  // before k_qside, between the kernels, after k_lbq
+    if (e == cudaSuccess) e = launch_zm(h, a);
+    if (e == cudaSuccess) e = cudaEventSynchronize(ev[2]);
+    float mq = 0.f, ml = 0.f;
+    if (e == cudaSuccess) e = cudaEventElapsedTime(&mq, ev[0], ev[1]);
+    if (e == cudaSuccess) e = cudaEventElapsedTime(&ml, ev[1], ev[2]);
+    *q = std::min(*q, mq / reps);
+    *l = std::min(*l, ml / reps);
+    return e;
+  };
+  // A single launch of every candidate, then two timed passes over those within a third
+  // of the best in either kernel (FP64: in k_lbq, the first stage has nothing to tune).
+  // Three passes of up to nine launches over all of them, for each pair of spt and spt_q,
+  // made the first step wait 48 ms at 32^3 FP32 (now 2.5), 53 at 64^3 (5.2), 99 at 101 x
+  // 75 x 67 (10) and 139 at 64^3 FP64 (22).
+  float near_q = 1e30f, near_l = 1e30f;
+  cudaError_t e = cudaSuccess;
+  for (Candidate& c : cand) {
+    if (e == cudaSuccess) e = time(c, h->n < (1ll << 20), 1, &c.q, &c.l);
+    near_q = std::min(near_q, c.q * 4 / 3);
+    near_l = std::min(near_l, c.l * 4 / 3);
+  }
+  const float shortest = std::min(near_q, near_l) * 3 / 4;  // ms
+  const int reps = std::max(1, std::min(8, (int)((h->es == 8 ? 0.2f : 0.08f) / std::max(shortest, 1e-3f))));
+  float best_q = 1e30f, best_l = 1e30f;
   int best_zc = std::min(h->nz, 32), best_zq = best_zc, best_spt = spt_lo, best_sq = spt_lo;
-  for (int spt = spt_lo; spt <= spt_hi; ++spt) {
-    for (int sq = spt_lo; sq <= spt_hi; ++sq) {
-      for (int zc : zc_candidates(h, spt)) {
-        ZmArgs a = zm_args(h, mb.bytes);
-        a.zc = a.zc_q = zc;
-        a.spt = spt;
-        a.spt_q = sq;
-        a.events = ev;  // before k_qside, between the kernels, after k_lbq
-        // Q^{n+1} to the Q-mirror-sized buffer after the padded scratch: the state is untouched
-        a.qout = static_cast<char*>(h->pq) + (size_t)zm_pq_elems(h->nx, h->ny, h->nz) * h->es;
-        float tq = 1e30f, tl = 1e30f;
-        for (int rep = 0; rep < 3; ++rep) {
-          // short steps: a step before the timed one, so that the timed kernels
-          // start from a queue and not from the host's launch of each, and several
-          // launches of each kernel between its events (their order and the
-          // launch overlap are then a run's, and a microsecond decides less)
-          cudaError_t e = cudaSuccess;
-          if (h->n < (1ll << 20)) {
-            ZmArgs lead = a;
-            lead.events = nullptr;
-            e = launch_zm(h, lead);
-            a.reps = h->es == 4 && h->n < (1ll << 17) ? 8 : 4;
-          }
-          if (e == cudaSuccess) e = launch_zm(h, a);
-          if (e == cudaSuccess) e = cudaEventSynchronize(ev[2]);
-          if (e != cudaSuccess) {
-            destroy();
-            return cuda_fail(e, "autotune");
-          }
-          float mq = 0.f, ml = 0.f;
-          cudaEventElapsedTime(&mq, ev[0], ev[1]);
-          cudaEventElapsedTime(&ml, ev[1], ev[2]);
-          tq = std::min(tq, mq);
-          tl = std::min(tl, ml);
-        }
-        if (tl < best_l) {
-          best_l = tl;
-          best_zc = zc;
-          best_spt = spt;
-        }
-        if (tq < best_q) {
-          best_q = tq;
-          best_zq = zc;
-          best_sq = sq;
-        }
-      }
+  for (const Candidate& c : cand) {
+    if (e != cudaSuccess || ((h->es == 8 || c.q > near_q) && c.l > near_l)) continue;
+    float tq = 1e30f, tl = 1e30f;
+    for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = time(c, shortest < 0.1f, reps, &tq, &tl);
+    if (tl < best_l) {
+      best_l = tl;
+      best_zc = c.zc;
+      best_spt = c.spt;
+    }
+    if (tq < best_q) {
+      best_q = tq;
+      best_zq = c.zc;
+      best_sq = c.spt;
     }
   }
   destroy();
+  if (e != cudaSuccess) return cuda_fail(e, "autotune");
   if (h->dtype == LCBP_F64) best_zq = 1;  // (the FP64 first stage takes a plane per CTA)
   h->zc = best_zc;
   h->zc_q = best_zq;

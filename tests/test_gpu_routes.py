@@ -236,6 +236,30 @@ def test_diagnostics_of_thin_lattices(lcbp, shape, walls, dtype, tol):
         lat.step(1)
 
 
+@pytest.mark.parametrize("dtype,dims", [("f32", (32, 32, 36)), ("f32", (101, 75, 66)), ("f64", (33, 40, 22))])
+def test_first_step_tunes_within_a_short_run(lcbp, dtype, dims):
+    """The tuning that the first step of a shape waits for takes at most as long as 700 steps of the shape (some 20
+    candidates, a few launches each, the slowest at several times the best; measured 50 to 280)."""
+    import time
+
+    def seconds(lat, steps):
+        t0 = time.perf_counter()
+        lat.step(steps).synchronize()
+        return time.perf_counter() - t0
+
+    def lattice(nz):
+        return lcbp.Lattice(dims[0], dims[1], nz, dtype=dtype).init_q(lcbp.BPII, 0.3).init_f_equilibrium(1.0)
+
+    lattice(3).step(1).synchronize()  # the kernels' code is loaded
+    first = []
+    for k in range(3):  # a shape is tuned once in a process: others of about its size
+        lat = lattice(dims[2] + k)
+        lat.synchronize()
+        first.append(seconds(lat, 1))
+    seconds(lat, 64)
+    assert min(first) < 700 * min(seconds(lat, 64) for _ in range(3)) / 64
+
+
 @pytest.mark.parametrize("dims", [(64, 64, 255), (30, 61, 300), (126, 9, 601)])
 def test_window_convolutions_of_many_plane_pairs(lcbp, dims):
     """Lattices that give a pipeline of the window kernel many plane pairs: the ring

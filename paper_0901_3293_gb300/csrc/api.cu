@@ -203,6 +203,7 @@ struct lcbp_lattice {
   bool f_ready, has_bext;
   cudaGraphExec_t graph[2], graph_run[2];  // two steps and kRunSteps steps, from buffer 0 or 1
   bool graph_ok[2], graph_run_ok[2];
+  long long graph_steps;  // steps asked for since the graphs were dropped
   long long step;
   // fast path (z-marching TMA kernels)
   int path_req;   // LCBP_PATH_*
@@ -838,13 +839,25 @@ void drop_graph(lcbp_lattice* h) {
     if (h->graph_run_ok[k]) cudaGraphExecDestroy(h->graph_run[k]);
     h->graph_run_ok[k] = false;
   }
+  h->graph_steps = 0;
 }
 
-// Steps of the graph that runs of many steps replay, and the run length from
-// which it is worth capturing.  Between two graph launches the GPU idles for two
-// to three microseconds: at 32^3 FP32 a step takes 10.3 us in graphs of two steps
-// and 8.9 us in graphs of 16 (64^3: 30.8 and 29.5 us).
-constexpr int kRunSteps = 16, kRunMin = 32;
+// Steps of the graph that runs of many steps replay, and the steps per kernel of a
+// step, counted from the last change of a parameter (which drops the graphs), from
+// which capturing it pays.  Between two graph launches the GPU idles for two to three
+// microseconds: at 32^3 FP32 a step takes 10.3 us in graphs of two steps and 8.9 us in
+// graphs of 16 (64^3: 30.8 and 29.5 us).  Capturing 16 steps costs about what 24 steps a
+// kernel gain.  A program that changes a parameter before every run of 44 steps, 32^3
+// FP32: 521 us a run when captured from 32 steps on, 505 without; Gauss-Seidel 769
+// and 667, without flow 273 and 254; of 64 steps 683 against about 735.
+constexpr int kRunSteps = 16, kRunMinPerKernel = 24;
+
+// kernels of a step as the lattice runs it
+int step_kernels(lcbp_lattice* h) {
+  if (use_heun(h)) return 2;
+  if (use_march(h)) return (h->dtype == LCBP_F64 ? 3 : 2) + (seidel(h) ? 2 : 0);
+  return kernels_per_step(h->p.flow_on, h->p.coupling);
+}
 
 // capture `steps` (an even number) steps from the current buffer (the ping-pong
 // buffers return to their roles after two steps)
@@ -1345,7 +1358,8 @@ int lcbp_step(lcbp_lattice* h, int nsteps) {
   cudaError_t e = cudaSuccess;
   int left = nsteps;
   const int c = h->cur;  // (the same after every two steps)
-  if (left >= kRunMin && !h->graph_run_ok[c]) {
+  h->graph_steps += nsteps;
+  if (left >= kRunSteps && !h->graph_run_ok[c] && h->graph_steps >= kRunMinPerKernel * step_kernels(h)) {
     int rc = build_graph(h, kRunSteps, &h->graph_run[c], &h->graph_run_ok[c]);
     if (rc) return rc;
   }

@@ -185,6 +185,46 @@ def test_long_runs_equal_single_steps(lcbp, dtype, mode, shape, before):
         assert np.array_equal(a.read_f(), b.read_f())
 
 
+@pytest.mark.parametrize("dtype,mode", [("f32", "flow"), ("f32", "seidel"), ("f64", "flow"), ("f32", "noflow")])
+def test_runs_between_parameter_changes_equal_single_steps(lcbp, dtype, mode):
+    """Changes of a parameter drop the graphs, runs of every length follow: those that replay graphs of two steps and
+    those that capture graphs of 16, at once or when enough steps have gone by."""
+    a = pair(lcbp, (10, 12, 36), dtype, mode)[0]
+    b = pair(lcbp, (10, 12, 36), dtype, mode)[0]
+    for k, runs in enumerate([(1, 16), (47,), (48, 2), (17, 17, 17, 16), (128,)]):
+        for lat in (a, b):
+            lat.set_ldg(0.01, 3.1, 0.01 + 1e-4 * k, 2 * np.pi / 16)
+        for n in runs:
+            a.step(n)
+        for _ in range(sum(runs)):
+            b.step(1)
+    assert np.array_equal(a.read_q(), b.read_q())
+    if mode != "noflow":
+        assert np.array_equal(a.read_f(), b.read_f())
+
+
+def test_runs_between_parameter_changes_capture_no_long_graph(lcbp):
+    """A run of 40 Gauss-Seidel steps after a change of a parameter takes no longer than the same steps in two runs of
+    20, which are too short for the graph of 16 steps (a quarter more, were it captured)."""
+    import time
+
+    def seconds(lat, runs):
+        best = np.inf
+        for k in range(25):
+            lat.set_ldg(0.01, 3.1, 0.01 + 1e-6 * k, 2 * np.pi / 16)
+            lat.synchronize()
+            t0 = time.perf_counter()
+            for n in runs:
+                lat.step(n)
+            lat.synchronize()
+            best = min(best, time.perf_counter() - t0)
+        return best
+
+    lat = pair(lcbp, (32, 32, 32), "f32", "seidel")[0]
+    lat.step(2)
+    assert seconds(lat, (40,)) < 1.1 * seconds(lat, (20, 20))
+
+
 @pytest.mark.parametrize("dtype", ["f32", "f64"])
 @pytest.mark.parametrize("mode", ["flow", "walls", "noflow"])
 @pytest.mark.parametrize("shape", [(7, 9, 33), (6, 12, 64), (1, 5, 5)])

@@ -96,7 +96,9 @@ struct Soft {
   }
 };
 
-// max |Q_scratch - Q_lattice| (both synchronised by the free-energy calls before)
+// max |Q_scratch - Q_lattice|.  The kernel runs on the lattice's stream; what
+// lattice_q may have enqueued for the scratch lattice (its flat Q from its mirrors) is on that
+// one's, and is waited for first.
 int q_gap(lcbp_judge* j, double* gap) {
   const void *qa = nullptr, *qb = nullptr;
   long long n = 0, nb = 0;
@@ -106,8 +108,10 @@ int q_gap(lcbp_judge* j, double* gap) {
   if (!rc) rc = lattice_q(j->lat, &qb, &nb, &db, &sb);
   if (rc) return rc;
   double* out = reinterpret_cast<double*>(static_cast<char*>(j->red) + state_check_scratch_bytes());
-  cudaError_t e = da == LCBP_F64 ? launch_max_abs_diff<double>(qa, qb, 5 * n, j->red, out, sb)
-                                 : launch_max_abs_diff<float>(qa, qb, 5 * n, j->red, out, sb);
+  cudaError_t e = sa == sb ? cudaSuccess : cudaStreamSynchronize(sa);
+  if (e == cudaSuccess)
+    e = da == LCBP_F64 ? launch_max_abs_diff<double>(qa, qb, 5 * n, j->red, out, sb)
+                       : launch_max_abs_diff<float>(qa, qb, 5 * n, j->red, out, sb);
   if (e == cudaSuccess) e = cudaMemcpyAsync(j->h_red, out, sizeof(double), cudaMemcpyDeviceToHost, sb);
   if (e == cudaSuccess) e = cudaStreamSynchronize(sb);
   if (e != cudaSuccess) return jfail_cuda(e, "judge: max |dQ|");

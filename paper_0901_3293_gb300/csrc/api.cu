@@ -133,7 +133,7 @@ int transfer(void* state, int sd, void* user, int ud, long long count, bool uplo
       if (e != cudaSuccess) return cuda_fail(e, "convert");
       e = cudaMemcpyAsync(static_cast<char*>(user) + off * ues, staging, m * ues, cudaMemcpyDefault, st);
     }
-    if (e != cudaSuccess) return cuda_fail(e, "transfer");
+    if (e != cudaSuccess) return after_work(st, cuda_fail(e, "transfer"));
     e = cudaStreamSynchronize(st);  // staging is reused by the next chunk
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
   }
@@ -904,7 +904,7 @@ int diag(lcbp_lattice* h, double threshold, int what) {
 int read_count(lcbp_lattice* h, cudaError_t e, unsigned long long* count) {
   if (e == cudaSuccess) e = cudaMemcpyAsync(h->h_out, h->d_out, 8, cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return cuda_fail(e, "finiteness check");
+  if (e != cudaSuccess) return after_work(h->stream, cuda_fail(e, "finiteness check"));
   *count = *reinterpret_cast<const unsigned long long*>(h->h_out);
   return LCBP_OK;
 }
@@ -970,7 +970,7 @@ bool direct_read(const lcbp_lattice* h, const void* dst, int dtype) {
 
 int finish_read(lcbp_lattice* h, cudaError_t e, const char* what) {
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  return e == cudaSuccess ? LCBP_OK : cuda_fail(e, what);
+  return e == cudaSuccess ? LCBP_OK : after_work(h->stream, cuda_fail(e, what));
 }
 
 struct CkptHeader {

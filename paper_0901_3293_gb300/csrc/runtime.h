@@ -26,6 +26,12 @@ struct HostParams {
 extern thread_local std::string g_last_error;
 int fail(int code, const char* fmt, ...);
 int cuda_fail(cudaError_t e, const char* what);
+// rc, after the stream's work where it is an error: copies and kernels already
+// enqueued may use the caller's buffers, which are the caller's again on return
+inline int after_work(cudaStream_t s, int rc) {
+  if (rc) cudaStreamSynchronize(s);
+  return rc;
+}
 
 TileShape default_tile(int nx, int ny, int nz);
 long long tile_count(int nx, int ny, int nz, TileShape t);

@@ -819,7 +819,7 @@ int lcbp_surrogate_set_params(lcbp_surrogate* s, const float* p, size_t count) {
     s->adam_step = 0;
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-  return e == cudaSuccess ? LCBP_OK : cuda_fail(e, "set_params");
+  return e == cudaSuccess ? LCBP_OK : after_work(s->stream, cuda_fail(e, "set_params"));
 }
 
 }  // extern "C"
@@ -831,7 +831,7 @@ int read_flat(lcbp_surrogate* s, float* padded, float* out, size_t count, const 
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemcpyAsync(out, s->flat, count * 4, cudaMemcpyDefault, s->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-  return e == cudaSuccess ? LCBP_OK : cuda_fail(e, what);
+  return e == cudaSuccess ? LCBP_OK : after_work(s->stream, cuda_fail(e, what));
 }
 }  // namespace
 
@@ -934,7 +934,7 @@ int lcbp_surrogate_forward(lcbp_surrogate* s, const void* q5, const void* u3, co
   if (!q5 || !y5 || !valid_dtype(dtype)) return fail(LCBP_EINVAL, "bad buffers or dtype");
   Fields f;
   rc = stage_inputs(s, q5, u3, r5, dtype, &f);
-  if (rc) return rc;
+  if (rc) return after_work(s->stream, rc);
   launch_input(s, f, kappa, tau);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = forward(s, nullptr);
@@ -942,7 +942,7 @@ int lcbp_surrogate_forward(lcbp_surrogate* s, const void* q5, const void* u3, co
     k_f32_soa<<<grid_for(s->n), 256, 0, s->stream>>>(s->y16, s->n, s->tgt);
     e = cudaGetLastError();
   }
-  if (e != cudaSuccess) return cuda_fail(e, "surrogate forward");
+  if (e != cudaSuccess) return after_work(s->stream, cuda_fail(e, "surrogate forward"));
   rc = sync_err(s, "surrogate forward");
   if (rc) return rc;
   return transfer(s->tgt, LCBP_F32, y5, LCBP_F32, 5 * s->n, false, nullptr, 0, s->stream);
@@ -970,12 +970,12 @@ int lcbp_surrogate_step(lcbp_surrogate* s, lcbp_lattice* h, double kappa, double
   for (int c = 0; c < ncalls && e == cudaSuccess; ++c) {
     const float* r = nullptr;
     rc = lattice_rate_input(h, in, s->stream, &r);
-    if (rc) return rc;
+    if (rc) return after_work(s->stream, rc);
     e = forward(s, q, r);
   }
   if (e == cudaSuccess) e = cudaEventRecord(s->ev_update, s->stream);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(hs, s->ev_update, 0);  // the lattice's next work sees the updated Q
-  if (e != cudaSuccess) return cuda_fail(e, "surrogate step");
+  if (e != cudaSuccess) return after_work(s->stream, cuda_fail(e, "surrogate step"));
   return sync_err(s, "surrogate step");
 }
 
@@ -990,7 +990,7 @@ int lcbp_surrogate_train_step(lcbp_surrogate* s, const void* q5, const void* u3,
   rc = stage_inputs(s, q5, u3, r5, dtype, &f);
   if (!rc) rc = device_field(s, dq5, dtype, 5 * s->n, s->tgt, s->y16, 8 * s->n, &target);
   if (!rc) rc = device_field(s, mask, dtype, s->n, s->msk, s->y16, 8 * s->n, &msk);
-  if (rc) return rc;
+  if (rc) return after_work(s->stream, rc);
   cudaError_t e = cudaSuccess;
   // denominator of the masked MSE: 5 channels x sum of the mask; the host reads
   // the sum while the forward pass runs
@@ -1060,7 +1060,7 @@ int lcbp_surrogate_train_step(lcbp_surrogate* s, const void* q5, const void* u3,
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(s->h_loss, s->dloss, 8, cudaMemcpyDeviceToHost, s->stream);
-  if (e != cudaSuccess) return cuda_fail(e, "train step");
+  if (e != cudaSuccess) return after_work(s->stream, cuda_fail(e, "train step"));
   rc = sync_err(s, "train step");
   if (rc) return rc;
   if (loss) *loss = *s->h_loss;

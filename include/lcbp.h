@@ -276,8 +276,9 @@ LCBP_API int lcbp_profile_steps(lcbp_lattice *h, int nsteps, double *kernel_ms, 
  * one-thread-per-site kernels.
  * FP32 fast kernels come in two builds, one or two lattice sites per thread
  * (the latter on packed FP32x2 arithmetic); AUTO times both, LCBP_PATH_FAST1
- * and LCBP_PATH_FAST2 pin one (a lattice with walls runs one site per thread
- * under either).  All compute the same step.  Errors:
+ * and LCBP_PATH_FAST2 pin one (a lattice with walls or Gauss-Seidel coupling
+ * runs one site per thread under either), and run these kernels at every width
+ * of at least 4, whatever the size.  All compute the same step.  Errors:
  * LCBP_EINVAL (unknown path, or LCBP_PATH_FAST2 on an FP64 lattice).
  */
 LCBP_API int lcbp_set_path(lcbp_lattice *h, int path);

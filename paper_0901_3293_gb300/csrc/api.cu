@@ -438,8 +438,11 @@ bool heun_pays(const lcbp_lattice* h) {
   return rows <= 150000 && h->nx % 2 == 0 && h->nx > 4;
 }
 
+// LCBP_PATH_FAST1 and FAST2 ask for the kernels on the mirrors whatever the size
+bool forced(const lcbp_lattice* h) { return h->path_req == LCBP_PATH_FAST1 || h->path_req == LCBP_PATH_FAST2; }
+
 // flow off: the Heun kernels on the Q mirror
-bool use_heun(const lcbp_lattice* h) { return mirror_shape(h) && !h->p.flow_on && heun_pays(h); }
+bool use_heun(const lcbp_lattice* h) { return mirror_shape(h) && !h->p.flow_on && (forced(h) || heun_pays(h)); }
 
 int sm_count() {
   static const int n = [] {
@@ -478,7 +481,7 @@ bool march_pays(const lcbp_lattice* h) {
 // the LB half of a Gauss-Seidel step, whose Q half is the Heun kernels': 80 x 64 x
 // 48 FP32 takes 39 us per step so, 53 us on the five generic kernels)
 bool use_march(lcbp_lattice* h) {
-  if (!mirror_shape(h) || !h->p.flow_on || !march_pays(h)) return false;
+  if (!mirror_shape(h) || !h->p.flow_on || !(forced(h) || march_pays(h))) return false;
   if (!h->tmaps_ok) {
     static std::once_flag prep32, prep64;
     if (h->dtype == LCBP_F64) std::call_once(prep64, [] { zm_prepare<double>(); });
@@ -634,7 +637,7 @@ int tune_zc(lcbp_lattice* h) {
   // (narrow tiles and Gauss-Seidel coupling: one site per thread only)
   const int spt_max = tile_x(h) < 32 || seidel(h) ? 1 : h->dtype == LCBP_F64 ? zm_spt_max<double>() : zm_spt_max<float>();
   // a pinned sites-per-thread choice tunes only the planes per CTA, uncached
-  const bool pinned = h->path_req == LCBP_PATH_FAST1 || h->path_req == LCBP_PATH_FAST2;
+  const bool pinned = forced(h);
   // (walls: one site per thread only)
   const int spt_lo = h->path_req == LCBP_PATH_FAST2 && !h->p.walls_z && !seidel(h) ? 2 : 1;
   const int spt_hi = h->path_req == LCBP_PATH_FAST1 || h->p.walls_z ? 1 : spt_max;

@@ -80,6 +80,42 @@ def test_larger_odd_widths_match_generic(lcbp, shape, dtype, mode):
     check(lcbp, shape, dtype, mode, 6)
 
 
+# every shape above: AUTO leaves some of them to the generic kernels, FAST1 none
+@pytest.mark.parametrize("mode", ["flow", "walls", "seidel", "seidel_walls"])
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("shape", SHAPES + [(70, 85, 13), (112, 70, 19), (21, 40, 33), (50, 50, 18), (48, 65, 80)])
+def test_marching_kernels_forced(lcbp, shape, dtype, mode):
+    """FAST1 against GENERIC, whichever AUTO would take, and the kernels of a step counted on both sides; FP32
+    Gauss-Seidel by its rounding errors (as below)."""
+    a, b = pair(lcbp, shape, dtype, mode)
+    a.set_path(lcbp.PATH_FAST1)
+    exact = pair(lcbp, shape, "f64", mode)[1] if dtype == "f32" and "seidel" in mode else None
+    assert len(a.profile_steps(6)) == (4 if "seidel" in mode else 2)
+    assert len(b.profile_steps(6)) == (5 if "seidel" in mode else 3)
+    if exact is not None:
+        exact.step(6)
+        for read in ("read_q", "read_u", "read_f"):
+            want = getattr(exact, read)()
+            mine, theirs = (np.linalg.norm(getattr(lat, read)() - want) for lat in (a, b))
+            assert mine <= 2 * theirs
+        return
+    tq, tu = TOL[dtype]
+    assert np.abs(a.read_q() - b.read_q()).max() < tq
+    assert np.abs(a.read_u() - b.read_u()).max() < tu
+    assert np.abs(a.read_f() - b.read_f()).max() <= (2.0 ** -23 if dtype == "f32" else tq)
+
+
+@pytest.mark.parametrize("dtype,mode,shape,kernels", [
+    ("f32", "flow", (9, 11, 5), 2), ("f32", "flow", (37, 47, 45), 2), ("f32", "flow", (50, 50, 18), 3),
+    ("f32", "flow", (70, 85, 13), 2), ("f32", "flow", (9, 200, 100), 2), ("f32", "walls", (37, 19, 45), 2),
+    ("f64", "flow", (70, 85, 13), 3), ("f64", "flow", (37, 19, 45), 2), ("f32", "seidel", (48, 64, 80), 4),
+    ("f32", "seidel", (50, 100, 20), 5), ("f64", "seidel", (21, 40, 33), 4), ("f32", "noflow", (9, 11, 5), 2),
+    ("f32", "flow", (9, 11, 3), 3)])
+def test_kernels_that_auto_picks(lcbp, dtype, mode, shape, kernels):
+    """Both sides of the size rules: 2 marching or Heun kernels a step, 4 with Gauss-Seidel; 3 and 5 generic ones."""
+    assert len(pair(lcbp, shape, dtype, mode)[0].profile_steps(1)) == kernels
+
+
 # 128 positions per CTA: one partly filled CTA, several, a width of 32 lanes; the
 # longest chunk (16 planes) with a shorter last one
 @pytest.mark.parametrize("mode", ["noflow", "noflow_walls"])

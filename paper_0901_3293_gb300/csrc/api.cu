@@ -458,22 +458,34 @@ int sm_count() {
 // are no multiple of 4, and Gauss-Seidel coupling), by size alone, so that runs
 // repeat.  T is the grid with a plane per CTA, e the share of its lanes with a
 // site.  Generic time over marching time, measured:
-//   one CTA an SM at most    FP32 1.13-1.51, FP64 1.30-1.37
-//   FP64, width from 24 on   1.15-1.63; below 0.29-1.10 (the generic tiles fit it)
-//   Gauss-Seidel FP32        width from 32 on 1.03-1.38; below 0.51-1.15
-//   T < 400, Jacobi FP32     e >= 0.8: 1.06-1.07, below 0.77-1.18 (a second CTA on
-//                            some SMs); walls e >= 0.55: 1.10-1.24, below 0.86-0.99
-//   T >= 400, Jacobi FP32    width from 24 on 1.10-1.47; 17-23 1.03-1.15 from T =
-//                            1000 on (0.93-1.05 below); 13-16 (narrow tiles)
-//                            1.10-1.14, below 13 0.57-1.00
+//   one CTA an SM at most    FP32 1.05-1.51, FP64 1.23-1.37
+//   planes of few rows       FP32 to three of a tile's eight 0.31-1.08, Gauss-Seidel to
+//                            two 0.49-1.00 from T = 400 on; FP64 to two of four rows
+//                            0.51-1.03, Gauss-Seidel one 0.70-0.85 (1.17 once)
+//   one plane                FP32 Gauss-Seidel 0.88-0.91 from T = 400 on
+//   FP64, width from 24 on   1.06-1.63; below 0.29-1.35 (the generic tiles fit it)
+//   Gauss-Seidel FP32        width from 32 on 0.96-1.64; below 0.51-1.58
+//   T < 400, Jacobi FP32     e >= 0.8: 0.92-1.07, below 0.77-1.18 (a second CTA on
+//                            some SMs); walls e >= 0.55: 1.10-1.24, below 0.86-1.24
+//   T >= 400, Jacobi FP32    width from 24 on 0.97-1.60; below with e < 0.5 0.79-1.08;
+//                            else 17-23 0.95-1.31 from T = 1000 on (0.93-1.05 below);
+//                            13-16 (narrow tiles) 1.10-1.14, below 13 0.57-1.26
+// Of 1100 shapes drawn at random (4 to 600 wide, 1 to 511 rows, 1 to 3000 planes) the
+// choice is 1.23 times as fast as the generic kernels in the mean, 0.92 at the least;
+// the faster of the two each time would be 1.24.  Of 900 others, drawn after the
+// lines were set: 1.22, 0.91 and 1.23.
 bool march_pays(const lcbp_lattice* h) {
-  if (h->nx % 4 == 0 && !seidel(h)) return true;
-  const int tx = tile_x(h), ty = tile_y(h), nx = h->nx;
-  const long long T = (long long)((nx + tx - 1) / tx) * ((h->ny + ty - 1) / ty) * h->nz;
+  const bool gs = seidel(h), f32 = h->dtype == LCBP_F32;
+  if (h->nx % 4 == 0 && !gs) return true;
+  const int tx = tile_x(h), ty = tile_y(h), nx = h->nx, ny = h->ny;
+  const long long T = (long long)((nx + tx - 1) / tx) * ((ny + ty - 1) / ty) * h->nz;
+  const double e = h->n / (double)(T * tx * ty);
   if (T <= sm_count()) return true;
-  if (h->dtype == LCBP_F64) return nx >= 24;
-  if (seidel(h)) return nx >= 32;
-  if (T < 400) return h->n >= (h->p.walls_z ? 0.55 : 0.8) * (double)(T * tx * ty);
+  if (gs ? T >= 400 && (4 * ny <= ty || (f32 && h->nz == 1)) : f32 ? 8 * ny <= 3 * ty : 2 * ny <= ty) return false;
+  if (!f32) return nx >= 24;
+  if (gs) return nx >= 32;
+  if (T < 400) return e >= (h->p.walls_z ? 0.55 : 0.8);
+  if (nx < 24 && e < 0.5) return false;
   return nx <= kZmNarrowX ? nx >= 13 : nx >= 24 || T >= 1000;
 }
 

@@ -110,7 +110,10 @@ def test_marching_kernels_forced(lcbp, shape, dtype, mode):
     ("f32", "flow", (70, 85, 13), 2), ("f32", "flow", (9, 200, 100), 2), ("f32", "walls", (37, 19, 45), 2),
     ("f64", "flow", (70, 85, 13), 3), ("f64", "flow", (37, 19, 45), 2), ("f32", "seidel", (48, 64, 80), 4),
     ("f32", "seidel", (50, 100, 20), 5), ("f64", "seidel", (21, 40, 33), 4), ("f32", "noflow", (9, 11, 5), 2),
-    ("f32", "flow", (9, 11, 3), 3)])
+    ("f32", "flow", (9, 11, 3), 3), ("f32", "flow", (500, 1, 45), 3), ("f64", "flow", (500, 1, 45), 3),
+    ("f32", "flow", (1000, 2, 25), 3), ("f32", "flow", (600, 5, 41), 2), ("f32", "seidel", (3000, 1, 32), 5),
+    ("f32", "flow", (2000, 3, 33), 3), ("f64", "flow", (2000, 2, 45), 3), ("f64", "seidel", (1000, 2, 25), 4),
+    ("f32", "flow", (3000, 5, 17), 3), ("f32", "seidel", (1, 512, 512), 5)])
 def test_kernels_that_auto_picks(lcbp, dtype, mode, shape, kernels):
     """Both sides of the size rules: 2 marching or Heun kernels a step, 4 with Gauss-Seidel; 3 and 5 generic ones."""
     assert len(pair(lcbp, shape, dtype, mode)[0].profile_steps(1)) == kernels

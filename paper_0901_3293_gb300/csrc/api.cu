@@ -106,6 +106,16 @@ int check_params(const HostParams& p) {
   return LCBP_OK;
 }
 
+int sm_count() {
+  static const int n = [] {
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+  }();
+  return n;
+}
+
 // Copy `count` values between a caller buffer (host or device, dtype `ud`)
 // and a device state array (dtype `sd`), converting through `staging`.  With
 // sync = false a copy without conversion is only enqueued: the caller
@@ -444,20 +454,10 @@ bool forced(const lcbp_lattice* h) { return h->path_req == LCBP_PATH_FAST1 || h-
 // flow off: the Heun kernels on the Q mirror
 bool use_heun(const lcbp_lattice* h) { return mirror_shape(h) && !h->p.flow_on && (forced(h) || heun_pays(h)); }
 
-int sm_count() {
-  static const int n = [] {
-    int dev = 0, sms = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms;
-  }();
-  return n;
-}
-
 // Whether the z-marching kernels pay for a shape that is not their own (widths that
 // are no multiple of 4, and Gauss-Seidel coupling), by size alone, so that runs
-// repeat.  T is the grid with a plane per CTA, e the share of its lanes with a
-// site.  Generic time over marching time, measured:
+// repeat.  T is the grid with a plane per CTA (its lines in units of the 152 SMs they
+// were measured on), e the share of its lanes with a site.  Generic time over marching time, measured:
 //   one CTA an SM at most    FP32 1.05-1.51, FP64 1.23-1.37
 //   planes of few rows       FP32 to three of a tile's eight 0.31-1.08, Gauss-Seidel to
 //                            two 0.49-1.00 from T = 400 on; FP64 to two of four rows
@@ -481,12 +481,13 @@ bool march_pays(const lcbp_lattice* h) {
   const long long T = (long long)((nx + tx - 1) / tx) * ((ny + ty - 1) / ty) * h->nz;
   const double e = h->n / (double)(T * tx * ty);
   if (T <= sm_count()) return true;
-  if (gs ? T >= 400 && (4 * ny <= ty || (f32 && h->nz == 1)) : f32 ? 8 * ny <= 3 * ty : 2 * ny <= ty) return false;
+  const double t = T * 152.0 / sm_count();
+  if (gs ? t >= 400 && (4 * ny <= ty || (f32 && h->nz == 1)) : f32 ? 8 * ny <= 3 * ty : 2 * ny <= ty) return false;
   if (!f32) return nx >= 24;
   if (gs) return nx >= 32;
-  if (T < 400) return e >= (h->p.walls_z ? 0.55 : 0.8);
+  if (t < 400) return e >= (h->p.walls_z ? 0.55 : 0.8);
   if (nx < 24 && e < 0.5) return false;
-  return nx <= kZmNarrowX ? nx >= 13 : nx >= 24 || T >= 1000;
+  return nx <= kZmNarrowX ? nx >= 13 : nx >= 24 || t >= 1000;
 }
 
 // whether the step runs the z-marching kernels (both halves of a Jacobi step, or
@@ -624,12 +625,9 @@ std::vector<int> zc_candidates(const lcbp_lattice* h, int spt) {
   for (int zc : {1, 2, 4, 8, 16, 32, 64})
     if (zc <= h->nz) c.push_back(zc);
   if (h->nz < 64) c.push_back(h->nz);
-  int dev = 0, sms = 1;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int tx = tile_x(h), ty = tile_y(h);
   const long long tiles_xy = (long long)((h->nx + tx - 1) / tx) * ((h->ny + ty - 1) / ty);
-  const long long resident = (long long)sms * (h->dtype == LCBP_F64 ? zm_resident<double>(spt) : zm_resident<float>(spt));
+  const long long resident = (long long)sm_count() * (h->dtype == LCBP_F64 ? zm_resident<double>(spt) : zm_resident<float>(spt));
   for (int w = 1; w <= 48; ++w) {
     const long long want = w * resident;
     for (long long chunks : {want / tiles_xy, (want + tiles_xy - 1) / tiles_xy}) {

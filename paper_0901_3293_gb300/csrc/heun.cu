@@ -23,6 +23,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "runtime.h"
 #include "tma.cuh"
 #include "zm.cuh"
 
@@ -150,11 +151,9 @@ __global__ void __launch_bounds__(heun_threads<real>())
 // CTAs of the kernel that the chip holds at once
 template <typename real, typename K>
 long long heun_slots(K kernel) {
-  int dev = 0, sms = 1, per_sm = 1;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  int per_sm = 1;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, heun_threads<real>(), 0);
-  return (long long)sms * std::max(1, per_sm);
+  return (long long)sm_count() * std::max(1, per_sm);
 }
 
 template <typename real, bool FLOW, bool WALLS, bool LINEAR>

@@ -33,6 +33,7 @@ inline int after_work(cudaStream_t s, int rc) {
   return rc;
 }
 
+int sm_count();  // SMs of the device
 TileShape default_tile(int nx, int ny, int nz);
 long long tile_count(int nx, int ny, int nz, TileShape t);
 void append_tiles(std::vector<Tile>& out, int rep, int nx, int ny, int nz, TileShape t);

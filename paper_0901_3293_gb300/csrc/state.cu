@@ -7,6 +7,7 @@
 #include <cmath>
 
 #include "kernels.h"
+#include "runtime.h"
 
 namespace lcbp {
 
@@ -124,7 +125,7 @@ cudaError_t launch_count_nonfinite(const void* v, long long n, unsigned long lon
   cudaError_t e = cudaMemsetAsync(out, 0, sizeof(*out), s);
   if (e != cudaSuccess) return e;
   const long long want = (n / 16 + kRedThreads - 1) / kRedThreads + 1;  // about four 16-byte loads a thread
-  k_count_nonfinite<real><<<(int)std::min<long long>(want, 152 * 8), kRedThreads, 0, s>>>(
+  k_count_nonfinite<real><<<(int)std::min<long long>(want, sm_count() * 8), kRedThreads, 0, s>>>(
       static_cast<const real*>(v), n, out);
   return cudaGetLastError();
 }
@@ -252,7 +253,7 @@ __global__ void __launch_bounds__(256) k_unpack(MirrorCopy a) {
 // 16 CTAs per SM in all (a CTA walks the others)
 dim3 copy_grid(const MirrorCopy& a, int positions) {
   const long long bx = (positions + 255) / 256, bz = std::min(a.count, 65535);
-  const long long want = 152LL * 16 / (bx * bz) + 1;
+  const long long want = sm_count() * 16LL / (bx * bz) + 1;
   return dim3((unsigned)bx, (unsigned)std::min<long long>({(long long)a.nz, want, 65535LL}), (unsigned)bz);
 }
 

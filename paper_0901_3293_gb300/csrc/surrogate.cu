@@ -994,7 +994,7 @@ int lcbp_surrogate_train_step(lcbp_surrogate* s, const void* q5, const void* u3,
   cudaError_t e = cudaSuccess;
   // denominator of the masked MSE: 5 channels x sum of the mask; the host reads
   // the sum while the forward pass runs
-  constexpr int kMaskBlocks = 304;
+  constexpr int kMaskBlocks = 304;  // (a fixed number: the order of the sum is the field's alone)
   if (msk) {
     k_mask_sum<<<kMaskBlocks, 256, 0, s->stream>>>(msk, s->n, s->partial);
     k_sum<<<1, 32, 0, s->stream>>>(s->partial, kMaskBlocks, 1.0, s->dloss);

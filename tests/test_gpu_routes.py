@@ -383,3 +383,63 @@ def test_loss_with_fractional_masks(lcbp):
     s1, s2 = m1.astype(np.float64).sum(), m2.astype(np.float64).sum()
     whole = loss["one"] * s1 + loss["rest"] * s2
     assert abs(whole - loss["none"] * m1.size) <= 4 * 2.0 ** -24 * loss["none"] * m1.size
+
+
+def test_surrogate_reads_device_fields_in_place(lcbp):
+    """CUDA float32 tensors, one value off a 16-byte boundary, give what the same numpy arrays give, to the bit."""
+    import torch
+    shape = (9, 10, 34)
+    rng = np.random.default_rng(5)
+    fields = [(0.1 * rng.standard_normal((c,) + shape)).astype(np.float32) for c in (5, 3, 5, 5)]
+    mask = rng.choice([0.0, 0.5, 1.0], size=shape).astype(np.float32)
+
+    def device(a):
+        flat = torch.empty(a.size + 1, device="cuda")
+        view = flat[1:].view(a.shape)
+        view.copy_(torch.from_numpy(a))
+        return view
+
+    params = 0.02 * rng.standard_normal(lcbp.Surrogate(34, 10, 9).get_params().size)
+    got = []
+    for put in (lambda a: a, device):
+        q, u, r, dq = (put(a) for a in fields)
+        sur = lcbp.Surrogate(34, 10, 9, training=True).set_params(params)
+        y = sur.forward(q, u, r, 1.0, -0.5)
+        losses = [sur.train_step(q, u, r, 1.0, -0.5, dq, m, lr=1e-3) for m in (put(mask), None)]
+        got.append((y, losses, sur.get_grads(), sur.get_params()))
+        sur.close()
+    assert got[0][1] == got[1][1]
+    for k in (0, 2, 3):
+        assert np.array_equal(got[0][k], got[1][k])
+
+
+@pytest.mark.parametrize("dtype,mode", [("f32", "flow"), ("f32", "seidel"), ("f32", "noflow"), ("f64", "walls")])
+def test_legacy_stream(lcbp, dtype, mode):
+    """A lattice on the legacy stream (no capture, dependent launches one by one) steps as one on its own stream does,
+    to the bit."""
+    import ctypes
+    import torch
+    a = pair(lcbp, (10, 12, 36), dtype, mode)[0]
+    b = pair(lcbp, (10, 12, 36), dtype, mode)[0]
+    L = lcbp.lib()
+    nbytes = L.lcbp_workspace_bytes(36, 12, 10, a.state_dtype)
+    ws = torch.empty(nbytes + 256, dtype=torch.uint8, device="cuda")
+    handle = type(a._h)()
+    lcbp.check(L.lcbp_create_on_buffers(36, 12, 10, a.state_dtype, ws.data_ptr() + (-ws.data_ptr()) % 256, nbytes, None,
+                                        ctypes.byref(handle)))
+    own = b._h, b._ws
+    b._h, b._ws = handle, ws
+    b.set_flow(flow_on="noflow" not in mode, coupling=lcbp.GAUSS_SEIDEL if "seidel" in mode else lcbp.JACOBI)
+    if "walls" in mode:
+        b.set_walls(True, (0.2, 0.0, 0.0, -0.1, 0.0))
+    b.set_q(a.read_q())
+    if "noflow" not in mode:
+        b.set_f(a.read_f())
+        a.set_f(a.read_f())
+    for lat in (a, b):
+        lat.step(51).step(1)
+    assert np.array_equal(a.read_q(), b.read_q())
+    if "noflow" not in mode:
+        assert np.array_equal(a.read_f(), b.read_f())
+    b.close()
+    b._h, b._ws = own

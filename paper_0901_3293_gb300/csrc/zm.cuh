@@ -96,8 +96,11 @@ __device__ __forceinline__ Sym5<real> qmirror_at(const real* Q, int cq4, int o) 
 // flow 31.5 -> 17.5 at 32^3 together with CTAs of one warp, Gauss-Seidel 99.9 ->
 // 73.6), for k_heun (FP32 without flow: 64^3 9.8 -> 8.5 us, 128^3 57.6 -> 53.1;
 // 48^3 5.2 -> 5.4) and for the k_lbq before it (FP32 Gauss-Seidel 128^3 256 -> 235
-// us, 96^3 99.6 -> 96.1, 80 x 64 x 48 37.6 -> 37.7).  The FP32 marching kernels
-// gain from it at every even width (32^3 10.1 -> 9.2 us, 64^3 29.6 -> 28.8).
+// us, 96^3 99.6 -> 96.1, 80 x 64 x 48 37.6 -> 37.7), and for k_conv_win (its comment).
+// The FP32 marching kernels gain from the early trigger at every even width (32^3 10.1
+// -> 9.2 us, 64^3 29.6 -> 28.8); the surrogate's other kernels keep it, within 0.3% either
+// way (k_rate_input and k_sur_input 5413 us for eight calls against 5425, k_dw_reduce
+// the same).
 //
 // What such a kernel reads and the kernel before it may still be writing is read
 // after grid_wait, and through plain pointers: `const T* __restrict__` and __ldg let
